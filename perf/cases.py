@@ -14,6 +14,7 @@ displacement, Maxwell velocities, types by a random permutation; sigma = eps = m
 dt = 0.005, FENE k = 30, R0 = 1.5.  A run starts from the lattice and every further pass continues it,
 so that the passes go through the melting of the lattice and then the reacting liquid.
 """
+import ctypes
 import math
 import time
 
@@ -48,7 +49,7 @@ def listed():
         # the smallest jobs of an ensemble, watched: ten steps and the observables, where latency counts
         dict(name="monitor_2048", call="monitor", scheme="chain", n=2048, share=0.01, f=1, k=1.0, steps=10),
         # the ensemble: 256 replicas of 1,024 to 65,536 beads
-        dict(name="ensemble_256", call="ensemble", replicas=256, lo=1024, hi=65536, steps=50),
+        dict(name="ensemble_256", call="ensemble", replicas=256, lo=1024, hi=65536, steps=200),
         # a burst of twelve jobs through the server: creation, admission, epochs, read-back
         dict(name="serve_12", call="serve", jobs=12, lo=2048, hi=262144, steps_lo=200, steps_hi=1000),
         # forces of a large configuration with bonds, for analysis or as another integrator's force call
@@ -68,7 +69,7 @@ def draw(rng):
     call = rng.choice(["run"] * 6 + ["monitor", "ensemble", "serve", "forces", "histogram", "noalloc"])
     if call == "ensemble":
         return dict(call=call, replicas=_log(rng, 8, 200), lo=_log(rng, 1024, 4096), hi=_log(rng, 8192, 65536),
-                    steps=rng.randrange(10, 51))
+                    steps=rng.randrange(20, 201))
     if call == "serve":
         return dict(call=call, jobs=rng.randrange(3, 13), lo=_log(rng, 2048, 8192), hi=_log(rng, 16384, 262144),
                     steps_lo=rng.randrange(100, 201), steps_hi=rng.randrange(300, 1001))
@@ -197,9 +198,19 @@ def _jobs(case):
             for c in _replicas(case["jobs"], case["lo"], case["hi"])]
 
 
-def _bond_buffer(n, cap):
-    """A bond list with room for every bond that can form, -1 where there is none yet."""
-    return np.full((n * cap // 2, 6), -1, np.int32)
+def _buffers(ns, caps):
+    """What a program that reads systems of these sizes back keeps: pinned arrays over all of them, the bond list with
+    room for every bond that can form (-1 where there is none yet), and each system's parts of them."""
+    rooms = [n * cap // 2 for n, cap in zip(ns, caps)]
+    whole = dict(positions=torch.zeros((sum(ns), 3), dtype=torch.float64).pin_memory().numpy(),
+                 velocities=torch.zeros((sum(ns), 3), dtype=torch.float64).pin_memory().numpy(),
+                 states=torch.zeros(sum(ns), dtype=torch.int8).pin_memory().numpy(),
+                 bonds=torch.full((sum(rooms), 6), -1, dtype=torch.int32).pin_memory().numpy())
+    parts, at, b = [], 0, 0
+    for n, room in zip(ns, rooms):
+        parts.append({key: v[b:b + room] if key == "bonds" else v[at:at + n] for key, v in whole.items()})
+        at, b = at + n, b + room
+    return whole, parts
 
 
 def _force_inputs(case, seed):
@@ -214,13 +225,15 @@ def prepare(case, seed):
     call = case["call"]
     if call in ("run", "monitor"):
         g = _system(case, seed)
-        return dict(case=case, g=g, bonds=_bond_buffer(g.n, g.desc.adj_cap))
+        whole, parts = _buffers([g.n], [g.desc.adj_cap])
+        return dict(case=case, g=[g], whole=whole, parts=parts)
     if call == "ensemble":
         reps = [_system(c, seed + 1 + r) for r, c in enumerate(_replicas(case["replicas"], case["lo"], case["hi"]))]
         batch = P.Batch()
         for g in reps:
             batch.add(g)
-        return dict(case=case, g=reps, batch=batch, bonds=[_bond_buffer(g.n, g.desc.adj_cap) for g in reps])
+        whole, parts = _buffers([g.n for g in reps], [g.desc.adj_cap for g in reps])
+        return dict(case=case, g=reps, batch=batch, whole=whole, parts=parts)
     if call == "serve":
         made = []
         for r, (c, steps) in enumerate(_jobs(case)):
@@ -231,8 +244,8 @@ def prepare(case, seed):
                               reaction=P.make_reaction(**i["reactions"][0]))))
         budget = 16 << 30
         backend = S.PolyrxBackend(P, positions=True, mem_budget=budget)
-        return dict(case=case, jobs=made, server=S.Server(backend, budget),
-                    bonds=[_bond_buffer(n, system["desc"].adj_cap) for _, n, system in made])
+        room = [np.full((n * system["desc"].adj_cap // 2, 6), -1, np.int32) for _, n, system in made]
+        return dict(case=case, jobs=made, server=S.Server(backend, budget), room=room)
     if call == "forces":
         x, box, pairs = _force_inputs(case, seed)
         n = case["n"]
@@ -256,29 +269,38 @@ def prepare(case, seed):
 
 
 # ---- one pass ------------------------------------------------------------------------------------------
-def _into(buffer, bonds):
-    buffer[: len(bonds)] = bonds.view(np.int32).reshape(-1, 6)
-    return buffer
+def _call(name, g, *args):
+    code = getattr(P.lib(), name)(g.h, *args)
+    if code != P.PRX_OK:
+        raise P.PolyrxError(code, name)
 
 
-def _read(g, buffer):
-    return dict(positions=g.positions(), velocities=g.velocities(), states=g.states(), bonds=_into(buffer, g.bonds()))
+def _read(g, part):
+    """Positions, velocities, states and bonds of a system into its part of the kept arrays."""
+    _call("prx_get_positions", g, part["positions"].ctypes.data)
+    _call("prx_get_velocities", g, part["velocities"].ctypes.data)
+    _call("prx_get_states", g, part["states"].ctypes.data)
+    _call("prx_get_bonds", g, part["bonds"].ctypes.data, len(part["bonds"]), ctypes.byref(ctypes.c_uint64()))
 
 
 def run(state):
     case = state["case"]
     call = case["call"]
     if call == "run":
-        state["g"].run(case["steps"])
-        return _read(state["g"], state["bonds"])
+        g = state["g"][0]
+        g.run(case["steps"])
+        _read(g, state["parts"][0])
+        return state["whole"]
     if call == "monitor":
-        state["g"].run(case["steps"])
-        return state["g"].observables()
+        g = state["g"][0]
+        g.run(case["steps"])
+        return g.observables()
     if call == "ensemble":
         state["batch"].run(case["steps"])
         state["batch"].sync()
-        got = [_read(g, b) for g, b in zip(state["g"], state["bonds"])]
-        return {key: np.concatenate([r[key] for r in got]) for key in got[0]}
+        for g, part in zip(state["g"], state["parts"]):
+            _read(g, part)
+        return state["whole"]
     if call == "serve":
         server = state["server"]
         now = time.perf_counter()
@@ -287,8 +309,10 @@ def run(state):
         while not server.idle():
             server.step()
         done, server.done = sorted(server.done, key=lambda j: j.job_id), []
-        return [dict(positions=j.result["positions"], states=j.result["states"],
-                     bonds=_into(b, j.result["bonds"])) for j, b in zip(done, state["bonds"])]
+        for j, room in zip(done, state["room"]):
+            room[: len(j.result["bonds"])] = j.result["bonds"].view(np.int32).reshape(-1, 6)
+        return [dict(positions=j.result["positions"], states=j.result["states"], bonds=room)
+                for j, room in zip(done, state["room"])]
     if call == "forces":
         return state["g"].forces()
     if call == "histogram":
