@@ -147,8 +147,9 @@ typedef struct {
   uint64_t steps;         /* MD steps completed */
   uint64_t reactions;     /* reaction steps completed */
   uint64_t rebins;        /* neighbour-list rebuilds (sort + lists), including the first */
-  uint64_t step_launches; /* step-kernel launches */
-  uint64_t kernel_launches; /* all kernels launched by this system so far */
+  uint64_t step_launches; /* step kernels run */
+  uint64_t kernel_launches; /* all kernels run by this system so far; a phase of a
+                               persistent run counts as the kernel it stands for */
   uint32_t cells[3];      /* cell grid */
   double cell_edge[3];
 } prx_stats;
@@ -211,7 +212,9 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
 /* ---- execution --------------------------------------------------------- */
 
 /* Queues nsteps MD steps (with the reaction every Theta steps) on the
- * system's stream and returns without waiting.  The run is one device-driven
+ * system's stream and returns without waiting.  A run of a small system is
+ * a few launches of a persistent kernel, each of some hundred steps with
+ * their rebuilds and reaction steps; otherwise the run is one device-driven
  * chain: after each step a kernel on the GPU launches the list rebuild when
  * a particle moved more than skin/2, the reaction step when it is due, and
  * the next step (device graph launches); where device graphs are not

@@ -17,10 +17,11 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libpolyrx.so")
-SOURCES = ["md_kernels.cu", "rx_kernels.cu", "runtime.cu", "noalloc.cu", "dg.cu"]
+SOURCES = ["engine.cu", "md_kernels.cu", "rx_kernels.cu", "runtime.cu", "noalloc.cu", "dg.cu"]
 # relocatable device code only where a kernel launches device graphs
 RDC = {"dg.cu"}
-HEADERS = [os.path.join(CSRC, "prx_internal.cuh"), os.path.join(ROOT, "include", "polyrx.h")]
+HEADERS = [os.path.join(CSRC, h) for h in ("prx_internal.cuh", "md_device.cuh", "rx_device.cuh")]
+HEADERS.append(os.path.join(ROOT, "include", "polyrx.h"))
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
                 "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include")]

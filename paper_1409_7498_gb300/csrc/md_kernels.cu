@@ -15,104 +15,12 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "md_device.cuh"
 #include "prx_internal.cuh"
 
 namespace prx {
 
 namespace {
-
-// WCA pair term in FP32; d = x_j - x_i.  Adds -g d to f and V/2 to e.
-// Reciprocals and quotients use the hardware approximation (relative error
-// about 2^-22), well inside the FP32 force tolerance.
-__device__ __forceinline__ void wca32(const Sys& S, float dx, float dy, float dz, float r2,
-                                      float& fx, float& fy, float& fz, float& e) {
-  const float r2i = __fdividef(1.0f, r2);
-  const float sr2 = S.sig2f * r2i;
-  const float sr6 = sr2 * sr2 * sr2;
-  float g = S.eps24f * sr6 * (2.0f * sr6 - 1.0f) * r2i;
-  if (S.fcapf > 0.0f) {
-    const float r = sqrtf(r2);
-    if (g * r > S.fcapf) g = __fdividef(S.fcapf, r);
-  }
-  fx -= g * dx;
-  fy -= g * dy;
-  fz -= g * dz;
-  e += 0.5f * S.eps4f * (sr6 * sr6 - sr6 + 0.25f);
-}
-
-// Bond term in FP32 (FENE or mirror LJ by style); returns false on FENE overstretch.
-__device__ __forceinline__ bool bond32(const Sys& S, uint32_t style, float dx, float dy, float dz,
-                                       float& fx, float& fy, float& fz, float& e) {
-  const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-  float g;
-  if (style == 0u) {
-    if (!(r2 < S.fr02f)) return false;
-    const float q = 1.0f - r2 * S.fr02if;
-    g = -__fdividef(S.fkf, q);
-    e += 0.5f * (-0.5f * S.fkf * S.fr02f * logf(q));
-  } else {
-    const float r = sqrtf(r2);
-    if (!(r > S.rcf && r < 2.0f * S.rcf)) return true;
-    const float sd = 2.0f * S.rcf - r;
-    const float ss2 = __fdividef(S.sig2f, sd * sd);
-    const float ss6 = ss2 * ss2 * ss2;
-    const float dVdr = __fdividef(S.eps24f * (2.0f * ss6 * ss6 - ss6), sd);
-    g = -__fdividef(dVdr, r);
-    e += 0.5f * S.eps4f * (ss6 * ss6 - ss6 + 0.25f);
-  }
-  fx -= g * dx;
-  fy -= g * dy;
-  fz -= g * dz;
-  return true;
-}
-
-// FP64 versions, arithmetic written as in the plain definitions.
-template <bool ENERGY = true>
-__device__ __forceinline__ void wca64(const Sys& S, double dx, double dy, double dz, double r2,
-                                      double& fx, double& fy, double& fz, double& e) {
-  const double sr2 = __ddiv_rn(S.sig2, r2);
-  const double sr6 = __dmul_rn(__dmul_rn(sr2, sr2), sr2);
-  const double sr12 = __dmul_rn(sr6, sr6);
-  double g = __ddiv_rn(__dmul_rn(S.eps24, __dsub_rn(__dmul_rn(2.0, sr12), sr6)), r2);
-  if (S.fcap > 0.0) {
-    const double r = __dsqrt_rn(r2);
-    if (__dmul_rn(g, r) > S.fcap) g = __ddiv_rn(S.fcap, r);
-  }
-  fx = __dsub_rn(fx, __dmul_rn(g, dx));
-  fy = __dsub_rn(fy, __dmul_rn(g, dy));
-  fz = __dsub_rn(fz, __dmul_rn(g, dz));
-  if constexpr (ENERGY)
-    e = __dadd_rn(e, __dmul_rn(0.5, __dmul_rn(S.eps4, __dadd_rn(__dsub_rn(sr12, sr6), 0.25))));
-}
-
-template <bool ENERGY = true>
-__device__ __forceinline__ bool bond64(const Sys& S, uint32_t style, double dx, double dy,
-                                       double dz, double& fx, double& fy, double& fz, double& e) {
-  const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-  double g;
-  if (style == 0u) {
-    if (!(r2 < S.fr02)) return false;
-    const double q = __dsub_rn(1.0, __ddiv_rn(r2, S.fr02));
-    g = __ddiv_rn(-S.fk, q);
-    if constexpr (ENERGY)
-      e = __dadd_rn(e, __dmul_rn(0.5, __dmul_rn(__dmul_rn(__dmul_rn(-0.5, S.fk), S.fr02), log(q))));
-  } else {
-    const double r = __dsqrt_rn(r2);
-    if (!(r > S.rc && r < 2.0 * S.rc)) return true;
-    const double sd = __dsub_rn(2.0 * S.rc, r);
-    const double ss2 = __ddiv_rn(S.sig2, __dmul_rn(sd, sd));
-    const double ss6 = __dmul_rn(__dmul_rn(ss2, ss2), ss2);
-    const double ss12 = __dmul_rn(ss6, ss6);
-    const double dVdr = __ddiv_rn(__dmul_rn(S.eps24, __dsub_rn(__dmul_rn(2.0, ss12), ss6)), sd);
-    g = __ddiv_rn(-dVdr, r);
-    if constexpr (ENERGY)
-      e = __dadd_rn(e, __dmul_rn(0.5, __dmul_rn(S.eps4, __dadd_rn(__dsub_rn(ss12, ss6), 0.25))));
-  }
-  fx = __dsub_rn(fx, __dmul_rn(g, dx));
-  fy = __dsub_rn(fy, __dmul_rn(g, dy));
-  fz = __dsub_rn(fz, __dmul_rn(g, dz));
-  return true;
-}
 
 // Last warp of a grid to finish, without a block barrier: each warp counts
 // itself out of its block in shared memory, and the last warp of a block
@@ -167,193 +75,6 @@ __device__ __forceinline__ void step_epilogue(const Sys& S, int ph, unsigned lon
   }
 }
 
-// k-th Verlet-list entry of slot i: the neighbour's slot (16-bit for systems
-// of at most 65,535 particles).  Entries past a slot's count hold stale
-// slots of some earlier list: still valid slots.
-template <bool NL16>
-__device__ __forceinline__ uint32_t nl_raw(const Sys& S, int k, uint32_t i) {
-  if constexpr (NL16) return __ldg(((const uint16_t*)S.nl) + (size_t)k * S.n + i);
-  else return __ldg(((const uint32_t*)S.nl) + (size_t)k * S.n + i);
-}
-template <bool NL16>
-__device__ __forceinline__ uint32_t nl_get(const Sys& S, int k, uint32_t i) {
-  return nl_raw<NL16>(S, k, i);
-}
-
-// Fetch the line holding *a into L2 (no register result).
-__device__ __forceinline__ void prefetch_l2(const void* a) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-}
-
-// Physical minimum-image displacement x_j - x_i: exact in fixed point,
-// converted with one rounding, scaled by L / 2^32.
-__device__ __forceinline__ void disp(const Sys& S, uint4 pj, uint4 pi, float& dx, float& dy,
-                                     float& dz) {
-  dx = __int2float_rn(pdiff(pj.x, pi.x)) * S.scale[0];
-  dy = __int2float_rn(pdiff(pj.y, pi.y)) * S.scale[1];
-  dz = __int2float_rn(pdiff(pj.z, pi.z)) * S.scale[2];
-}
-
-// Displacement since the last list build exceeds skin/2 (coarse reference in .w).
-__device__ __forceinline__ bool moved_beyond_skin(const Sys& S, uint32_t X, uint32_t Y, uint32_t Z,
-                                                  uint32_t W) {
-  const int ax = (int)(((X >> S.wshift[0]) - W) << 22) >> 22;
-  const int ay = (int)(((Y >> S.wshift[1]) - (W >> 10)) << 22) >> 22;
-  const int az = (int)(((Z >> S.wshift[2]) - (W >> 20)) << 22) >> 22;
-  const float ex = (float)ax * S.wunit[0], ey = (float)ay * S.wunit[1], ez = (float)az * S.wunit[2];
-  return fmaf(ez, ez, fmaf(ey, ey, ex * ex)) > S.disp2_max;
-}
-
-// periodic_fx for the step kernel: the scaling by 2^32 added to the binary64
-// exponent field (exact for normal x; zero and subnormals stay below 1) and
-// the truncation done by the hardware FP64 -> s64 conversion, which costs
-// one FP64-pipe instruction instead of fx32's variable 64-bit shifts.  The
-// same value as periodic_fx for |x| < 2^29.
-__device__ __forceinline__ uint32_t periodic_fx_cvt(double x, long long Lfx, unsigned long long M) {
-  const double y = __longlong_as_double(__double_as_longlong(x) + (32LL << 52));
-  const unsigned long long a = (unsigned long long)(__double2ll_rz(y) + Lfx);
-  return (uint32_t)__umul64hi(a, M);
-}
-
-// End of an FP32-mode step for one slot: Langevin kick (friction applied
-// exactly in FP64), drift, new fixed-point position, rebuild trigger.
-//   v' = a v + b (F_c + R),  x' = x + dt v'
-__device__ __forceinline__ void integrate32(const Sys& S, Ctl* ctl, const SoA& B, uint4* Pn,
-                                            uint32_t i, uint32_t pid, uint32_t W,
-                                            unsigned long long step, float fx, float fy, float fz,
-                                            double xi, double yi, double zi, double vx, double vy,
-                                            double vz) {
-  float Rx = 0.f, Ry = 0.f, Rz = 0.f;
-  if (S.thermo) {
-    const uint4 w = keyed_draw(S.seed, step, pid, 0u, TAG_THERMO);
-    Rx = S.cRf * (u24f(w.x) - 0.5f);
-    Ry = S.cRf * (u24f(w.y) - 0.5f);
-    Rz = S.cRf * (u24f(w.z) - 0.5f);
-  }
-  const float kx = S.b_kickf * (fx + Rx), ky = S.b_kickf * (fy + Ry), kz = S.b_kickf * (fz + Rz);
-  if (!(fabsf(kx) + fabsf(ky) + fabsf(kz) < 1e30f)) set_status(ctl, PRX_ENONFINITE);
-  vx = __fma_rn(vx, S.a_fric, f2d_exact(kx));
-  vy = __fma_rn(vy, S.a_fric, f2d_exact(ky));
-  vz = __fma_rn(vz, S.a_fric, f2d_exact(kz));
-  const double nx = __fma_rn(S.dt, vx, xi);
-  const double ny = __fma_rn(S.dt, vy, yi);
-  const double nz = __fma_rn(S.dt, vz, zi);
-  const uint32_t X = periodic_fx_cvt(nx, S.Lfx[0], S.M64[0]);
-  const uint32_t Y = periodic_fx_cvt(ny, S.Lfx[1], S.M64[1]);
-  const uint32_t Z = periodic_fx_cvt(nz, S.Lfx[2], S.M64[2]);
-  if (moved_beyond_skin(S, X, Y, Z, W)) raise_rebuild(S);
-  B.vx[i] = vx;
-  B.vy[i] = vy;
-  B.vz[i] = vz;
-  B.x[i] = nx;
-  B.y[i] = ny;
-  B.z[i] = nz;
-  Pn[i] = make_uint4(X, Y, Z, W);
-}
-
-// ---------------------------------------------------------------------------
-// FP32 step kernel: one thread per slot, WCA over the Verlet list.
-// ---------------------------------------------------------------------------
-// The step of slot i: forces over its list and bonds, then the integration
-// (or, FORCES_ONLY, the forces written out).
-template <bool NL16, bool FORCES_ONLY, bool CUBIC>
-__device__ __forceinline__ void step_one(const Sys& S, Ctl* ctl, const SoA& B,
-                                         const uint4* __restrict__ P, uint4* __restrict__ Pn,
-                                         uint32_t i, unsigned long long step) {
-  // every load that does not depend on another goes out first
-  const int cnt = __ldg(S.nn + i);
-  uint32_t rn[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) rn[u] = nl_raw<NL16>(S, u, i);
-  const uint4 pi = __ldg(P + i);
-  // the bond count and adjacency row are read after the list loop; a
-  // prefetch into L2 now hides their DRAM latency without holding
-  // registers across the loop
-  prefetch_l2(B.nadj + i);
-  prefetch_l2(B.adj + (size_t)i * S.cap);
-  float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
-  // software pipeline over the list, four entries per stage: the next
-  // stage's list entries (when this list has one) load while this stage's
-  // four gathers complete.
-  // The build pads every list to whole stages with the slot itself (r = 0,
-  // skipped).  In a cubic box displacements stay in position units and the
-  // neighbour force is scaled once at the end.
-  for (int k = 0; k < cnt; k += 4) {
-    uint4 pj[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) pj[u] = __ldg(P + rn[u]);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) rn[u] = k + 4 < cnt ? nl_raw<NL16>(S, k + 4 + u, i) : 0u;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if constexpr (CUBIC) {
-        const float ux = __int2float_rn(pdiff(pj[u].x, pi.x));
-        const float uy = __int2float_rn(pdiff(pj[u].y, pi.y));
-        const float uz = __int2float_rn(pdiff(pj[u].z, pi.z));
-        const float r2u = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
-        if (r2u > 0.f && r2u < S.rc2u) wca32(S, ux, uy, uz, r2u * S.s2f, fx, fy, fz, e);
-      } else {
-        float dx, dy, dz;
-        disp(S, pj[u], pi, dx, dy, dz);
-        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        if (r2 > 0.f && r2 < S.rc2f) wca32(S, dx, dy, dz, r2, fx, fy, fz, e);
-      }
-    }
-  }
-  if constexpr (CUBIC) {
-    fx *= S.scale[0];
-    fy *= S.scale[0];
-    fz *= S.scale[0];
-  }
-  bool ok = true;
-  // bonds two at a time: both entries, then both partners' positions, in
-  // flight together (half the dependent load chains).  The first pair's
-  // entries load beside the bond count, and its gathers do not wait for it:
-  // entries past the count (stale or never written) are clamped to a valid
-  // slot and their terms skipped.
-  const uint32_t* arow0 = B.adj + (size_t)i * S.cap;
-  const uint32_t nb = __ldg(B.nadj + i);
-  {
-    const uint32_t e0 = __ldg(arow0), e1 = S.cap > 1 ? __ldg(arow0 + 1) : i;
-    const uint32_t s0 = min(e0 & SLOT_MASK, S.n - 1u), s1 = min(e1 & SLOT_MASK, S.n - 1u);
-    const uint4 p0 = __ldg(P + s0), p1 = __ldg(P + s1);
-    float dx, dy, dz;
-    if (nb > 0u) {
-      disp(S, p0, pi, dx, dy, dz);
-      ok = bond32(S, e0 >> 31, dx, dy, dz, fx, fy, fz, e) && ok;
-    }
-    if (nb > 1u) {
-      disp(S, p1, pi, dx, dy, dz);
-      ok = bond32(S, e1 >> 31, dx, dy, dz, fx, fy, fz, e) && ok;
-    }
-  }
-  for (int b = 2; b < (int)nb; b += 2) {
-    const uint32_t* arow = B.adj + (size_t)i * S.cap + b;
-    const bool two = b + 1 < (int)nb;
-    const uint32_t e0 = __ldg(arow), e1 = two ? __ldg(arow + 1) : i;
-    const uint4 p0 = __ldg(P + (e0 & SLOT_MASK)), p1 = __ldg(P + (e1 & SLOT_MASK));
-    float dx, dy, dz;
-    disp(S, p0, pi, dx, dy, dz);
-    ok = bond32(S, e0 >> 31, dx, dy, dz, fx, fy, fz, e) && ok;
-    if (two) {
-      disp(S, p1, pi, dx, dy, dz);
-      ok = bond32(S, e1 >> 31, dx, dy, dz, fx, fy, fz, e) && ok;
-    }
-  }
-  if (!ok) set_status(ctl, PRX_EOVERSTRETCH);
-  if constexpr (FORCES_ONLY) {
-    S.fout[3 * (size_t)i + 0] = (double)fx;
-    S.fout[3 * (size_t)i + 1] = (double)fy;
-    S.fout[3 * (size_t)i + 2] = (double)fz;
-    S.eout[i] = (double)e;
-  } else {
-    const double xi = B.x[i], yi = B.y[i], zi = B.z[i];
-    const double vx = B.vx[i], vy = B.vy[i], vz = B.vz[i];
-    const uint32_t pid = __ldg(B.id + i);
-    integrate32(S, ctl, B, Pn, i, pid, pi.w, step, fx, fy, fz, xi, yi, zi, vx, vy, vz);
-  }
-}
-
 template <bool NL16, bool FORCES_ONLY, bool CUBIC>
 __device__ __forceinline__ void step_nl_body(const Sys& S, const Blk blk,
                                              cudaGraphConditionalHandle cond, int use_cond) {
@@ -368,7 +89,7 @@ __device__ __forceinline__ void step_nl_body(const Sys& S, const Blk blk,
   const uint4* __restrict__ P = ph ? S.P1 : S.P0;
   uint4* __restrict__ Pn = ph ? S.P0 : S.P1;
   const uint32_t i = blk.b * blockDim.x + threadIdx.x;
-  if (i < S.n) step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step);
+  if (i < S.n && step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
   if constexpr (!FORCES_ONLY) step_epilogue(S, ph, step, cond, use_cond, &warps_left, blk.nb);
 }
 
@@ -396,7 +117,7 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
   auto run = [&](const SoA& B) {
     for (uint32_t c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c * 32u < S.n; c += W) {
       const uint32_t i = c * 32u + (threadIdx.x & 31u);
-      if (i < S.n) step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step);
+      if (i < S.n && step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
     }
   };
   if (ctl->set) run(S.s1);
@@ -442,20 +163,7 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
 #pragma unroll
           for (int u = 0; u < 4; ++u) pj[u] = __ldg(P + rn[u]);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if constexpr (CUBIC) {
-              const float ux = __int2float_rn(pdiff(pj[u].x, pi.x));
-              const float uy = __int2float_rn(pdiff(pj[u].y, pi.y));
-              const float uz = __int2float_rn(pdiff(pj[u].z, pi.z));
-              const float r2u = fmaf(uz, uz, fmaf(uy, uy, ux * ux));
-              if (r2u > 0.f && r2u < S.rc2u) wca32(S, ux, uy, uz, r2u * S.s2f, fx, fy, fz, e);
-            } else {
-              float dx, dy, dz;
-              disp(S, pj[u], pi, dx, dy, dz);
-              const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-              if (r2 > 0.f && r2 < S.rc2f) wca32(S, dx, dy, dz, r2, fx, fy, fz, e);
-            }
-          }
+          for (int u = 0; u < 4; ++u) pair32<CUBIC>(S, pj[u], pi, fx, fy, fz, e);
         }
         if constexpr (CUBIC) {
           fx *= S.scale[0];
@@ -497,7 +205,7 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
           const double xi = B.x[ii], yi = B.y[ii], zi = B.z[ii];
           const double vx = B.vx[ii], vy = B.vy[ii], vz = B.vz[ii];
           const uint32_t pid = __ldg(B.id + ii);
-          integrate32(S, ctl, B, Pn, ii, pid, gw, step, gx, gy, gz, xi, yi, zi, vx, vy, vz);
+          if (integrate32(S, ctl, B, Pn, ii, pid, gw, step, gx, gy, gz, xi, yi, zi, vx, vy, vz)) raise_rebuild(S);
         }
       }
     }
@@ -629,17 +337,6 @@ __global__ void __launch_bounds__(STEP_THREADS)
 // per-particle array into the other SoA set with fresh fixed-point positions,
 // adjacency remap, then the Verlet lists.
 // ---------------------------------------------------------------------------
-// v >= L: v - L; then v < 0: v + L.  The tests compare binary64 bit
-// patterns on the integer pipe (for non-negative doubles the bit order is the
-// numeric order; -0.0 counts as 0), so the FP64 pipe only sees the rare
-// particle that left the box.
-__device__ __forceinline__ double wrap_into_box(double v, double L) {
-  if (__double_as_longlong(v) >= __double_as_longlong(L)) v = __dsub_rn(v, L);
-  const long long b = __double_as_longlong(v);
-  if (b < 0 && (b << 1) != 0) v = __dadd_rn(v, L);
-  return v;
-}
-
 // Cell of every slot from the fixed-point position the last step wrote.
 __device__ __forceinline__ void rebin_keys_body(const Sys& S, const Blk blk) {
   Ctl* ctl = S.ctl;
@@ -720,33 +417,6 @@ __global__ void kb_scan_tiles(const Sys* __restrict__ T, const BlkMap* __restric
   const Sys& S = T[m.sys];
   if (!S.ctl->rebin_flag) return;
   scan_tiles_body(S, Blk{m.b, m.nb});
-}
-
-__device__ __forceinline__ uint32_t block_exclusive_scan_256(uint32_t v, uint32_t& total) {
-  __shared__ uint32_t warp_tot[8];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_tot[wid] = x;
-  __syncthreads();
-  if (wid == 0) {
-    uint32_t t = lane < 8 ? warp_tot[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, t, o);
-      if (lane >= o) t += y;
-    }
-    if (lane < 8) warp_tot[lane] = t;
-  }
-  __syncthreads();
-  const uint32_t before = wid ? warp_tot[wid - 1] : 0u;
-  total = warp_tot[7];
-  __syncthreads();
-  return before + x - v;
 }
 
 // Single block: exclusive scan of the tile sums in place.
@@ -993,274 +663,15 @@ __global__ void kb_rebin_permute(const Sys* __restrict__ T, const BlkMap* __rest
   rebin_permute_body(S, Blk{m.b, m.nb}, true);
 }
 
-// ---------------------------------------------------------------------------
-// Verlet-list build.  One block per tile of TY consecutive cell rows (cy0 ..
-// cy0+TY-1 at one cz); threads = the tile's particles, contiguous in slot
-// order (in passes of blockDim when a tile is longer).  All (TY+2) x 3
-// neighbour rows are staged in shared memory as FP32 coordinates in the
-// tile's frame (one pass in the common case), each row extended by one
-// periodic image cell at both ends, so every particle's 3 x 3 x 3 cell
-// neighbourhood is 9 contiguous ranges.  A pair enters the list when its
-// FP32 distance is below r_c + skin (widened by the rounding bound).
-// ---------------------------------------------------------------------------
-// 16-byte copy global -> shared that does not wait for the data (cp.async,
-// L2 only); cp_async_wait_all() waits for every copy the thread issued.
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-struct RowInfo {
-  int base;        // first staged index of the row
-  int padL;        // particles of the left image cell (cell nx-1)
-  int rowcount;    // particles of the row
-  int tot;         // padL + rowcount + padR
-  int row_lo;      // first slot of the row
-  int left_start;  // first slot of cell nx-1
-  int c1;          // first slot of cell 1 (end of cell 0)
-  uint32_t yref;   // fixed-point lower edge of the (wrapped) row in y
-  uint32_t zref;   // and in z
-  float yoff;      // that edge's offset from the tile's lower edge, unwrapped
-  float zoff;
-  int pad;
-};
-constexpr int TILE_ROWS_MAX = 18;  // (TY + 2) x 3 for TY <= 4
-
-// FP32 coordinates of a staged particle in the tile's frame: y and z relative
-// to the tile's lower cell edges (each row's images unwrapped), x in [0, L)
-// with the left and right image cells shifted by -L and +L.  A slot keyed to
-// cell 0 (nx-1) whose position rounds to the far end of the box (possible by
-// one rounding step after a restore) is taken back to the near side.  The
-// values carry ~1e-5 sigma of rounding; the list radius has a margin for it.
-__device__ __forceinline__ float4 build_coords(const uint4 p, const RowInfo& r, int kr,
-                                               uint32_t slot, float sx, float sy, float sz,
-                                               float Lx) {
-  float xf = __uint2float_rn(p.x) * sx;
-  if (slot < (uint32_t)r.c1 && p.x >= 0x80000000u) xf -= Lx;
-  if (slot >= (uint32_t)r.left_start && p.x < 0x80000000u) xf += Lx;
-  if (kr < r.padL) xf -= Lx;
-  else if (kr >= r.padL + r.rowcount) xf += Lx;
-  const float yf = fmaf(__int2float_rn(pdiff(p.y, r.yref)), sy, r.yoff);
-  const float zf = fmaf(__int2float_rn(pdiff(p.z, r.zref)), sz, r.zoff);
-  return make_float4(xf, yf, zf, __uint_as_float(slot));
-}
-
-// One candidate: hit = r2 < rv2; a hit is written to row `cnt` of the
-// slot's column while cnt < cap, and cnt counts every hit (cnt > cap
-// afterwards means the list overflowed).  The caller never passes the
-// particle itself.  Predicated PTX, so that the warp does not diverge on the
-// (frequent) hits.
-template <bool NL16>
-__device__ __forceinline__ void list_candidate(unsigned char* col, uint32_t stride, float r2,
-                                               float rv2, uint32_t qslot, int cap, int& cnt) {
-  if constexpr (NL16) {
-    asm volatile(
-        "{\n\t.reg .pred h, w;\n\t.reg .u64 a;\n\t"
-        "setp.lt.f32 h, %1, %2;\n\t"
-        "setp.lt.and.s32 w, %0, %4, h;\n\t"
-        "mad.wide.u32 a, %0, %5, %6;\n\t"
-        "@w st.global.u16 [a], %7;\n\t"
-        "@h add.s32 %0, %0, 1;\n\t}"
-        : "+r"(cnt)
-        : "f"(r2), "f"(rv2), "r"(qslot), "r"(cap), "r"(stride), "l"(col), "h"((uint16_t)qslot)
-        : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred h, w;\n\t.reg .u64 a;\n\t"
-        "setp.lt.f32 h, %1, %2;\n\t"
-        "setp.lt.and.s32 w, %0, %4, h;\n\t"
-        "mad.wide.u32 a, %0, %5, %6;\n\t"
-        "@w st.global.u32 [a], %3;\n\t"
-        "@h add.s32 %0, %0, 1;\n\t}"
-        : "+r"(cnt)
-        : "f"(r2), "f"(rv2), "r"(qslot), "r"(cap), "r"(stride), "l"(col)
-        : "memory");
-  }
-}
-
+// One tile per block; the last warp of the system's tiles flips the SoA set
+// and clears the flag (a warp count, not a block barrier: warps that finish
+// early leave).
 template <bool NL16>
 __device__ __forceinline__ void build_nlist_body(const Sys& S, const Blk blk, unsigned char* smem) {
-  const int CAP = S.tile_cap;
-  float4* sX = reinterpret_cast<float4*>(smem);
-  RowInfo* ri = reinterpret_cast<RowInfo*>(smem + 16 * (size_t)CAP);
-  uint32_t* sCS = reinterpret_cast<uint32_t*>(ri + TILE_ROWS_MAX);
-  __shared__ int sTOT;
   __shared__ unsigned int warps_left;
   if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
-
   Ctl* ctl = S.ctl;
-  const uint4* __restrict__ P = ctl->phase ? S.P1 : S.P0;
-  const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
-  const int ty = blk.b % S.tiles_y, cz = blk.b / S.tiles_y;
-  const int cy0 = ty * S.tile_y;
-  const int TYb = min(S.tile_y, ny - cy0);
-  const int RY = TYb + 2, R = 3 * RY;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const uint32_t rs = S.cell_start[(cz * ny + cy0) * nx];
-  const uint32_t re = S.cell_start[(cz * ny + cy0 + TYb - 1) * nx + nx];
-
-  for (int k = threadIdx.x; k < R * (nx + 1); k += blockDim.x) {
-    const int sr = k / (nx + 1), c = k - sr * (nx + 1);
-    const int dzi = sr / RY, yi = sr - dzi * RY;
-    const int qz = wrap_cell(cz - 1 + dzi, nz), qy = wrap_cell(cy0 - 1 + yi, ny);
-    sCS[k] = S.cell_start[(qz * ny + qy) * nx + c];
-  }
-  __syncthreads();
-  if (threadIdx.x < R) {
-    const uint32_t* cs = sCS + threadIdx.x * (nx + 1);
-    const int dzi = threadIdx.x / RY, yi = threadIdx.x - dzi * RY;
-    const int uy = cy0 - 1 + yi, uz = cz - 1 + dzi;  // unwrapped row indices
-    const int qy = wrap_cell(uy, ny), qz = wrap_cell(uz, nz);
-    RowInfo r;
-    r.padL = (int)(cs[nx] - cs[nx - 1]);
-    r.rowcount = (int)(cs[nx] - cs[0]);
-    r.tot = r.padL + r.rowcount + (int)(cs[1] - cs[0]);
-    r.row_lo = (int)cs[0];
-    r.left_start = (int)cs[nx - 1];
-    r.c1 = (int)cs[1];
-    r.yref = (uint32_t)(((unsigned long long)qy << 32) / (unsigned)ny);
-    r.zref = (uint32_t)(((unsigned long long)qz << 32) / (unsigned)nz);
-    r.yoff = (float)((double)(uy - cy0) * (S.L[1] / ny));
-    r.zoff = (float)((double)(uz - cz) * (S.L[2] / nz));
-    r.base = 0;
-    r.pad = 0;
-    ri[threadIdx.x] = r;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int sr = 0; sr < R; ++sr) {
-      ri[sr].base = run;
-      run += ri[sr].tot;
-    }
-    sTOT = run;
-  }
-  __syncthreads();
-  const int TOT = sTOT;
-  const float sx = S.scale[0], sy = S.scale[1], sz = S.scale[2], rv2 = S.rv2_build;
-  const float Lx = (float)S.L[0];
-
-  // Stages entries [c0, c0 + cn) of the neighbour rows, one warp per row:
-  // raw copies in flight at once (cp.async), then each lane turns the
-  // entries it copied into tile-frame FP32 coordinates in place (the same
-  // warp/lane mapping, so no block barrier in between).
-  auto stage = [&](int c0, int cn) {
-    for (int sr = warp; sr < R; sr += nwarps) {
-      const RowInfo& r = ri[sr];
-      const int k0 = max(r.base, c0), k1 = min(r.base + r.tot, c0 + cn);
-      const int padL = r.padL, rc = r.rowcount, lo = r.row_lo, ls = r.left_start, b = r.base;
-      for (int ent = k0 + lane; ent < k1; ent += 32) {
-        const int kr = ent - b;
-        const int slot = kr < padL ? ls + kr : (kr < padL + rc ? lo + kr - padL : lo + kr - padL - rc);
-        cp_async16(&sX[ent - c0], P + slot);
-      }
-    }
-    cp_async_wait_all();
-    __syncwarp();
-    for (int sr = warp; sr < R; sr += nwarps) {
-      const RowInfo r = ri[sr];
-      const int k0 = max(r.base, c0), k1 = min(r.base + r.tot, c0 + cn);
-      for (int ent = k0 + lane; ent < k1; ent += 32) {
-        const int kr = ent - r.base;
-        const int slot = kr < r.padL ? r.left_start + kr
-                                     : r.row_lo + (kr < r.padL + r.rowcount ? kr - r.padL
-                                                                            : kr - r.padL - r.rowcount);
-        const float4 raw = sX[ent - c0];
-        const uint4 p = make_uint4(__float_as_uint(raw.x), __float_as_uint(raw.y),
-                                   __float_as_uint(raw.z), 0u);
-        sX[ent - c0] = build_coords(p, r, kr, (uint32_t)slot, sx, sy, sz, Lx);
-      }
-    }
-  };
-  const bool one = TOT <= CAP;  // the common case: every row staged once
-  if (one) {
-    stage(0, TOT);
-    __syncthreads();
-  }
-
-  for (uint32_t base = rs; base < re; base += blockDim.x) {
-    const uint32_t i = base + threadIdx.x;
-    const bool act = i < re;
-    const uint4 pi = act ? P[i] : make_uint4(0u, 0u, 0u, 0u);
-    // the cell the sort put this slot in (not the one its current position
-    // maps to: after a checkpoint restore the two can differ by one)
-    const uint32_t kc = act ? S.tmp[i] : (uint32_t)((cz * ny + cy0) * nx);
-    int cx = (int)(kc % (uint32_t)nx);
-    int yrel = (int)((kc / (uint32_t)nx) % (uint32_t)ny) - cy0;
-    if (yrel < 0 || yrel >= TYb) {  // cannot happen for a consistent sort
-      set_status(ctl, PRX_EINVAL);
-      yrel = 0;
-      cx = 0;
-    }
-    uint32_t win[9];
-#pragma unroll
-    for (int w = 0; w < 9; ++w) {
-      const int sr = (w / 3) * RY + yrel + (w % 3);
-      const uint32_t* cs = sCS + sr * (nx + 1);
-      const RowInfo& r = ri[sr];
-      const int lo = r.base + (cx == 0 ? 0 : r.padL + (int)cs[cx - 1] - r.row_lo);
-      const int hi = r.base + (cx + 2 > nx ? r.tot : r.padL + (int)cs[cx + 2] - r.row_lo);
-      win[w] = (uint32_t)lo | ((uint32_t)hi << 16);
-    }
-    float4 fi;
-    int kself0;  // the particle's own entry in the staged centre row
-    {
-      const RowInfo& r = ri[RY + yrel + 1];
-      fi = build_coords(pi, r, r.padL + ((int)i - r.row_lo), i, sx, sy, sz, Lx);
-      kself0 = r.base + r.padL + ((int)i - r.row_lo);
-    }
-    int cnt = 0;
-    const int cap = S.list_cap;
-    unsigned char* col = (unsigned char*)S.nl + (size_t)i * (NL16 ? 2 : 4);
-    const uint32_t stride = S.n * (NL16 ? 2u : 4u);
-    for (int c0 = 0; c0 < TOT; c0 += CAP) {
-      const int cn = min(CAP, TOT - c0);
-      if (!one) {  // neighbour rows longer than the buffer: staged per chunk
-        __syncthreads();
-        stage(c0, cn);
-        __syncthreads();
-      }
-      if (act) {
-        // the particle itself is staged once, in the centre row's window
-        // (w = 4), whose walk skips it: no candidate needs a self test
-        const int kself = kself0 - c0;
-#pragma unroll
-        for (int w = 0; w < 9; ++w) {
-          const int lo = max((int)(win[w] & 0xFFFFu), c0) - c0;
-          const int hi = min((int)(win[w] >> 16), c0 + cn) - c0;
-          auto walk = [&](int a, int b) {
-#pragma unroll 2
-            for (int k = a; k < b; ++k) {
-              const float4 q = sX[k];
-              const float dx = q.x - fi.x, dy = q.y - fi.y, dz = q.z - fi.z;
-              list_candidate<NL16>(col, stride, fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rv2,
-                                   __float_as_uint(q.w), cap, cnt);
-            }
-          };
-          if (w == 4) {
-            walk(lo, min(hi, max(lo, kself)));
-            walk(max(lo, kself + 1), hi);
-          } else {
-            walk(lo, hi);
-          }
-        }
-      }
-    }
-    if (act) {
-      const int m = min(cnt, cap);
-      S.nn[i] = (uint8_t)m;
-      if (cnt > cap) set_status(ctl, PRX_ECAPACITY);
-      // pad to a whole stage of four with the slot itself (the step kernel
-      // gathers four entries at a time; the self pair has r = 0 and no force)
-      for (int k = m; k < ((m + 3) & ~3); ++k) {
-        if constexpr (NL16) ((uint16_t*)S.nl)[(size_t)k * S.n + i] = (uint16_t)i;
-        else ((uint32_t*)S.nl)[(size_t)k * S.n + i] = i;
-      }
-    }
-  }
-  // the last warp of the system's tiles flips the SoA set and clears the
-  // flag (a warp count, not a block barrier: warps that finish early leave)
+  build_tile<NL16>(S, ctl->phase ? S.P1 : S.P0, S.tmp, blk.b, smem);
   if (last_warp(&ctl->done_rebin, &warps_left, blk.nb)) {
     ctl->done_rebin = 0u;
     ctl->set ^= 1;

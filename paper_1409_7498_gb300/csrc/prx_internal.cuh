@@ -38,6 +38,8 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t SLOT_MASK = 0x7FFFFFFFu;
 constexpr int STEP_THREADS = 128;
 constexpr int RX_THREADS = 256;
+constexpr unsigned ENG_BUCKET = 16;    // slots per cell bucket of the persistent runs
+constexpr unsigned ENG_CELLS = 32768;  // cells up to which a block scans all counts itself
 constexpr int SCAN_TILE = 2048;  // elements per scan tile (256 threads x 8)
 
 // Counter tags of the keyed Philox draws (fourth counter word, low byte).
@@ -180,6 +182,12 @@ struct Sys {
   float rv2_build;                // (r_c + skin + rounding margin)^2, list build test (FP32)
   // list-build tiling (cells of edge >= r_c + skin)
   int tile_y, tiles_y, tile_threads, tile_cap;
+  // persistent runs of small systems: buckets of the cells (ENG_BUCKET slots
+  // each), tiles of their list build (rows, staged entries, slots)
+  uint32_t* bucket;
+  int eng_ty, eng_tiles_y, eng_cap, eng_slots;
+  unsigned long long inv_nc64[2];  // ceil(2^64 / nc) for y and z
+  float cell_edge_f[2];            // cell edges in y and z
   // physics (FP32 and FP64 copies)
   float rc2f, sig2f, eps24f, eps4f, fcapf, fkf, fr02f, fr02if, rcf, sigf;
   int cubic;        // equal edges: the neighbour loop runs in position units
@@ -389,6 +397,17 @@ void launch_stage_input(const Sys& S, cudaStream_t st, const double* buf, int wh
 // 0 states, 1 types, 2 positions wrapped into the box, 3 velocities.
 void launch_gather_by_id(const Sys& S, cudaStream_t st, int what, void* out);
 int configure_build_kernel(size_t smem_bytes);
+// Multiprocessors of the current device.
+unsigned device_sms();
+// Persistent runs (engine.cu).
+struct EngPlan {
+  const void* kernel = nullptr;
+  unsigned blocks = 0;  // 0: the system's runs do not go through a persistent kernel
+  size_t smem = 0;
+};
+EngPlan engine_plan(const Sys& S, int fp64);
+cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint32_t nsteps, uint32_t theta,
+                          unsigned long long* bar, unsigned long long* bar_next);
 // Device-driven runs (dg.cu): k_dg_arm stores the run's step count and the
 // rebuild and reaction device graphs in the control block; k_dg_next, the
 // last kernel of the step's device graph, tail-launches what follows.

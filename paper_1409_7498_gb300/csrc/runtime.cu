@@ -1,7 +1,9 @@
 // Host runtime of polyrx: the C ABI of include/polyrx.h.
 //
-// A system owns its device buffers (layout in prx_internal.cuh), a private
-// capture stream and three CUDA graphs built once per reaction scheme:
+// A system owns its device buffers (layout in prx_internal.cuh) and a private
+// capture stream.  Runs of small systems go through the persistent kernel of
+// engine.cu; the others through CUDA graphs built once per reaction scheme:
+// the device graphs of dg.cu or, where those are not available,
 //   step   : one step kernel followed by an IF node whose body rebuilds the
 //            cell list; the step kernel's last block sets the condition from
 //            the device flag, so a rebuild runs exactly when some particle
@@ -73,6 +75,12 @@ struct prx_system {
   cudaGraphExec_t dg_step = nullptr, dg_rebuild = nullptr, dg_react = nullptr;
   bool dg_ok = false;
   bool graphs_valid = false;
+  // persistent runs (engine.cu): the barrier words, the plan (once asked
+  // for), the launches so far
+  unsigned long long* eng_bar = nullptr;
+  EngPlan eng;
+  bool eng_planned = false;
+  uint64_t eng_launches = 0;
   bool profiling = false;
   std::vector<ProfEvent> prof;
   std::string err;
@@ -310,10 +318,11 @@ int setup_grid(prx_system* sys, double rc) {
   }
   S.ncell = (int)ncell;
   sys->grid_rcut = rc;
+  sys->eng_planned = false;
   free_list(sys->grid_allocs);
   int rc2;
   DevArena A;
-  A.add(&S.cell_start, (size_t)ncell + 1), A.add(&S.count, (size_t)ncell), A.add(&S.fill, (size_t)ncell);
+  A.add(&S.cell_start, (size_t)ncell + 1), A.add(&S.count, ((size_t)ncell + 3) & ~(size_t)3), A.add(&S.fill, (size_t)ncell);
   const size_t nblk = std::max<size_t>((S.n + RX_THREADS - 1) / RX_THREADS,
                                        ((size_t)ncell + SCAN_TILE - 1) / SCAN_TILE) + 1;
   A.add(&S.blk_count, nblk), A.add(&S.blk_off, nblk);
@@ -327,6 +336,7 @@ int setup_grid(prx_system* sys, double rc) {
   S.nl16 = S.n <= 65535 ? 1 : 0;
   A.add((uint8_t**)&S.nl, (size_t)S.list_cap * S.n * (S.nl16 ? 2 : 4));
   A.add(&S.nn, (size_t)S.n);
+  A.add(&S.bucket, ncell <= (long long)ENG_CELLS ? (size_t)ncell * ENG_BUCKET : 0);
   if ((rc2 = A.commit(sys, sys->grid_allocs))) return rc2;
   {
     // list-build tiling: the largest tile of 1..4 cell rows whose particles
@@ -350,6 +360,31 @@ int setup_grid(prx_system* sys, double rc) {
     const size_t budget = 160 * 1024;
     if (fixed + 16 * (size_t)cap > budget) cap = (int)((budget - fixed) / 16);
     S.tile_cap = std::max(64, std::min(cap, 65535));
+    // persistent runs: the rows per tile whose list build is shortest when one
+    // block per SM takes the tiles in turn (a tile's staging costs about as
+    // much as 1.6 rounds of its 512 threads over (slot, layer) pairs)
+    double best = 0.0;
+    S.eng_ty = 0;  // 0: rows or windows too long for its tiles and masks
+    const bool windows = 3.0 * per_cell + 4.0 * std::sqrt(3.0 * per_cell) <= 32.0;
+    for (int c = 1; c <= 4 && c <= S.nc[1] && windows; ++c) {
+      const double slots = c * per_row + 4.0 * std::sqrt(c * per_row) + 16.0;
+      if (3.0 * slots > 1024.0) break;
+      const double tiles = (double)((S.nc[1] + c - 1) / c) * S.nc[2];
+      const double cost = std::ceil(tiles / (double)device_sms()) * (1.6 + std::ceil(3.0 * c * per_row / 512.0));
+      if (!S.eng_ty || cost < best) {
+        best = cost;
+        S.eng_ty = c;
+        S.eng_slots = (int)slots;
+        const double tot = 3.0 * (c + 2) * (per_row + 2.0 * per_cell);
+        S.eng_cap = (int)std::ceil((tot + 4.0 * std::sqrt(tot) + 64.0) / 32.0) * 32;
+      }
+    }
+    S.eng_cap = std::min(S.eng_cap, 6000);  // (a tile that needs more takes the unstaged path)
+    S.eng_tiles_y = S.eng_ty ? (S.nc[1] + S.eng_ty - 1) / S.eng_ty : 0;
+    for (int k = 0; k < 2; ++k) {
+      S.inv_nc64[k] = ~0ull / (unsigned long long)S.nc[1 + k] + 1ull;
+      S.cell_edge_f[k] = (float)(S.L[1 + k] / S.nc[1 + k]);
+    }
     if (configure_build_kernel(build_tile_smem(S)))
       return fail(sys, PRX_ECUDA, "cannot set the list-build kernel's shared-memory size");
   }
@@ -515,6 +550,34 @@ int ensure_graphs(prx_system* sys) {
     if (m > 1 && (rc = build_graph(sys, kNoRxChunk, false, &sys->g_chunk1))) return rc;
   }
   sys->graphs_valid = true;
+  return PRX_OK;
+}
+
+// Whether the system's runs go through the persistent kernel.
+bool engine_fits(prx_system* sys) {
+  if (!sys->eng_planned) {
+    sys->eng = engine_plan(sys->S, sys->d.force_precision == PRX_FORCE_FP64);
+    sys->eng_planned = true;
+  }
+  return sys->eng.blocks > 0;
+}
+
+// nsteps steps in persistent launches of a few hundred steps each (so that
+// other streams' work gets its turn on the GPU in between).
+int engine_run(prx_system* sys, uint64_t nsteps) {
+  const uint64_t per = std::min<uint64_t>(std::max<uint64_t>(256, (nsteps + 511) / 512), 1u << 16);
+  const uint32_t theta = sys->has_rx ? sys->rxd.theta : 0u;
+  while (nsteps) {
+    const uint64_t k = std::min(per, nsteps);
+    unsigned long long* bar = sys->eng_bar + 32 * (sys->eng_launches & 1u);
+    unsigned long long* next = sys->eng_bar + 32 * ((sys->eng_launches + 1u) & 1u);
+    CK(launch_engine(sys->S, sys->stream, sys->eng, (uint32_t)k, theta, bar, next));
+    sys->eng_launches++;
+    if (theta) sys->graph_rx_launches += (sys->host_step + k) / theta - sys->host_step / theta;
+    sys->host_step += k;
+    sys->step_launches += k;
+    nsteps -= k;
+  }
   return PRX_OK;
 }
 
@@ -694,6 +757,7 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   A.add(&S.pop, (size_t)POP_REPLICAS * PRX_MAX_TYPES * PRX_MAX_STATES);
   A.add(&S.red, 4 * ((size_t)(n + RX_THREADS - 1) / RX_THREADS + 1));
   A.add(&S.fout, 3 * (size_t)n), A.add(&S.eout, (size_t)n);
+  A.add(&sys->eng_bar, 64);
   if ((rc = A.commit(sys, sys->dev_allocs))) return bail(rc);
   if ((rc = setup_grid(sys, grid_rc > rc_w ? grid_rc : rc_w))) return bail(rc);
 
@@ -826,7 +890,8 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   c0.step = step0;
   if ((rc = up(S.ctl, &c0, sizeof(Ctl)))) return bail(rc);
   sys->host_step = step0;
-  if (cudaMemsetAsync(S.hist, 0, sizeof(HistRec) * (S.hist_cap + 2), sys->stream) != cudaSuccess)
+  if (cudaMemsetAsync(S.hist, 0, sizeof(HistRec) * (S.hist_cap + 2), sys->stream) != cudaSuccess ||
+      cudaMemsetAsync(sys->eng_bar, 0, 8 * 64, sys->stream) != cudaSuccess)
     return bail(fail(sys, PRX_ECUDA, "memset failed"));
 
   if (slot_cells) {
@@ -1072,7 +1137,7 @@ uint64_t estimate_bytes(const prx_system_desc& d, double r_react) {
   const uint64_t allocs = 40;  // separate cudaMalloc calls, each rounded up
   return 2 * per_set + n * (2 * 16 + 4 * 4) + (n * cap / 2 + 1) * sizeof(prx_bond) +
            (kHistCap + 2ull) * sizeof(prx_history_record) + sizeof(Ctl) + 32 * (n / RX_THREADS + 2) +
-           32 * n + ncell * 12 + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + allocs * 4096;
+           32 * n + ncell * 12 + (ncell <= ENG_CELLS ? ncell * 4 * ENG_BUCKET : 0) + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + allocs * 4096;
 }
 
 
@@ -1245,6 +1310,7 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
     }
     return PRX_OK;
   }
+  if (engine_fits(sys)) return engine_run(sys, nsteps);
   int rc = ensure_graphs(sys);
   if (rc) return rc;
   if (sys->dg_ok) {
@@ -1861,6 +1927,7 @@ int prx_set_launch_config(prx_system* sys, const prx_launch_config* cfg) {
   sys->S.step_lanes = (int)lanes;
   sys->S.step_bpsm = (int)cfg->step_blocks_per_sm;
   sys->chunk_m = cfg->chunk_intervals ? cfg->chunk_intervals : 1u;
+  sys->eng_planned = false;
   destroy_graphs(sys);
   return PRX_OK;
 }
