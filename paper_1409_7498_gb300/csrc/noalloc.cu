@@ -9,7 +9,9 @@
 // library until the process exits.
 //
 // The candidate search is all-pairs (at most PRX_NOALLOC_MAX_N particles), so
-// no cell list or neighbour list is needed.  Both selection rules of
+// no cell list or neighbour list is needed: one kind of particle fits in an
+// SM's shared memory as FP32 coordinates, which decide every pair that is
+// clearly out of range; the few others take the exact FP64 test.  Both selection rules of
 // prx_react_once are implemented with its keyed Philox draws, its FP64
 // distance test and its tie-breaking, so the two agree bit for bit on the
 // same state: Table I's random rule (one T per A, then one A per T, each the
@@ -17,6 +19,7 @@
 // (mutual nearest A-T pairs, then the acceptance draw).
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <mutex>
 
 #include "prx_internal.cuh"
@@ -29,9 +32,11 @@ struct NaScratch {
   uint32_t win[PRX_NOALLOC_MAX_N];  // random rule: chosen T of each A (Table I step 5);
                                     // nearest rule: nearest partner of each A and T
   uint32_t fin[PRX_NOALLOC_MAX_N];  // surviving pairs (step 7), by A
+  uint16_t list[PRX_NOALLOC_MAX_N]; // the A's that chose a T, in any order
   unsigned long long trace[4];
   unsigned int nbonds;
   int status;
+  unsigned int nlist;
 };
 
 // The scratch.  Every call shares it and it keeps the last call's contents;
@@ -53,6 +58,8 @@ struct NaArgs {
   uint64_t seed;
   unsigned long long step;
   RxParams R;
+  float Lf[3], invLf[3];
+  float near2;  // FP32 r^2 from which a pair is out of range for sure
   NaScratch* sc;
 };
 
@@ -83,104 +90,180 @@ __device__ __forceinline__ bool na_bonded(const NaArgs& a, uint32_t i, uint32_t 
   return bonded;
 }
 
-// LAMMPS rule (Sec. IV.A): the eligible partner of the other kind (a T when
-// want_T, else an A) within r_react of particle i, not bonded to it, of
-// smallest exact r^2, ties to the smaller id; in_range counts the pairs in
-// range.
-__device__ __forceinline__ uint32_t na_nearest(const NaArgs& a, uint32_t i, bool want_T,
-                                               unsigned long long& in_range) {
-  const double xi = a.pos[3 * (size_t)i], yi = a.pos[3 * (size_t)i + 1], zi = a.pos[3 * (size_t)i + 2];
-  uint32_t best = NONE;
-  double best_r2 = 0.0;
-  for (uint32_t j = 0; j < a.n; ++j) {
-    if (j == i) continue;
-    const bool ok = want_T ? na_window(a.R.mask_T, a.R.t_lo, a.R.t_hi, a.type[j], a.state[j])
-                           : na_window(a.R.mask_A, a.R.a_lo, a.R.a_hi, a.type[j], a.state[j]);
-    if (!ok) continue;
-    const double r2 = na_r2(a, i, j, xi, yi, zi);
-    if (r2 < 0.0 || na_bonded(a, i, j)) continue;
-    ++in_range;
-    // j ascends, so a tie keeps the earlier (smaller) id
-    if (best == NONE || r2 < best_r2) {
-      best = j;
-      best_r2 = r2;
-    }
-  }
-  return best;
+// The particles a block searches for: NA_BLOCKS blocks share them in ranges.
+constexpr int NA_BLOCKS = 128, NA_THREADS = 1024, NA_WARPS = NA_THREADS / 32;
+constexpr int NA_RANGE = (PRX_NOALLOC_MAX_N + NA_BLOCKS - 1) / NA_BLOCKS;
+
+// binary64 -> binary32 towards zero on the integer pipe (error below 2^-23
+// of the value; values below 2^-126 become 0, beyond 2^128 or not finite a
+// NaN, which no later test rejects).
+__device__ __forceinline__ float na_f32(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const uint32_t e = (uint32_t)(b >> 52) & 0x7FFu, sign = (uint32_t)(b >> 32) & 0x80000000u;
+  if (e < 897u) return __uint_as_float(sign);
+  if (e > 1150u) return __uint_as_float(0x7FC00000u);
+  return __uint_as_float(sign | ((uint32_t)(b >> 29) & 0x7FFFFFu) | ((e - 896u) << 23));
 }
 
-// Steps 1-5, one thread per particle id, all pairs (random rule); for the
-// nearest rule each eligible A records its nearest eligible T.
-__global__ void k_na_find(NaArgs a) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.n) return;
-  uint32_t best = NONE;
+// Steps 1-5.  Random rule: each eligible A's retained T of smallest selection
+// key.  Nearest rule: each eligible A's nearest eligible T and, in a second
+// pass, each eligible T's nearest eligible A (smallest exact r^2, ties to the
+// smaller id).  Per pass every block stages all particles of the partner's
+// kind (FP32 coordinates, 14 bytes each) and searches them for its own range
+// of particles; the warps are shared out over the block's particles, so that
+// a few A's among many T's still keep all of them busy.  Bound by the FP32
+// instructions of the pair test (16 per pair) and the staging: a call with
+// 8,192 particles, 11% of them A, takes 102 us (one thread per particle and
+// FP64 tests of every pair: 11,900 us).  A coordinate more than a box edge outside the
+// box sends every pair to the exact test.
+__global__ void __launch_bounds__(NA_THREADS, 1) k_na_find(NaArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  float* sx = reinterpret_cast<float*>(smem);
+  float *sy = sx + a.n, *sz = sy + a.n;
+  uint16_t* sid = reinterpret_cast<uint16_t*>(sz + a.n);
+  __shared__ uint16_t own[NA_RANGE];
+  __shared__ unsigned long long ckey[NA_WARPS];
+  __shared__ uint32_t cid[NA_WARPS];
+  __shared__ uint32_t nstaged, nown;
+  __shared__ int far;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool nearest = a.R.rule == PRX_SELECT_NEAREST;
+  const uint32_t lo = (uint32_t)((unsigned long long)a.n * blockIdx.x / NA_BLOCKS);
+  const uint32_t hi = (uint32_t)((unsigned long long)a.n * (blockIdx.x + 1u) / NA_BLOCKS);
+  auto is_A = [&](uint32_t j) { return na_window(a.R.mask_A, a.R.a_lo, a.R.a_hi, a.type[j], a.state[j]); };
+  auto is_T = [&](uint32_t j) { return na_window(a.R.mask_T, a.R.t_lo, a.R.t_hi, a.type[j], a.state[j]); };
+  for (uint32_t i = lo + threadIdx.x; i < hi; i += NA_THREADS) a.sc->win[i] = a.sc->fin[i] = NONE;
   unsigned long long cand = 0, ret = 0;
-  const bool isA = na_window(a.R.mask_A, a.R.a_lo, a.R.a_hi, a.type[i], a.state[i]);
-  if (isA && a.R.rule == PRX_SELECT_NEAREST) {
-    best = na_nearest(a, i, true, cand);
-  } else if (isA) {
-    const double xi = a.pos[3 * (size_t)i], yi = a.pos[3 * (size_t)i + 1], zi = a.pos[3 * (size_t)i + 2];
-    unsigned long long bestkey = 0ull;
-    for (uint32_t j = 0; j < a.n; ++j) {
-      if (j == i || !na_window(a.R.mask_T, a.R.t_lo, a.R.t_hi, a.type[j], a.state[j])) continue;
-      if (na_r2(a, i, j, xi, yi, zi) < 0.0 || na_bonded(a, i, j)) continue;
-      ++cand;
-      const uint4 wa = keyed_draw(a.seed, a.step, i, j, TAG_ACCEPT);
-      if (!u53_below(wa.x, wa.y, a.R.p53)) continue;
-      ++ret;
-      const unsigned long long k = na_key64(keyed_draw(a.seed, a.step, i, j, TAG_SEL_A));
-      if (best == NONE || k < bestkey || (k == bestkey && j < best)) {
-        best = j;
-        bestkey = k;
+  for (int pass = 0; pass < (nearest ? 2 : 1); ++pass) {
+    __syncthreads();
+    if (threadIdx.x == 0) nstaged = nown = 0u, far = 0;
+    __syncthreads();
+    for (uint32_t base = 0; base < a.n; base += NA_THREADS) {
+      const uint32_t j = base + threadIdx.x;
+      const bool el = j < a.n && (pass ? is_A(j) : is_T(j));
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, el);
+      uint32_t at = 0u;
+      if (lane == 0 && bal) at = atomicAdd(&nstaged, (uint32_t)__popc(bal));
+      at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+      if (el) {
+        const double x = a.pos[3 * (size_t)j], y = a.pos[3 * (size_t)j + 1], z = a.pos[3 * (size_t)j + 2];
+        sx[at] = na_f32(x), sy[at] = na_f32(y), sz[at] = na_f32(z);
+        sid[at] = (uint16_t)j;
+        // (also true for values that are not numbers)
+        if (!(fabsf(sx[at]) <= 2.f * a.Lf[0] && fabsf(sy[at]) <= 2.f * a.Lf[1] && fabsf(sz[at]) <= 2.f * a.Lf[2]))
+          far = 1;
       }
     }
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += NA_THREADS)
+      if (pass ? is_T(i) : is_A(i)) own[atomicAdd(&nown, 1u)] = (uint16_t)i;
+    __syncthreads();
+    const uint32_t ns = nstaged, nq = nown;
+    // W warps per particle of the block's own
+    uint32_t W = NA_WARPS;
+    while (W > 1u && (NA_WARPS / W) < nq) W >>= 1;
+    const uint32_t groups = NA_WARPS / W, grp = (uint32_t)warp / W, part = (uint32_t)warp % W;
+    for (uint32_t q0 = 0; q0 < nq; q0 += groups) {
+      const bool has = q0 + grp < nq;
+      const uint32_t i = has ? own[q0 + grp] : 0u;
+      unsigned long long best = ~0ull;  // selection key, or the bits of r^2
+      uint32_t bestid = NONE;
+      if (has) {
+        const double xi = a.pos[3 * (size_t)i], yi = a.pos[3 * (size_t)i + 1], zi = a.pos[3 * (size_t)i + 2];
+        const float fx = na_f32(xi), fy = na_f32(yi), fz = na_f32(zi);
+        const bool all = far || !(fabsf(fx) <= 2.f * a.Lf[0] && fabsf(fy) <= 2.f * a.Lf[1] && fabsf(fz) <= 2.f * a.Lf[2]);
+        for (uint32_t e = part * 32u + (uint32_t)lane; e < ns; e += W * 32u) {
+          // nearest image: adding and taking off 1.5 2^23 rounds to an integer
+          float dx = sx[e] - fx, dy = sy[e] - fy, dz = sz[e] - fz;
+          dx = fmaf(-a.Lf[0], __fsub_rn(fmaf(dx, a.invLf[0], 12582912.f), 12582912.f), dx);
+          dy = fmaf(-a.Lf[1], __fsub_rn(fmaf(dy, a.invLf[1], 12582912.f), 12582912.f), dy);
+          dz = fmaf(-a.Lf[2], __fsub_rn(fmaf(dz, a.invLf[2], 12582912.f), 12582912.f), dz);
+          if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) >= a.near2 && !all) continue;
+          const uint32_t j = sid[e];
+          const double r2 = na_r2(a, i, j, xi, yi, zi);
+          if (r2 < 0.0 || na_bonded(a, i, j)) continue;
+          cand += pass ? 0u : 1u;
+          unsigned long long key;
+          if (nearest) {
+            key = (unsigned long long)__double_as_longlong(r2);  // (r2 >= 0: ordered as the values)
+          } else {
+            const uint4 wa = keyed_draw(a.seed, a.step, i, j, TAG_ACCEPT);
+            if (!u53_below(wa.x, wa.y, a.R.p53)) continue;
+            ++ret;
+            key = na_key64(keyed_draw(a.seed, a.step, i, j, TAG_SEL_A));
+          }
+          if (bestid == NONE || key < best || (key == best && j < bestid)) {
+            best = key;
+            bestid = j;
+          }
+        }
+      }
+      auto merge = [&](unsigned long long k2, uint32_t j2) {
+        if (j2 != NONE && (bestid == NONE || k2 < best || (k2 == best && j2 < bestid))) {
+          best = k2;
+          bestid = j2;
+        }
+      };
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long k2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        const uint32_t j2 = __shfl_xor_sync(0xFFFFFFFFu, bestid, o);
+        merge(k2, j2);
+      }
+      if (lane == 0) ckey[warp] = best, cid[warp] = bestid;
+      __syncthreads();
+      if (has && part == 0u && lane == 0) {
+        for (uint32_t w = 1; w < W; ++w) merge(ckey[warp + w], cid[warp + w]);
+        a.sc->win[i] = bestid;
+        if (bestid != NONE && !pass) a.sc->list[atomicAdd(&a.sc->nlist, 1u)] = (uint16_t)i;
+      }
+      __syncthreads();
+    }
   }
-  a.sc->win[i] = best;
-  if (cand) atomicAdd(&a.sc->trace[0], cand);
-  if (ret) atomicAdd(&a.sc->trace[1], ret);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    cand += __shfl_xor_sync(0xFFFFFFFFu, cand, o);
+    ret += __shfl_xor_sync(0xFFFFFFFFu, ret, o);
+  }
+  if (lane == 0 && cand) atomicAdd(&a.sc->trace[0], cand);
+  if (lane == 0 && ret) atomicAdd(&a.sc->trace[1], ret);
 }
 
-// Nearest rule: each eligible T records its nearest eligible A.  A and T
-// are disjoint sets, so the two kinds share win[].
-__global__ void k_na_find_T(NaArgs a) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.n || !na_window(a.R.mask_T, a.R.t_lo, a.R.t_hi, a.type[i], a.state[i])) return;
-  unsigned long long unused = 0;
-  a.sc->win[i] = na_nearest(a, i, false, unused);
-}
-
-// Steps 6-7 (random rule): an A keeps its T only if its key
-// Philox(step, id_T, id_A) is the smallest among the A's that chose the same
-// T.  Nearest rule: an A and the T it picked react when the T picked it too
-// and u < k dt Theta, drawn with the pair's smaller id first.
-__global__ void k_na_select(NaArgs a) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= a.n) return;
-  const uint32_t T = a.sc->win[i];
-  uint32_t fin = NONE;
-  const bool isA = na_window(a.R.mask_A, a.R.a_lo, a.R.a_hi, a.type[i], a.state[i]);
-  if (T != NONE && isA && a.R.rule == PRX_SELECT_NEAREST) {
-    if (a.sc->win[T] == i) {
+// Steps 6-7, one warp per A that chose a T (random rule): it keeps its T only
+// if its key Philox(step, id_T, id_A) is the smallest among the A's that
+// chose the same T, which are found in the list of those A's.  Nearest rule:
+// an A and the T it picked react when the T picked it too and u < k dt Theta,
+// drawn with the pair's smaller id first.
+__global__ void __launch_bounds__(256) k_na_select(NaArgs a) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t nl = a.sc->nlist;
+  for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nl; w += (gridDim.x * blockDim.x) >> 5) {
+    const uint32_t i = a.sc->list[w], T = a.sc->win[i];
+    if (a.R.rule == PRX_SELECT_NEAREST) {
+      if (lane != 0 || a.sc->win[T] != i) continue;
       atomicAdd(&a.sc->trace[1], 1ull);  // mutual pairs
-      const uint4 w = keyed_draw(a.seed, a.step, min(i, T), max(i, T), TAG_NEAREST);
-      if (u53_below(w.x, w.y, a.R.p53)) {
+      const uint4 d = keyed_draw(a.seed, a.step, min(i, T), max(i, T), TAG_NEAREST);
+      if (u53_below(d.x, d.y, a.R.p53)) {
         atomicAdd(&a.sc->trace[2], 1ull);  // accepted pairs
-        fin = T;
+        a.sc->fin[i] = T;
       }
+      continue;
     }
-  } else if (T != NONE && isA) {
-    atomicAdd(&a.sc->trace[2], 1ull);
-    const unsigned long long mine = na_key64(keyed_draw(a.seed, a.step, T, i, TAG_SEL_T));
-    bool keep = true;
-    for (uint32_t k = 0; k < a.n && keep; ++k) {
+    bool lost = false;
+    unsigned long long mine = 0ull;
+    bool drawn = false;
+    for (uint32_t v = (uint32_t)lane; v < nl; v += 32u) {
+      const uint32_t k = a.sc->list[v];
       if (k == i || a.sc->win[k] != T) continue;
+      if (!drawn) mine = na_key64(keyed_draw(a.seed, a.step, T, i, TAG_SEL_T)), drawn = true;
       const unsigned long long other = na_key64(keyed_draw(a.seed, a.step, T, k, TAG_SEL_T));
-      if (other < mine || (other == mine && k < i)) keep = false;
+      lost |= other < mine || (other == mine && k < i);
     }
-    if (keep) fin = T;
+    lost = __any_sync(0xFFFFFFFFu, lost);
+    if (lane == 0) {
+      atomicAdd(&a.sc->trace[2], 1ull);
+      if (!lost) a.sc->fin[i] = T;
+    }
   }
-  a.sc->fin[i] = fin;
 }
 
 // Step 9 in one block: bonds appended in ascending id of A (a running count
@@ -266,6 +349,9 @@ int na_scratch(NaScratch** out) {
   if (!g_na_ready[dev]) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || !p) return PRX_ECUDA;
+    if (cudaFuncSetAttribute(k_na_find, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             PRX_NOALLOC_MAX_N * (3 * (int)sizeof(float) + (int)sizeof(uint16_t))) != cudaSuccess)
+      return PRX_ECUDA;
     g_na_addr[dev] = static_cast<NaScratch*>(p);
     g_na_ready[dev] = true;
   }
@@ -334,23 +420,35 @@ extern "C" int prx_react_noalloc(const prx_reaction_desc* rx, const double* box,
   a.R.rule = rx->selection;
   for (int t = 0; t < PRX_MAX_TYPES; ++t) a.R.maxval[t] = rx->max_valence[t];
   a.sc = sc;
+  // bound on the FP32 search's distances for coordinates within two box edges
+  // of the origin: 2^-23 of the value lost in each conversion, three roundings
+  // of at most 2 L each: below 2e-6 L per distance
+  const double Lmax = std::fmax(box[0], std::fmax(box[1], box[2]));
+  const double reach = rx->r_react * (1.0 + 1e-5) + 4e-6 * Lmax;
+  a.near2 = (float)(reach * reach * (1.0 + 1e-5));
+  for (int k = 0; k < 3; ++k) {
+    a.Lf[k] = (float)box[k];
+    a.invLf[k] = (float)(1.0 / box[k]);
+  }
 
   // counters and status start at zero on every call
-  if (cudaMemsetAsync(&sc->trace[0], 0, sizeof(sc->trace) + sizeof(sc->nbonds) + sizeof(sc->status),
-                      st) != cudaSuccess)
+  struct Result {
+    unsigned long long trace[4];
+    unsigned int nbonds;
+    int status;
+    unsigned int nlist;
+  } got;
+  if (cudaMemsetAsync(&sc->trace[0], 0, offsetof(Result, nlist) + sizeof(got.nlist), st) != cudaSuccess)
     return PRX_ECUDA;
-  const unsigned g = n ? (n + 255u) / 256u : 1u;
-  k_na_find<<<g, 256, 0, st>>>(a);
-  if (a.R.rule == PRX_SELECT_NEAREST) k_na_find_T<<<g, 256, 0, st>>>(a);
-  k_na_select<<<g, 256, 0, st>>>(a);
+  k_na_find<<<NA_BLOCKS, NA_THREADS, (size_t)n * (3 * sizeof(float) + sizeof(uint16_t)), st>>>(a);
+  k_na_select<<<NA_BLOCKS, 256, 0, st>>>(a);
   k_na_apply<<<1, 1024, 0, st>>>(a);
   if (cudaGetLastError() != cudaSuccess) return PRX_ECUDA;
-  unsigned long long tr[4];
-  int status = 0;
-  if (cudaMemcpyAsync(tr, &sc->trace[0], sizeof(tr), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-      cudaMemcpyAsync(&status, &sc->status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  if (cudaMemcpyAsync(&got, &sc->trace[0], sizeof(got), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return PRX_ECUDA;
+  const unsigned long long* tr = got.trace;
+  const int status = got.status;
   if (trace) {
     trace->candidates = (int64_t)tr[0];
     trace->retained = (int64_t)tr[1];
