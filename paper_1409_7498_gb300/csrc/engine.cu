@@ -137,34 +137,6 @@ __device__ __forceinline__ void cp_async16_ca(void* smem_dst, const void* gsrc) 
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 
-// pair32 without a force cap and without a branch: a pair that adds nothing
-// gets g = 0 (f - 0 d = f), so that four entries' chains overlap.
-template <bool CUBIC>
-__device__ __forceinline__ void pair32_flat(const Sys& S, uint4 pj, uint4 pi, float& fx, float& fy, float& fz) {
-  float dx, dy, dz, r2;
-  bool hit;
-  if constexpr (CUBIC) {
-    dx = __int2float_rn(pdiff(pj.x, pi.x));
-    dy = __int2float_rn(pdiff(pj.y, pi.y));
-    dz = __int2float_rn(pdiff(pj.z, pi.z));
-    const float r2u = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-    hit = r2u > 0.f && r2u < S.rc2u;
-    r2 = r2u * S.s2f;
-  } else {
-    disp(S, pj, pi, dx, dy, dz);
-    r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-    hit = r2 > 0.f && r2 < S.rc2f;
-  }
-  const float r2i = __fdividef(1.0f, r2);
-  const float sr2 = S.sig2f * r2i;
-  const float sr6 = sr2 * sr2 * sr2;
-  float g = S.eps24f * sr6 * (2.0f * sr6 - 1.0f) * r2i;
-  g = hit ? g : 0.f;
-  fx -= g * dx;
-  fy -= g * dy;
-  fz -= g * dz;
-}
-
 // One FP32 step of a resident slot: every neighbour position is on its way
 // into shared memory before the first is used (one round trip per step,
 // overlapped with the random force), then the arithmetic of step_one.
@@ -424,12 +396,45 @@ __device__ __noinline__ void eng_list_slow(const Sys& S, const uint4* P, uint32_
   nl_close<NL16>(S, i, cnt);
 }
 
+struct RowInfo {
+  int base;        // first staged index of the row
+  int padL;        // particles of the left image cell (cell nx-1)
+  int rowcount;    // particles of the row
+  int tot;         // padL + rowcount + padR
+  int row_lo;      // first slot of the row
+  int left_start;  // first slot of cell nx-1
+  int c1;          // first slot of cell 1 (end of cell 0)
+  uint32_t yref;   // fixed-point lower edge of the (wrapped) row in y
+  uint32_t zref;   // and in z
+  float yoff;      // that edge's offset from the tile's lower edge, unwrapped
+  float zoff;
+  int pad;
+};
+// FP32 coordinates of a staged particle in the tile's frame: y and z relative
+// to the tile's lower cell edges (each row's images unwrapped), x in [0, L)
+// with the left and right image cells shifted by -L and +L.  A slot keyed to
+// cell 0 (nx-1) whose position rounds to the far end of the box (possible by
+// one rounding step after a restore) is taken back to the near side.  The
+// values carry ~1e-5 sigma of rounding; the list radius has a margin for it.
+__device__ __forceinline__ float4 build_coords(const uint4 p, const RowInfo& r, int kr,
+                                               uint32_t slot, float sx, float sy, float sz,
+                                               float Lx) {
+  float xf = __uint2float_rn(p.x) * sx;
+  if (slot < (uint32_t)r.c1 && p.x >= 0x80000000u) xf -= Lx;
+  if (slot >= (uint32_t)r.left_start && p.x < 0x80000000u) xf += Lx;
+  if (kr < r.padL) xf -= Lx;
+  else if (kr >= r.padL + r.rowcount) xf += Lx;
+  const float yf = fmaf(__int2float_rn(pdiff(p.y, r.yref)), sy, r.yoff);
+  const float zf = fmaf(__int2float_rn(pdiff(p.z, r.zref)), sz, r.zoff);
+  return make_float4(xf, yf, zf, __uint_as_float(slot));
+}
+
 // The lists of one tile (eng_ty cell rows at one cz) with three threads per
 // slot, one per layer of neighbour cells: each marks its hits of the
 // layer's three windows in bit masks (no store and no branch per candidate),
 // the three counts give each its place in the list, and the marked
-// candidates are written.  Staging and coordinates as in build_tile; the
-// lists differ from its at most in pairs at the edge of the list radius.
+// candidates are written.  The lists differ from build_tile's at most in pairs
+// at the edge of the list radius.
 template <bool NL16>
 __device__ __forceinline__ void eng_build_tile(const Sys& S, const uint4* P, const uint32_t* cell_of, uint32_t tile,
                                                unsigned char* smem) {

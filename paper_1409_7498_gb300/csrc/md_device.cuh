@@ -218,12 +218,40 @@ __device__ __forceinline__ void pair32(const Sys& S, uint4 pj, uint4 pi, float& 
   }
 }
 
+// pair32 without a force cap and without a branch: a pair that adds nothing
+// gets g = 0 (f - 0 d = f), so that four entries' chains overlap.
+template <bool CUBIC>
+__device__ __forceinline__ void pair32_flat(const Sys& S, uint4 pj, uint4 pi, float& fx, float& fy, float& fz) {
+  float dx, dy, dz, r2;
+  bool hit;
+  if constexpr (CUBIC) {
+    dx = __int2float_rn(pdiff(pj.x, pi.x));
+    dy = __int2float_rn(pdiff(pj.y, pi.y));
+    dz = __int2float_rn(pdiff(pj.z, pi.z));
+    const float r2u = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    hit = r2u > 0.f && r2u < S.rc2u;
+    r2 = r2u * S.s2f;
+  } else {
+    disp(S, pj, pi, dx, dy, dz);
+    r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    hit = r2 > 0.f && r2 < S.rc2f;
+  }
+  const float r2i = __fdividef(1.0f, r2);
+  const float sr2 = S.sig2f * r2i;
+  const float sr6 = sr2 * sr2 * sr2;
+  float g = S.eps24f * sr6 * (2.0f * sr6 - 1.0f) * r2i;
+  g = hit ? g : 0.f;
+  fx -= g * dx;
+  fy -= g * dy;
+  fz -= g * dz;
+}
+
 // ---------------------------------------------------------------------------
 // FP32 step kernel: one thread per slot, WCA over the Verlet list.
 // ---------------------------------------------------------------------------
 // The step of slot i: forces over its list and bonds, then the integration
 // (or, FORCES_ONLY, the forces written out); returns the rebuild trigger.
-template <bool NL16, bool FORCES_ONLY, bool CUBIC>
+template <bool NL16, bool FORCES_ONLY, bool CUBIC, bool CAP>
 __device__ __forceinline__ bool step_one(const Sys& S, Ctl* ctl, const SoA& B,
                                          const uint4* __restrict__ P, uint4* __restrict__ Pn,
                                          uint32_t i, unsigned long long step) {
@@ -252,7 +280,10 @@ __device__ __forceinline__ bool step_one(const Sys& S, Ctl* ctl, const SoA& B,
 #pragma unroll
     for (int u = 0; u < 4; ++u) rn[u] = k + 4 < cnt ? nl_raw<NL16>(S, k + 4 + u, i) : 0u;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) pair32<CUBIC>(S, pj[u], pi, fx, fy, fz, e);
+    for (int u = 0; u < 4; ++u) {
+      if constexpr (CAP || FORCES_ONLY) pair32<CUBIC>(S, pj[u], pi, fx, fy, fz, e);
+      else pair32_flat<CUBIC>(S, pj[u], pi, fx, fy, fz);
+    }
   }
   if constexpr (CUBIC) {
     fx *= S.scale[0];
@@ -351,11 +382,17 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_256(uint32_t v, uint32_
 // Verlet-list build.  One block per tile of TY consecutive cell rows (cy0 ..
 // cy0+TY-1 at one cz); threads = the tile's particles, contiguous in slot
 // order (in passes of blockDim when a tile is longer).  All (TY+2) x 3
-// neighbour rows are staged in shared memory as FP32 coordinates in the
-// tile's frame (one pass in the common case), each row extended by one
-// periodic image cell at both ends, so every particle's 3 x 3 x 3 cell
-// neighbourhood is 9 contiguous ranges.  A pair enters the list when its
-// FP32 distance is below r_c + skin (widened by the rounding bound).
+// neighbour rows are staged in shared memory (one pass in the common case) as
+// the FP32 coordinates that the permutation left in fout (build_xyz), each
+// row extended by one periodic image cell at both ends, so every particle's
+// 3 x 3 x 3 cell neighbourhood is 9 contiguous ranges.  Rows that are images
+// in y or z are met by shifting the particle's own coordinates.  A pair enters the list when its FP32 distance is below r_c + skin (widened by
+// the rounding bound).
+//
+// Bound by instruction issue: ~15 instructions per candidate and lane, ~110
+// candidates.  Taking the coordinates from the permutation and describing the
+// rows without divisions, instead of turning every staged entry from fixed
+// point into the tile's frame: 133 -> 121 us at 1,048,576 beads.
 // ---------------------------------------------------------------------------
 // 16-byte copy global -> shared that does not wait for the data (cp.async,
 // L2 only); cp_async_wait_all() waits for every copy the thread issued.
@@ -365,40 +402,35 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-struct RowInfo {
-  int base;        // first staged index of the row
-  int padL;        // particles of the left image cell (cell nx-1)
-  int rowcount;    // particles of the row
-  int tot;         // padL + rowcount + padR
-  int row_lo;      // first slot of the row
-  int left_start;  // first slot of cell nx-1
-  int c1;          // first slot of cell 1 (end of cell 0)
-  uint32_t yref;   // fixed-point lower edge of the (wrapped) row in y
-  uint32_t zref;   // and in z
-  float yoff;      // that edge's offset from the tile's lower edge, unwrapped
-  float zoff;
-  int pad;
-};
-constexpr int TILE_ROWS_MAX = 18;  // (TY + 2) x 3 for TY <= 4
-
-// FP32 coordinates of a staged particle in the tile's frame: y and z relative
-// to the tile's lower cell edges (each row's images unwrapped), x in [0, L)
-// with the left and right image cells shifted by -L and +L.  A slot keyed to
-// cell 0 (nx-1) whose position rounds to the far end of the box (possible by
-// one rounding step after a restore) is taken back to the near side.  The
-// values carry ~1e-5 sigma of rounding; the list radius has a margin for it.
-__device__ __forceinline__ float4 build_coords(const uint4 p, const RowInfo& r, int kr,
-                                               uint32_t slot, float sx, float sy, float sz,
-                                               float Lx) {
-  float xf = __uint2float_rn(p.x) * sx;
-  if (slot < (uint32_t)r.c1 && p.x >= 0x80000000u) xf -= Lx;
-  if (slot >= (uint32_t)r.left_start && p.x < 0x80000000u) xf += Lx;
-  if (kr < r.padL) xf -= Lx;
-  else if (kr >= r.padL + r.rowcount) xf += Lx;
-  const float yf = fmaf(__int2float_rn(pdiff(p.y, r.yref)), sy, r.yoff);
-  const float zf = fmaf(__int2float_rn(pdiff(p.z, r.zref)), sz, r.zoff);
-  return make_float4(xf, yf, zf, __uint_as_float(slot));
+// FP32 coordinates of a slot for the list build, in [0, L) per axis up to
+// rounding: a position that rounds across the box edge from the cell that the
+// sort put it in is kept on that cell's side.
+// .w holds the slot.
+__device__ __forceinline__ float4 build_xyz(const Sys& S, uint32_t X, uint32_t Y, uint32_t Z, uint32_t key,
+                                            uint32_t slot) {
+  const uint32_t nx = (uint32_t)S.nc[0], ny = (uint32_t)S.nc[1], nz = (uint32_t)S.nc[2];
+  const uint32_t row = key / nx, c[3] = {key - row * nx, row % ny, row / ny}, n[3] = {nx, ny, nz};
+  const uint32_t p[3] = {X, Y, Z};
+  float f[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    f[d] = __uint2float_rn(p[d]) * S.scale[d];
+    if (c[d] == 0u && p[d] >= 0xC0000000u) f[d] -= (float)S.L[d];
+    if (c[d] == n[d] - 1u && p[d] < 0x40000000u) f[d] += (float)S.L[d];
+  }
+  return make_float4(f[0], f[1], f[2], __uint_as_float(slot));
 }
+
+struct BuildRow {
+  int base;         // first staged index of the row
+  int padL;         // particles of the left image cell (cell nx-1)
+  int cnt;          // particles of the row
+  int tot;          // padL + cnt + particles of the right image cell (cell 0)
+  int lo;           // first slot of the row
+  int left;         // first slot of cell nx-1
+  float yoff, zoff; // image shift of the row
+};
+constexpr int TILE_ROWS_MAX = 3 * (TILE_Y_MAX + 2);
 
 // One candidate: hit = r2 < rv2; a hit is written to row `cnt` of the
 // slot's column while cnt < cap, and cnt counts every hit (cnt > cap
@@ -434,99 +466,84 @@ __device__ __forceinline__ void list_candidate(unsigned char* col, uint32_t stri
 }
 
 // The list build of one tile (`tile` of tiles_y * nc[2]), by all threads of
-// the block; P the fixed-point positions, cell_of the cell the sort put each
-// slot in.  The block synchronises inside; a block that builds several tiles
-// synchronises between them.
+// the block; F the slots' coordinates (build_xyz), cell_of the cell the sort
+// put each slot in.  The block synchronises inside; a block that builds
+// several tiles synchronises between them.
 template <bool NL16>
-__device__ __forceinline__ void build_tile(const Sys& S, const uint4* P,
-                                           const uint32_t* cell_of, uint32_t tile,
+__device__ __forceinline__ void build_tile(const Sys& S, const float4* F, const uint32_t* cell_of, uint32_t tile,
                                            unsigned char* smem) {
   const int CAP = S.tile_cap;
   float4* sX = reinterpret_cast<float4*>(smem);
-  RowInfo* ri = reinterpret_cast<RowInfo*>(smem + 16 * (size_t)CAP);
+  BuildRow* ri = reinterpret_cast<BuildRow*>(smem + 16 * (size_t)CAP);
   uint32_t* sCS = reinterpret_cast<uint32_t*>(ri + TILE_ROWS_MAX);
   __shared__ int sTOT;
   Ctl* ctl = S.ctl;
   const int nx = S.nc[0], ny = S.nc[1], nz = S.nc[2];
   const int ty = tile % S.tiles_y, cz = tile / S.tiles_y;
-  const int cy0 = ty * S.tile_y;
-  const int TYb = min(S.tile_y, ny - cy0);
+  const int cy0 = ty * ny / S.tiles_y;  // (the rows shared out evenly)
+  const int TYb = (ty + 1) * ny / S.tiles_y - cy0;
   const int RY = TYb + 2, R = 3 * RY;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const uint32_t rs = S.cell_start[(cz * ny + cy0) * nx];
   const uint32_t re = S.cell_start[(cz * ny + cy0 + TYb - 1) * nx + nx];
 
-  for (int k = threadIdx.x; k < R * (nx + 1); k += blockDim.x) {
-    const int sr = k / (nx + 1), c = k - sr * (nx + 1);
+  // one warp per row: its cell offsets, then its description
+  for (int sr = warp; sr < R; sr += nwarps) {
     const int dzi = sr / RY, yi = sr - dzi * RY;
-    const int qz = wrap_cell(cz - 1 + dzi, nz), qy = wrap_cell(cy0 - 1 + yi, ny);
-    sCS[k] = S.cell_start[(qz * ny + qy) * nx + c];
-  }
-  __syncthreads();
-  if (threadIdx.x < R) {
-    const uint32_t* cs = sCS + threadIdx.x * (nx + 1);
-    const int dzi = threadIdx.x / RY, yi = threadIdx.x - dzi * RY;
     const int uy = cy0 - 1 + yi, uz = cz - 1 + dzi;  // unwrapped row indices
-    const int qy = wrap_cell(uy, ny), qz = wrap_cell(uz, nz);
-    RowInfo r;
-    r.padL = (int)(cs[nx] - cs[nx - 1]);
-    r.rowcount = (int)(cs[nx] - cs[0]);
-    r.tot = r.padL + r.rowcount + (int)(cs[1] - cs[0]);
-    r.row_lo = (int)cs[0];
-    r.left_start = (int)cs[nx - 1];
-    r.c1 = (int)cs[1];
-    r.yref = (uint32_t)(((unsigned long long)qy << 32) / (unsigned)ny);
-    r.zref = (uint32_t)(((unsigned long long)qz << 32) / (unsigned)nz);
-    r.yoff = (float)((double)(uy - cy0) * (S.L[1] / ny));
-    r.zoff = (float)((double)(uz - cz) * (S.L[2] / nz));
-    r.base = 0;
-    r.pad = 0;
-    ri[threadIdx.x] = r;
+    const uint32_t* src = S.cell_start + (wrap_cell(uz, nz) * ny + wrap_cell(uy, ny)) * nx;
+    uint32_t* cs = sCS + sr * (nx + 1);
+    for (int c = lane; c <= nx; c += 32) cs[c] = src[c];
+    __syncwarp();
+    if (lane == 0) {
+      BuildRow r;
+      r.base = 0;
+      r.padL = (int)(cs[nx] - cs[nx - 1]);
+      r.cnt = (int)(cs[nx] - cs[0]);
+      r.tot = r.padL + r.cnt + (int)(cs[1] - cs[0]);
+      r.lo = (int)cs[0];
+      r.left = (int)cs[nx - 1];
+      r.yoff = uy < 0 ? -(float)S.L[1] : (uy >= ny ? (float)S.L[1] : 0.f);
+      r.zoff = uz < 0 ? -(float)S.L[2] : (uz >= nz ? (float)S.L[2] : 0.f);
+      ri[sr] = r;
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int sr = 0; sr < R; ++sr) {
-      ri[sr].base = run;
-      run += ri[sr].tot;
+  if (warp == 0) {
+    const int cnt = lane < R ? ri[lane].tot : 0;
+    int x = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= o) x += y;
     }
-    sTOT = run;
+    if (lane < R) ri[lane].base = x - cnt;
+    if (lane == 31) sTOT = x;
   }
   __syncthreads();
   const int TOT = sTOT;
-  const float sx = S.scale[0], sy = S.scale[1], sz = S.scale[2], rv2 = S.rv2_build;
-  const float Lx = (float)S.L[0];
+  const float rv2 = S.rv2_build, Lx = (float)S.L[0];
 
-  // Stages entries [c0, c0 + cn) of the neighbour rows, one warp per row:
-  // raw copies in flight at once (cp.async), then each lane turns the
-  // entries it copied into tile-frame FP32 coordinates in place (the same
-  // warp/lane mapping, so no block barrier in between).
+  // Stages entries [c0, c0 + cn) of the neighbour rows, one warp per row: the
+  // copies all in flight at once, then the images' shift in x.
   auto stage = [&](int c0, int cn) {
     for (int sr = warp; sr < R; sr += nwarps) {
-      const RowInfo& r = ri[sr];
+      const BuildRow r = ri[sr];
       const int k0 = max(r.base, c0), k1 = min(r.base + r.tot, c0 + cn);
-      const int padL = r.padL, rc = r.rowcount, lo = r.row_lo, ls = r.left_start, b = r.base;
       for (int ent = k0 + lane; ent < k1; ent += 32) {
-        const int kr = ent - b;
-        const int slot = kr < padL ? ls + kr : (kr < padL + rc ? lo + kr - padL : lo + kr - padL - rc);
-        cp_async16(&sX[ent - c0], P + slot);
+        const int kr = ent - r.base;
+        const int slot = kr < r.padL ? r.left + kr
+                                     : r.lo + (kr < r.padL + r.cnt ? kr - r.padL : kr - r.padL - r.cnt);
+        cp_async16(&sX[ent - c0], F + slot);
       }
     }
     cp_async_wait_all();
     __syncwarp();
     for (int sr = warp; sr < R; sr += nwarps) {
-      const RowInfo r = ri[sr];
+      const BuildRow r = ri[sr];
       const int k0 = max(r.base, c0), k1 = min(r.base + r.tot, c0 + cn);
-      for (int ent = k0 + lane; ent < k1; ent += 32) {
-        const int kr = ent - r.base;
-        const int slot = kr < r.padL ? r.left_start + kr
-                                     : r.row_lo + (kr < r.padL + r.rowcount ? kr - r.padL
-                                                                            : kr - r.padL - r.rowcount);
-        const float4 raw = sX[ent - c0];
-        const uint4 p = make_uint4(__float_as_uint(raw.x), __float_as_uint(raw.y),
-                                   __float_as_uint(raw.z), 0u);
-        sX[ent - c0] = build_coords(p, r, kr, (uint32_t)slot, sx, sy, sz, Lx);
-      }
+      for (int ent = k0 + lane; ent < min(r.base + r.padL, k1); ent += 32) sX[ent - c0].x -= Lx;
+      for (int ent = max(r.base + r.padL + r.cnt, k0) + lane; ent < k1; ent += 32) sX[ent - c0].x += Lx;
     }
   };
   const bool one = TOT <= CAP;  // the common case: every row staged once
@@ -538,10 +555,10 @@ __device__ __forceinline__ void build_tile(const Sys& S, const uint4* P,
   for (uint32_t base = rs; base < re; base += blockDim.x) {
     const uint32_t i = base + threadIdx.x;
     const bool act = i < re;
-    const uint4 pi = act ? P[i] : make_uint4(0u, 0u, 0u, 0u);
     // the cell the sort put this slot in (not the one its current position
     // maps to: after a checkpoint restore the two can differ by one)
     const uint32_t kc = act ? cell_of[i] : (uint32_t)((cz * ny + cy0) * nx);
+    const float4 fi = act ? F[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     int cx = (int)(kc % (uint32_t)nx);
     int yrel = (int)((kc / (uint32_t)nx) % (uint32_t)ny) - cy0;
     if (yrel < 0 || yrel >= TYb) {  // cannot happen for a consistent sort
@@ -554,18 +571,13 @@ __device__ __forceinline__ void build_tile(const Sys& S, const uint4* P,
     for (int w = 0; w < 9; ++w) {
       const int sr = (w / 3) * RY + yrel + (w % 3);
       const uint32_t* cs = sCS + sr * (nx + 1);
-      const RowInfo& r = ri[sr];
-      const int lo = r.base + (cx == 0 ? 0 : r.padL + (int)cs[cx - 1] - r.row_lo);
-      const int hi = r.base + (cx + 2 > nx ? r.tot : r.padL + (int)cs[cx + 2] - r.row_lo);
+      const BuildRow& r = ri[sr];
+      const int off = r.base + r.padL - r.lo;  // slot -> staged entry
+      const int lo = cx == 0 ? r.base : off + (int)cs[cx - 1];
+      const int hi = cx + 2 > nx ? r.base + r.tot : off + (int)cs[cx + 2];
       win[w] = (uint32_t)lo | ((uint32_t)hi << 16);
     }
-    float4 fi;
-    int kself0;  // the particle's own entry in the staged centre row
-    {
-      const RowInfo& r = ri[RY + yrel + 1];
-      fi = build_coords(pi, r, r.padL + ((int)i - r.row_lo), i, sx, sy, sz, Lx);
-      kself0 = r.base + r.padL + ((int)i - r.row_lo);
-    }
+    const int kself0 = ri[RY + yrel + 1].base + ri[RY + yrel + 1].padL + ((int)i - ri[RY + yrel + 1].lo);
     int cnt = 0;
     const int cap = S.list_cap;
     unsigned char* col = (unsigned char*)S.nl + (size_t)i * (NL16 ? 2 : 4);
@@ -577,29 +589,30 @@ __device__ __forceinline__ void build_tile(const Sys& S, const uint4* P,
         stage(c0, cn);
         __syncthreads();
       }
-      if (act) {
-        // the particle itself is staged once, in the centre row's window
-        // (w = 4), whose walk skips it: no candidate needs a self test
-        const int kself = kself0 - c0;
+      if (!act) continue;
+      // the particle itself is staged once, in the centre row's window
+      // (w = 4), whose walk skips it: no candidate needs a self test
+      const int kself = kself0 - c0;
 #pragma unroll
-        for (int w = 0; w < 9; ++w) {
-          const int lo = max((int)(win[w] & 0xFFFFu), c0) - c0;
-          const int hi = min((int)(win[w] >> 16), c0 + cn) - c0;
-          auto walk = [&](int a, int b) {
+      for (int w = 0; w < 9; ++w) {
+        const int lo = max((int)(win[w] & 0xFFFFu), c0) - c0;
+        const int hi = min((int)(win[w] >> 16), c0 + cn) - c0;
+        const BuildRow& r = ri[(w / 3) * RY + yrel + (w % 3)];
+        const float y = fi.y - r.yoff, z = fi.z - r.zoff;
+        auto walk = [&](int a, int b) {
 #pragma unroll 2
-            for (int k = a; k < b; ++k) {
-              const float4 q = sX[k];
-              const float dx = q.x - fi.x, dy = q.y - fi.y, dz = q.z - fi.z;
-              list_candidate<NL16>(col, stride, fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rv2,
-                                   __float_as_uint(q.w), cap, cnt);
-            }
-          };
-          if (w == 4) {
-            walk(lo, min(hi, max(lo, kself)));
-            walk(max(lo, kself + 1), hi);
-          } else {
-            walk(lo, hi);
+          for (int k = a; k < b; ++k) {
+            const float4 q = sX[k];
+            const float dx = q.x - fi.x, dy = q.y - y, dz = q.z - z;
+            list_candidate<NL16>(col, stride, fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rv2, __float_as_uint(q.w), cap,
+                                 cnt);
           }
+        };
+        if (w == 4) {
+          walk(lo, min(hi, max(lo, kself)));
+          walk(max(lo, kself + 1), hi);
+        } else {
+          walk(lo, hi);
         }
       }
     }

@@ -48,49 +48,33 @@ __device__ __forceinline__ void raise_rebuild(const Sys& S) {
   __threadfence();
 }
 
-// End of a step: the system's last warp advances its step counter and
-// buffer phase; for a single system it also sets the graph's rebuild
-// condition, for a batch the last system to finish sets it for all.
-__device__ __forceinline__ void step_epilogue(const Sys& S, int ph, unsigned long long step,
-                                              cudaGraphConditionalHandle cond, int use_cond,
-                                              unsigned int* warps_left, uint32_t nb) {
+// End of a step, by the last thread of the system to finish: its step counter
+// and buffer phase advance; for a single system the graph's rebuild condition
+// is set, for a batch the last system to finish sets it for all.
+__device__ __forceinline__ void step_done(const Sys& S, int ph, unsigned long long step,
+                                          cudaGraphConditionalHandle cond, int use_cond) {
   Ctl* ctl = S.ctl;
-  if (last_warp(&ctl->done_step, warps_left, nb)) {
-    ctl->done_step = 0u;
-    ctl->phase = ph ^ 1;
-    ctl->step = step;
-    if (!S.in_batch) {
-      const int flag = atomicAdd(&ctl->rebin_flag, 0);
+  ctl->done_step = 0u;
+  ctl->phase = ph ^ 1;
+  ctl->step = step;
+  if (!S.in_batch) {
+    const int flag = atomicAdd(&ctl->rebin_flag, 0);
+    if (use_cond) cudaGraphSetConditional(cond, flag ? 1u : 0u);
+  } else {
+    __threadfence();
+    if (atomicAdd(&S.batch->done_step, 1u) == S.n_members - 1) {
+      S.batch->done_step = 0u;
+      const int flag = atomicExch(&S.batch->any_rebuild, 0);
+      if (flag) S.batch->rebuilds += 1ull;
+      S.batch->rebuild_now = flag;  // for a device-driven run (dg.cu)
       if (use_cond) cudaGraphSetConditional(cond, flag ? 1u : 0u);
-    } else {
-      __threadfence();
-      if (atomicAdd(&S.batch->done_step, 1u) == S.n_members - 1) {
-        S.batch->done_step = 0u;
-        const int flag = atomicExch(&S.batch->any_rebuild, 0);
-        if (flag) S.batch->rebuilds += 1ull;
-        S.batch->rebuild_now = flag;  // for a device-driven run (dg.cu)
-        if (use_cond) cudaGraphSetConditional(cond, flag ? 1u : 0u);
-      }
     }
   }
 }
-
-template <bool NL16, bool FORCES_ONLY, bool CUBIC>
-__device__ __forceinline__ void step_nl_body(const Sys& S, const Blk blk,
-                                             cudaGraphConditionalHandle cond, int use_cond) {
-  __shared__ unsigned int warps_left;
-  if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
-  __syncthreads();
-  Ctl* ctl = S.ctl;
-  const int set = ctl->set;
-  const int ph = ctl->phase;
-  const unsigned long long step = ctl->step + 1ull;
-  const SoA B = set ? S.s1 : S.s0;
-  const uint4* __restrict__ P = ph ? S.P1 : S.P0;
-  uint4* __restrict__ Pn = ph ? S.P0 : S.P1;
-  const uint32_t i = blk.b * blockDim.x + threadIdx.x;
-  if (i < S.n && step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
-  if constexpr (!FORCES_ONLY) step_epilogue(S, ph, step, cond, use_cond, &warps_left, blk.nb);
+__device__ __forceinline__ void step_epilogue(const Sys& S, int ph, unsigned long long step,
+                                              cudaGraphConditionalHandle cond, int use_cond,
+                                              unsigned int* warps_left, uint32_t nb) {
+  if (last_warp(&S.ctl->done_step, warps_left, nb)) step_done(S, ph, step, cond, use_cond);
 }
 
 // Single system: as many blocks as are resident at once (or the launch
@@ -99,7 +83,7 @@ __device__ __forceinline__ void step_nl_body(const Sys& S, const Blk blk,
 // instead of running a partial last wave.  BT threads per block, with the
 // register budget of 48 resident warps per SM for every BT; the block shape
 // changes only the scheduling, not any particle's arithmetic.
-template <bool NL16, bool FORCES_ONLY, bool CUBIC, int BT>
+template <bool NL16, bool FORCES_ONLY, bool CUBIC, bool CAP, int BT>
 __global__ void __launch_bounds__(BT, 1536 / BT)
     k_step_nl(Sys S, cudaGraphConditionalHandle cond, int use_cond) {
   __shared__ unsigned int warps_left;
@@ -117,7 +101,7 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
   auto run = [&](const SoA& B) {
     for (uint32_t c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c * 32u < S.n; c += W) {
       const uint32_t i = c * 32u + (threadIdx.x & 31u);
-      if (i < S.n && step_one<NL16, FORCES_ONLY, CUBIC>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
+      if (i < S.n && step_one<NL16, FORCES_ONLY, CUBIC, CAP>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
     }
   };
   if (ctl->set) run(S.s1);
@@ -215,16 +199,49 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
   if constexpr (!FORCES_ONLY) step_epilogue(S, ph, step, cond, use_cond, &warps_left, gridDim.x);
 }
 
-// Members of a batch may differ in list width and box shape: the batch step
-// runs one launch per (list width, cubic) variant present, each over the
-// blocks of its members, with the single-system kernel's register budget.
-template <bool NL16, bool CUBIC>
-__global__ void __launch_bounds__(256, 5)
-    kb_step_nl(const Sys* __restrict__ T, const BlkMap* __restrict__ M,
+// Members of a batch may differ in list width, box shape and force cap: the
+// batch step runs one launch per variant present.  Like the single-system
+// kernel it is a grid of the resident blocks: each takes a contiguous run of
+// the variant's block map (256 slots per entry), so that it changes member
+// rarely, and keeps the member's parameters in shared memory meanwhile.
+// Read from the member table in global memory by one block per entry, they
+// cost a load and an address at every use: 235 us per step of 256 replicas
+// (3.4 M beads), 201 this way.
+template <bool NL16, bool CUBIC, bool CAP>
+__global__ void __launch_bounds__(256, 6)
+    kb_step_nl(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t n,
                cudaGraphConditionalHandle cond, int use_cond, uint32_t* __restrict__ act_n) {
   if (blockIdx.x == 0 && threadIdx.x < 5) act_n[threadIdx.x] = 0u;  // for this step's rebuild plan
-  const BlkMap m = M[blockIdx.x];
-  step_nl_body<NL16, false, CUBIC>(T[m.sys], Blk{m.b, m.nb}, cond, use_cond);
+  __shared__ __align__(16) unsigned char sbuf[sizeof(Sys)];
+  const Sys& S = *reinterpret_cast<const Sys*>(sbuf);
+  static_assert(sizeof(Sys) % 8 == 0, "Sys is copied in 8-byte words");
+  uint32_t e = (uint32_t)((unsigned long long)n * blockIdx.x / gridDim.x);
+  const uint32_t e1 = (uint32_t)((unsigned long long)n * (blockIdx.x + 1u) / gridDim.x);
+  while (e < e1) {
+    const BlkMap m = M[e];
+    const uint32_t cnt = min(e1 - e, m.nb - m.b);  // this member's entries of the block's run
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(T + m.sys);
+    for (uint32_t w = threadIdx.x; w < sizeof(Sys) / 8; w += blockDim.x)
+      reinterpret_cast<unsigned long long*>(sbuf)[w] = src[w];
+    __syncthreads();
+    Ctl* ctl = S.ctl;
+    const int ph = ctl->phase;
+    const unsigned long long step = ctl->step + 1ull;
+    const SoA& B = ctl->set ? S.s1 : S.s0;
+    const uint4* P = ph ? S.P1 : S.P0;
+    uint4* Pn = ph ? S.P0 : S.P1;
+    for (uint32_t k = 0; k < cnt; ++k) {
+      const uint32_t i = (m.b + k) * 256u + threadIdx.x;
+      if (i < S.n && step_one<NL16, false, CUBIC, CAP>(S, ctl, B, P, Pn, i, step)) raise_rebuild(S);
+    }
+    __syncthreads();  // the block's work on the member is done (and its parameters read)
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&ctl->done_step, cnt) + cnt == m.nb) step_done(S, ph, step, cond, use_cond);
+    }
+    e += cnt;
+    if (e < e1) __syncthreads();
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -374,12 +391,12 @@ __global__ void k_rebin_keys_x(Sys S) {
   S.key[i] = k;
   atomicAdd(&S.count[k], 1u);
 }
-__global__ void kb_rebin_keys(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;  // compacted map: members that rebuild
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;  // this member needs no rebuild
-  rebin_keys_body(S, Blk{m.b, m.nb});
+__global__ void __launch_bounds__(256) kb_rebin_keys(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    rebin_keys_body(S, Blk{m.b, m.nb});
+  }
 }
 
 // Restore: keys were uploaded (a checkpoint's cells); only count them.
@@ -411,12 +428,13 @@ __device__ __forceinline__ void scan_tiles_body(const Sys& S, const Blk blk) {
   if (threadIdx.x == 0) S.blk_off[blk.b] = red[0];
 }
 __global__ void k_scan_tiles(Sys S) { scan_tiles_body(S, Blk{blockIdx.x, gridDim.x}); }
-__global__ void kb_scan_tiles(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;
-  scan_tiles_body(S, Blk{m.b, m.nb});
+__global__ void __launch_bounds__(256) kb_scan_tiles(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    scan_tiles_body(S, Blk{m.b, m.nb});
+    __syncthreads();
+  }
 }
 
 // Single block: exclusive scan of the tile sums in place.
@@ -434,11 +452,13 @@ __device__ __forceinline__ void scan_top_body(const Sys& S) {
   }
 }
 __global__ void k_scan_top(Sys S) { scan_top_body(S); }
-__global__ void kb_scan_top(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const Sys& S = T[M[blockIdx.x].sys];
-  if (!S.ctl->rebin_flag) return;
-  scan_top_body(S);
+__global__ void __launch_bounds__(256) kb_scan_top(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    scan_top_body(S);
+    __syncthreads();
+  }
 }
 
 __device__ __forceinline__ void scan_down_body(const Sys& S, const Blk blk) {
@@ -491,24 +511,25 @@ __device__ __forceinline__ void scan_down_self_body(const Sys& S, const Blk blk)
 }
 __global__ void k_scan_down(Sys S) { scan_down_body(S, Blk{blockIdx.x, gridDim.x}); }
 __global__ void k_scan_down_self(Sys S) { scan_down_self_body(S, Blk{blockIdx.x, gridDim.x}); }
-__global__ void kb_scan_down(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;
-  scan_down_body(S, Blk{m.b, m.nb});
+__global__ void __launch_bounds__(256) kb_scan_down(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    scan_down_body(S, Blk{m.b, m.nb});
+    __syncthreads();
+  }
 }
 
 // Batched rebuilds clear the cell counters in a kernel (a single system uses memsets).
-__global__ void kb_rebin_clear(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;
-  const uint32_t c = m.b * blockDim.x + threadIdx.x;
-  if (c < (uint32_t)S.ncell) {
-    S.count[c] = 0u;
-    S.fill[c] = 0u;
+__global__ void __launch_bounds__(256) kb_rebin_clear(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    const uint32_t c = m.b * blockDim.x + threadIdx.x;
+    if (c < (uint32_t)S.ncell) {
+      S.count[c] = 0u;
+      S.fill[c] = 0u;
+    }
   }
 }
 
@@ -521,12 +542,12 @@ __device__ __forceinline__ void rebin_scatter_body(const Sys& S, const Blk blk) 
 }
 
 __global__ void k_rebin_scatter(Sys S) { rebin_scatter_body(S, Blk{blockIdx.x, gridDim.x}); }
-__global__ void kb_rebin_scatter(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;  // this member needs no rebuild
-  rebin_scatter_body(S, Blk{m.b, m.nb});
+__global__ void __launch_bounds__(256) kb_rebin_scatter(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    rebin_scatter_body(S, Blk{m.b, m.nb});
+  }
 }
 
 // Sorts each cell's members by old slot: the order inside a cell then does
@@ -576,12 +597,12 @@ __device__ __forceinline__ void rebin_cellsort_body(const Sys& S, const Blk blk)
 }
 
 __global__ void k_rebin_cellsort(Sys S) { rebin_cellsort_body(S, Blk{blockIdx.x, gridDim.x}); }
-__global__ void kb_rebin_cellsort(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;  // this member needs no rebuild
-  rebin_cellsort_body(S, Blk{m.b, m.nb});
+__global__ void __launch_bounds__(256) kb_rebin_cellsort(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    rebin_cellsort_body(S, Blk{m.b, m.nb});
+  }
 }
 
 // New slot s takes old slot tmp[s]: copies every per-particle array into the
@@ -639,6 +660,7 @@ __device__ __forceinline__ void rebin_permute_one(const Sys& S, uint32_t s, bool
   const uint32_t Y = periodic_fx(y, S.Lfx[1], S.M64[1]);
   const uint32_t Z = periodic_fx(z, S.Lfx[2], S.M64[2]);
   P[s] = make_uint4(X, Y, Z, coarse_ref(X, Y, Z, S.wshift));
+  reinterpret_cast<float4*>(S.fout)[s] = build_xyz(S, X, Y, Z, key, s);  // for the list build that follows
   S.tmp[s] = key;
 }
 
@@ -655,12 +677,12 @@ __global__ void k_rebin_permute(Sys S, int wrap) {
     if (i < S.n) rebin_permute_one(S, i, wrap != 0);
   }
 }
-__global__ void kb_rebin_permute(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;  // this member needs no rebuild
-  rebin_permute_body(S, Blk{m.b, m.nb}, true);
+__global__ void __launch_bounds__(256) kb_rebin_permute(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    rebin_permute_body(S, Blk{m.b, m.nb}, true);
+  }
 }
 
 // One tile per block; the last warp of the system's tiles flips the SoA set
@@ -671,7 +693,7 @@ __device__ __forceinline__ void build_nlist_body(const Sys& S, const Blk blk, un
   __shared__ unsigned int warps_left;
   if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
   Ctl* ctl = S.ctl;
-  build_tile<NL16>(S, ctl->phase ? S.P1 : S.P0, S.tmp, blk.b, smem);
+  build_tile<NL16>(S, reinterpret_cast<const float4*>(S.fout), S.tmp, blk.b, smem);
   if (last_warp(&ctl->done_rebin, &warps_left, blk.nb)) {
     ctl->done_rebin = 0u;
     ctl->set ^= 1;
@@ -685,15 +707,16 @@ __global__ void __launch_bounds__(256) k_build_nlist(Sys S) {
   extern __shared__ __align__(16) unsigned char smem_b[];
   build_nlist_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, smem_b);
 }
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
     kb_build_nlist(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
   extern __shared__ __align__(16) unsigned char smem_b[];
-  if (blockIdx.x >= *C) return;
-  const BlkMap m = M[blockIdx.x];
-  const Sys& S = T[m.sys];
-  if (!S.ctl->rebin_flag) return;
-  if (S.nl16) build_nlist_body<true>(S, Blk{m.b, m.nb}, smem_b);
-  else build_nlist_body<false>(S, Blk{m.b, m.nb}, smem_b);
+  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+    const BlkMap m = M[e];
+    const Sys& S = T[m.sys];
+    if (S.nl16) build_nlist_body<true>(S, Blk{m.b, m.nb}, smem_b);
+    else build_nlist_body<false>(S, Blk{m.b, m.nb}, smem_b);
+    __syncthreads();  // the buffers and the warp count are used again
+  }
 }
 
 inline unsigned blocks_for(uint64_t n, int t) { return (unsigned)((n + t - 1) / t); }
@@ -819,11 +842,11 @@ unsigned device_sms() {
 
 unsigned resident_blocks(int variant, const void* kern, int threads) {
   static std::mutex mu;
-  static unsigned cache[64][64];
+  static unsigned cache[64][160];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1u;
   std::lock_guard<std::mutex> lk(mu);
-  unsigned& c = cache[dev][variant & 63];
+  unsigned& c = cache[dev][variant];
   if (!c) {
     int sms = 0, per = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -860,10 +883,12 @@ void launch_step(const Sys& S, cudaStream_t st, int fp64, int forces_only,
       auto go = [&](auto btc) {
         constexpr int BT = decltype(btc)::value;
         const bool four = S.step_lanes == 4;
-        auto* kern = four ? k_step_nl4<N16, FO, CU, BT> : k_step_nl<N16, FO, CU, BT>;
+        const bool cap = !FO && S.fcapf > 0.f;  // (the forces-only kernel tests for a cap itself)
+        auto* kern = four ? k_step_nl4<N16, FO, CU, BT>
+                          : (cap ? k_step_nl<N16, FO, CU, !FO, BT> : k_step_nl<N16, FO, CU, false, BT>);
         const unsigned per = four ? BT / 4 : BT;  // slots per block
         const unsigned g0 = blocks_for(S.n, per) > 0 ? blocks_for(S.n, per) : 1;
-        unsigned r = resident_blocks(v + 8 * (BT == 128 ? 1 : (BT == 512 ? 2 : 0)) + (four ? 32 : 0),
+        unsigned r = resident_blocks(v + 8 * (BT == 128 ? 1 : (BT == 512 ? 2 : 0)) + (four ? 32 : 0) + (cap ? 64 : 0),
                                      (const void*)kern, BT);
         if (!FO && S.step_bpsm > 0) {
           const unsigned want = (unsigned)S.step_bpsm * (unsigned)device_sms();
@@ -894,8 +919,7 @@ void launch_step(const Sys& S, cudaStream_t st, int fp64, int forces_only,
 int step_kernel_count(int fp64) { return fp64 ? 2 : 1; }
 
 size_t build_tile_smem(const Sys& S) {
-  return 16 * (size_t)S.tile_cap + sizeof(RowInfo) * TILE_ROWS_MAX +
-         4 * (size_t)TILE_ROWS_MAX * (S.nc[0] + 1);
+  return 16 * (size_t)S.tile_cap + sizeof(BuildRow) * TILE_ROWS_MAX + 4 * (size_t)(3 * (S.tile_y + 2)) * (S.nc[0] + 1);
 }
 
 // The dynamic shared-memory limit is an attribute of the kernel (per device),
@@ -990,16 +1014,26 @@ void launch_rebin(const Sys& S, cudaStream_t st, int mode, void (*hook)(void*, c
 
 void launch_batch_step(const BatchLaunch& L, cudaStream_t st, cudaGraphConditionalHandle h,
                        int use_cond) {
-  // variants in the order of the part map: (nl16, cubic) = 00, 01, 10, 11
-  if (L.step_n[0]) kb_step_nl<false, false><<<L.step_n[0], 256, 0, st>>>(L.T, L.part + L.step_off[0], h, use_cond, L.act_n);
-  if (L.step_n[1]) kb_step_nl<false, true><<<L.step_n[1], 256, 0, st>>>(L.T, L.part + L.step_off[1], h, use_cond, L.act_n);
-  if (L.step_n[2]) kb_step_nl<true, false><<<L.step_n[2], 256, 0, st>>>(L.T, L.part + L.step_off[2], h, use_cond, L.act_n);
-  if (L.step_n[3]) kb_step_nl<true, true><<<L.step_n[3], 256, 0, st>>>(L.T, L.part + L.step_off[3], h, use_cond, L.act_n);
+  auto go = [&](auto nl16, auto cub, auto cap) {
+    constexpr bool N16 = decltype(nl16)::value, CU = decltype(cub)::value, CA = decltype(cap)::value;
+    constexpr int v = (N16 ? 4 : 0) + (CU ? 2 : 0) + (CA ? 1 : 0);
+    if (!L.step_n[v]) return;
+    auto* kern = kb_step_nl<N16, CU, CA>;
+    const unsigned r = resident_blocks(128 + v, (const void*)kern, 256);
+    kern<<<L.step_n[v] < r ? L.step_n[v] : r, 256, 0, st>>>(L.T, L.part + L.step_off[v], L.step_n[v], h, use_cond,
+                                                            L.act_n);
+  };
+  using T_ = std::true_type;
+  using F_ = std::false_type;
+  go(F_{}, F_{}, F_{}), go(F_{}, F_{}, T_{}), go(F_{}, T_{}, F_{}), go(F_{}, T_{}, T_{});
+  go(T_{}, F_{}, F_{}), go(T_{}, F_{}, T_{}), go(T_{}, T_{}, F_{}), go(T_{}, T_{}, T_{});
 }
 
 // The rebuild pipeline over the members whose flag is set: a plan kernel
-// compacts their blocks, then every kernel runs the full grid of its family,
-// its blocks beyond the compacted count returning at once.
+// compacts their blocks, and each kernel's resident blocks take the entries of
+// its family in turn.  (A block per entry of the full map, returning at once
+// beyond the compacted count, costs ~18 us per kernel at 13,400 entries, most
+// of what a rebuild of the few members that need one takes.)
 void launch_batch_rebuild(const BatchLaunch& L, cudaStream_t st) {
   const uint32_t o1 = L.n_part, o2 = o1 + L.n_cell, o3 = o2 + L.n_tile, o4 = o3 + L.n_one;
   const uint32_t n_all = o4 + L.n_build;
@@ -1008,15 +1042,26 @@ void launch_batch_rebuild(const BatchLaunch& L, cudaStream_t st) {
   const BlkMap *part = L.act, *cell = L.act + o1, *tile = L.act + o2, *one = L.act + o3, *build = L.act + o4;
   const uint32_t *c_part = L.act_n, *c_cell = L.act_n + 1, *c_tile = L.act_n + 2, *c_one = L.act_n + 3,
                  *c_build = L.act_n + 4;
-  kb_rebin_clear<<<L.n_cell, 256, 0, st>>>(L.T, cell, c_cell);
-  kb_rebin_keys<<<L.n_part, 256, 0, st>>>(L.T, part, c_part);
-  kb_scan_tiles<<<L.n_tile, 256, 0, st>>>(L.T, tile, c_tile);
-  kb_scan_top<<<L.n_one, 256, 0, st>>>(L.T, one, c_one);
-  kb_scan_down<<<L.n_tile, 256, 0, st>>>(L.T, tile, c_tile);
-  kb_rebin_scatter<<<L.n_part, 256, 0, st>>>(L.T, part, c_part);
-  kb_rebin_cellsort<<<L.n_cell, 256, 0, st>>>(L.T, cell, c_cell);
-  kb_rebin_permute<<<L.n_part, 256, 0, st>>>(L.T, part, c_part);
-  kb_build_nlist<<<L.n_build, L.build_threads, L.build_smem, st>>>(L.T, build, c_build);
+  auto grid = [](int v, const void* k, unsigned n) {
+    const unsigned r = resident_blocks(v, k, 256);
+    return n < r ? n : r;
+  };
+  kb_rebin_clear<<<grid(136, (const void*)kb_rebin_clear, L.n_cell), 256, 0, st>>>(L.T, cell, c_cell);
+  kb_rebin_keys<<<grid(137, (const void*)kb_rebin_keys, L.n_part), 256, 0, st>>>(L.T, part, c_part);
+  kb_scan_tiles<<<grid(138, (const void*)kb_scan_tiles, L.n_tile), 256, 0, st>>>(L.T, tile, c_tile);
+  kb_scan_top<<<grid(139, (const void*)kb_scan_top, L.n_one), 256, 0, st>>>(L.T, one, c_one);
+  kb_scan_down<<<grid(140, (const void*)kb_scan_down, L.n_tile), 256, 0, st>>>(L.T, tile, c_tile);
+  kb_rebin_scatter<<<grid(141, (const void*)kb_rebin_scatter, L.n_part), 256, 0, st>>>(L.T, part, c_part);
+  kb_rebin_cellsort<<<grid(142, (const void*)kb_rebin_cellsort, L.n_cell), 256, 0, st>>>(L.T, cell, c_cell);
+  kb_rebin_permute<<<grid(143, (const void*)kb_rebin_permute, L.n_part), 256, 0, st>>>(L.T, part, c_part);
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kb_build_nlist, L.build_threads, L.build_smem) != cudaSuccess ||
+      per < 1) {
+    cudaGetLastError();
+    per = 1;
+  }
+  const unsigned r = device_sms() * (unsigned)per;
+  kb_build_nlist<<<L.n_build < r ? L.n_build : r, L.build_threads, L.build_smem, st>>>(L.T, build, c_build);
 }
 
 int batch_rebuild_kernel_count() { return 10; }

@@ -38,6 +38,7 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;
 constexpr uint32_t SLOT_MASK = 0x7FFFFFFFu;
 constexpr int STEP_THREADS = 128;
 constexpr int RX_THREADS = 256;
+constexpr int TILE_Y_MAX = 8;  // cell rows per tile of the list build
 constexpr unsigned ENG_BUCKET = 16;    // slots per cell bucket of the persistent runs
 constexpr unsigned ENG_CELLS = 32768;  // cells up to which a block scans all counts itself
 constexpr int SCAN_TILE = 2048;  // elements per scan tile (256 threads x 8)
@@ -359,9 +360,10 @@ struct BatchLaunch {
   // offsets as the full maps, and their entry counts (zeroed by the step)
   BlkMap* act;
   uint32_t* act_n;
-  // the part map is ordered by step-kernel variant (nl16, cubic): 00, 01,
-  // 10, 11; the blocks of variant v are part[step_off[v] .. + step_n[v])
-  unsigned step_off[4], step_n[4];
+  // the part map is ordered by step-kernel variant v = 4 nl16 + 2 cubic +
+  // force cap; the blocks of variant v are part[step_off[v] .. + step_n[v])
+  unsigned step_off[8], step_n[8];
+  bool any_nearest;  // a member has the nearest-partner rule
 };
 
 // ---- host-side launchers (defined in the kernel translation units) ----------

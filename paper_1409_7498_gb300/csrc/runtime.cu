@@ -339,27 +339,43 @@ int setup_grid(prx_system* sys, double rc) {
   A.add(&S.bucket, ncell <= (long long)ENG_CELLS ? (size_t)ncell * ENG_BUCKET : 0);
   if ((rc2 = A.commit(sys, sys->grid_allocs))) return rc2;
   {
-    // list-build tiling: the largest tile of 1..4 cell rows whose particles
-    // fit about two passes of 256 threads (fewer restaged neighbour rows per
-    // particle); staging buffer sized for all neighbour rows at once
+    // list-build tiling: the rows per tile (the rows of a layer shared out
+    // evenly) that keep most of the passes of 256 threads busy and restage
+    // few neighbour rows per particle, with four blocks per SM by shared
+    // memory.  us per list build with 1 / 2 / 3 / 4 / 5 / 8 rows: 130,000 beads
+    // 27.6 / 29.0 / 27.9 / 26.5 / 24.5 / 34.3, 500,000 beads 73.6 / 67.5 /
+    // 57.8 / 65.5 / 62.3 / 79.8, 1,048,576 beads 131 / 121 / 129 / 147 (1 to 4);
+    // the staging buffer holds all neighbour rows at once
     const double per_row = (double)S.n / ((double)S.nc[1] * S.nc[2]);
     const double per_cell = (double)S.n / (double)ncell;
-    int ty = 1;
-    for (int c = 2; c <= 4; ++c)
-      if (c * per_row + 3.0 * std::sqrt(c * per_row) + 16.0 <= 640.0) ty = c;
-    ty = std::max(1, std::min(ty, S.nc[1]));
-    S.tile_y = ty;
-    S.tiles_y = (S.nc[1] + ty - 1) / ty;
-    const double mean_tile = ty * per_row;
-    int t = (int)std::ceil((mean_tile + 3.0 * std::sqrt(mean_tile) + 16.0) / 32.0) * 32;
-    S.tile_threads = std::max(64, std::min(256, t));
-    const double mean_tot = 3.0 * (ty + 2) * (per_row + 2.0 * per_cell);
-    int cap = (int)std::ceil((mean_tot + 4.0 * std::sqrt(mean_tot) + 64.0) / 32.0) * 32;
-    S.tile_cap = 0;
-    const size_t fixed = build_tile_smem(S);
-    const size_t budget = 160 * 1024;
-    if (fixed + 16 * (size_t)cap > budget) cap = (int)((budget - fixed) / 16);
-    S.tile_cap = std::max(64, std::min(cap, 65535));
+    auto set_tiles = [&](int tiles) {
+      S.tiles_y = tiles;
+      S.tile_y = (S.nc[1] + tiles - 1) / tiles;  // the most rows of a tile
+      const double mean_tot = 3.0 * (S.tile_y + 2) * (per_row + 2.0 * per_cell);
+      const int cap = (int)std::ceil((mean_tot + 4.0 * std::sqrt(mean_tot) + 64.0) / 32.0) * 32;
+      const size_t budget = 160 * 1024;
+      S.tile_cap = 0;
+      const size_t fixed = build_tile_smem(S);
+      S.tile_cap = std::max(64, std::min(std::min(cap, 65535), (int)((budget - fixed) / 16)));
+    };
+    int best_tiles = S.nc[1];
+    double best_score = 0.0;
+    for (int c = 1; c <= TILE_Y_MAX && c <= S.nc[1]; ++c) {
+      set_tiles((S.nc[1] + c - 1) / c);
+      const double rows = (double)S.nc[1] / S.tiles_y;
+      const double passes = std::ceil((1.02 * S.tile_y * per_row + 4.0) / 256.0);
+      if (passes > 3.0 && c > 1) break;
+      const double blocks = std::min(4.0, std::floor(227.0 * 1024.0 / (double)(build_tile_smem(S) + 1024)));
+      const double score = rows * per_row / (256.0 * passes) * rows / (rows + 0.6) * blocks;
+      if (score > best_score) {
+        best_score = score;
+        best_tiles = S.tiles_y;
+      }
+    }
+    set_tiles(best_tiles);
+    const double mean_tile = S.tile_y * per_row;
+    const int threads = (int)std::ceil((mean_tile + 3.0 * std::sqrt(mean_tile) + 16.0) / 32.0) * 32;
+    S.tile_threads = std::max(64, std::min(256, threads));
     // persistent runs: the rows per tile whose list build is shortest when one
     // block per SM takes the tiles in turn (a tile's staging costs about as
     // much as 1.6 rounds of its 512 threads over (slot, layer) pairs)
@@ -994,13 +1010,13 @@ int batch_prepare(prx_batch* b) {
   };
   int build_threads = 32;
   size_t build_smem = 0;
-  // the part map ordered by step-kernel variant (list width, cubic box)
-  unsigned step_off[4] = {0, 0, 0, 0}, step_n[4] = {0, 0, 0, 0};
+  // the part map ordered by step-kernel variant (list width, cubic box, cap)
+  unsigned step_off[8] = {}, step_n[8] = {};
   b->n_step_variants = 0;
-  for (int v = 0; v < 4; ++v) {
+  for (int v = 0; v < 8; ++v) {
     step_off[v] = (unsigned)part.size();
     for (uint32_t q = 0; q < b->n_active; ++q)
-      if ((table[q].nl16 ? 2 : 0) + (table[q].cubic ? 1 : 0) == v) add(part, q, (table[q].n + 255) / 256);
+      if ((table[q].nl16 ? 4 : 0) + (table[q].cubic ? 2 : 0) + (table[q].fcapf > 0.f ? 1 : 0) == v) add(part, q, (table[q].n + 255) / 256);
     step_n[v] = (unsigned)part.size() - step_off[v];
     if (step_n[v]) b->n_step_variants += 1;
   }
@@ -1052,7 +1068,9 @@ int batch_prepare(prx_batch* b) {
   L.build_smem = build_smem;
   L.act = b->maps + nmaps;
   L.act_n = b->act_n;
-  for (int v = 0; v < 4; ++v) {
+  L.any_nearest = false;
+  for (const Sys& m : table) L.any_nearest = L.any_nearest || (m.has_rx && m.R.rule == PRX_SELECT_NEAREST);
+  for (int v = 0; v < 8; ++v) {
     L.step_off[v] = step_off[v];
     L.step_n[v] = step_n[v];
   }

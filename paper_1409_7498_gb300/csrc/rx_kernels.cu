@@ -52,48 +52,16 @@ __device__ __forceinline__ long long block_sum_ll(long long v) {
 }
 
 // Work list of the eligible A's (their order does not matter: each A's
-// result goes to its own slot), and win[] cleared for every slot.
-__device__ __forceinline__ void rx_compact_body(const Sys& S, const Blk blk) {
-  const RxParams& R = S.R;
-
-  Ctl* ctl = S.ctl;
-  const SoA B = ctl->set ? S.s1 : S.s0;
-  const uint32_t i = blk.b * blockDim.x + threadIdx.x;
-  bool el = false;
-  if (i < S.n) {
-    S.win[i] = NONE;
-    el = R.nr > 1 ? rx_elig_A(R, B.type[i], B.state[i]) != 0u
-                  : in_window(R.mask_A, R.a_lo, R.a_hi, B.type[i], B.state[i]);
-  }
-  // one atomic per block: warp ballots, block prefix in shared memory
-  __shared__ uint32_t wcnt[RX_THREADS / 32];
-  __shared__ uint32_t bbase;
-  const uint32_t bal = __ballot_sync(0xFFFFFFFFu, el);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) wcnt[wid] = __popc(bal);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t t = 0;
-    for (int w = 0; w < RX_THREADS / 32; ++w) {
-      const uint32_t c = wcnt[w];
-      wcnt[w] = t;
-      t += c;
-    }
-    bbase = t ? atomicAdd(&ctl->n_active, t) : 0u;
-  }
-  __syncthreads();
-  if (el) S.tmp[bbase + wcnt[wid] + __popc(bal & ((1u << lane) - 1u))] = i;
-}
-
-// The compaction of a single system: four slots per thread (one 4-byte load
-// of types and one of states, one 16-byte clear of win), so a quarter of
-// the blocks and of the block-level atomics on the work-list counter.  The
-// list's order differs from rx_compact_body's, which does not matter.
-__global__ void __launch_bounds__(RX_THREADS) k_rx_compact4(Sys S) {
+// result goes to its own slot), and win[] cleared for every slot.  Four slots
+// per thread (one 4-byte load of types and one of states, one 16-byte clear
+// of win), so a quarter of the blocks and of the block-level atomics on the
+// work-list counter that one slot per thread takes.  b: the block's index
+// among the blocks of 4 RX_THREADS slots.
+__device__ __forceinline__ void rx_compact_body(const Sys& S, uint32_t b) {
   const RxParams& R = S.R;
   Ctl* ctl = S.ctl;
   const SoA B = ctl->set ? S.s1 : S.s0;
-  const uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4u;
+  const uint32_t i0 = (b * blockDim.x + threadIdx.x) * 4u;
   uint32_t bits = 0u;
   if (i0 + 3u < S.n) {
     const uchar4 t4 = *reinterpret_cast<const uchar4*>(B.type + i0);
@@ -144,13 +112,15 @@ __global__ void __launch_bounds__(RX_THREADS) k_rx_compact4(Sys S) {
   for (uint32_t u = 0; u < 4u; ++u)
     if ((bits >> u) & 1u) S.tmp[pos++] = i0 + u;
 }
+__global__ void __launch_bounds__(RX_THREADS) k_rx_compact4(Sys S) { rx_compact_body(S, blockIdx.x); }
 
 __global__ void __launch_bounds__(RX_THREADS)
     kb_rx_compact(const Sys* __restrict__ T, const BlkMap* __restrict__ M) {
   const BlkMap m = M[blockIdx.x];
   const Sys& S = T[m.sys];
   if (!S.has_rx) return;  // this member has no reaction scheme
-  rx_compact_body(S, Blk{m.b, m.nb});
+  if (m.b & 3u) return;  // (the map's entries are blocks of RX_THREADS slots)
+  rx_compact_body(S, m.b >> 2);
 }
 
 template <bool NL16>
@@ -162,8 +132,11 @@ __device__ __forceinline__ void rx_find_body(const Sys& S, const Blk blk, long l
   const SoA B = ctl->set ? S.s1 : S.s0;
   const uint4* P = ctl->phase ? S.P1 : S.P0;
   const uint32_t nact = ctl->n_active;
+  // four lanes per eligible A (random rule) or one: blocks past them have nothing to do
+  const bool four = R.rule != PRX_SELECT_NEAREST && R.nr <= 1;
+  if (blk.b * (four ? blockDim.x / 4u : blockDim.x) >= nact) return;
   long long ncand = 0, nret = 0;
-  if (R.rule != PRX_SELECT_NEAREST && R.nr <= 1) {
+  if (four) {
     rx_find_random4<NL16>(S, blk, B, P, step, S.tmp, nact, ncand, nret);
   } else {
     // the nearest rule and concurrent reactions: one thread per eligible A
@@ -192,7 +165,7 @@ template <bool NL16>
 __global__ void __launch_bounds__(RX_THREADS) k_rx_find(Sys S, long long step_arg) {
   rx_find_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, step_arg);
 }
-__global__ void __launch_bounds__(RX_THREADS)
+__global__ void __launch_bounds__(RX_THREADS, 4)
     kb_rx_find(const Sys* __restrict__ T, const BlkMap* __restrict__ M) {
   const BlkMap m = M[blockIdx.x];
   const Sys& S = T[m.sys];
@@ -246,6 +219,10 @@ __device__ __forceinline__ void rx_select_apply_body(const Sys& S, const Blk blk
   const unsigned long long step = step_arg >= 0 ? (unsigned long long)step_arg : ctl->step;
   const SoA B = ctl->set ? S.s1 : S.s0;
   const uint32_t nact = ctl->n_active;
+  // blocks past the eligible A's have nothing to do; the last of the others
+  // (of the first, when there is no A) writes the record
+  const uint32_t busy = max(1u, min(blk.nb, (nact + blockDim.x - 1u) / blockDim.x));
+  if (blk.b >= busy) return;
   long long nwin = 0, nfin = 0;
   // population changes of this block's bonds, per (type, state)
   __shared__ int32_t dpop[PRX_MAX_TYPES * PRX_MAX_STATES];
@@ -285,7 +262,7 @@ __device__ __forceinline__ void rx_select_apply_body(const Sys& S, const Blk blk
   __threadfence();
   __shared__ bool is_last;
   __syncthreads();
-  if (threadIdx.x == 0) is_last = atomicAdd(&ctl->done_rx, 1u) == blk.nb - 1;
+  if (threadIdx.x == 0) is_last = atomicAdd(&ctl->done_rx, 1u) == busy - 1;
   __syncthreads();
   if (is_last) {
     if (threadIdx.x == 0) ctl->done_rx = 0u;
@@ -297,7 +274,7 @@ template <bool NL16>
 __global__ void __launch_bounds__(RX_THREADS) k_rx_select_apply(Sys S, long long step_arg) {
   rx_select_apply_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, step_arg);
 }
-__global__ void __launch_bounds__(RX_THREADS)
+__global__ void __launch_bounds__(RX_THREADS, 4)
     kb_rx_select_apply(const Sys* __restrict__ T, const BlkMap* __restrict__ M) {
   const BlkMap m = M[blockIdx.x];
   const Sys& S = T[m.sys];
@@ -533,7 +510,8 @@ void launch_batch_rx(const BatchLaunch& L, cudaStream_t st) {
   kb_rx_begin<<<L.n_one, 32, 0, st>>>(L.T, L.one);
   kb_rx_compact<<<L.n_part, RX_THREADS, 0, st>>>(L.T, L.part);
   kb_rx_find<<<L.n_part, RX_THREADS, 0, st>>>(L.T, L.part);
-  kb_rx_find_T<<<L.n_part, RX_THREADS, 0, st>>>(L.T, L.part);
+  // (one entry when no member has the nearest-partner rule: it then does nothing)
+  kb_rx_find_T<<<L.any_nearest ? L.n_part : 1u, RX_THREADS, 0, st>>>(L.T, L.part);
   kb_rx_select_apply<<<L.n_part, RX_THREADS, 0, st>>>(L.T, L.part);
 }
 
