@@ -17,7 +17,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libpolyrx.so")
-SOURCES = ["engine.cu", "md_kernels.cu", "rx_kernels.cu", "runtime.cu", "noalloc.cu", "dg.cu"]
+SOURCES = ["engine.cu", "bonds.cu", "md_kernels.cu", "rx_kernels.cu", "runtime.cu", "noalloc.cu", "dg.cu"]
 # relocatable device code only where a kernel launches device graphs
 RDC = {"dg.cu"}
 HEADERS = [os.path.join(CSRC, h) for h in ("prx_internal.cuh", "md_device.cuh", "rx_device.cuh")]

@@ -149,6 +149,14 @@ __device__ __forceinline__ uint32_t periodic_fx_cvt(double x, long long Lfx, uns
   return (uint32_t)__umul64hi(a, M);
 }
 
+// Forces read-back: force and energy of particle p.
+__device__ __forceinline__ void store_force(const Sys& S, uint32_t p, double fx, double fy, double fz, double e) {
+  S.fout[3 * (size_t)p + 0] = fx;
+  S.fout[3 * (size_t)p + 1] = fy;
+  S.fout[3 * (size_t)p + 2] = fz;
+  S.eout[p] = e;
+}
+
 // Random force of the Langevin step (zero without a thermostat).
 __device__ __forceinline__ float3 random_force(const Sys& S, unsigned long long step, uint32_t pid) {
   float3 R = make_float3(0.f, 0.f, 0.f);
@@ -250,7 +258,8 @@ __device__ __forceinline__ void pair32_flat(const Sys& S, uint4 pj, uint4 pi, fl
 // FP32 step kernel: one thread per slot, WCA over the Verlet list.
 // ---------------------------------------------------------------------------
 // The step of slot i: forces over its list and bonds, then the integration
-// (or, FORCES_ONLY, the forces written out); returns the rebuild trigger.
+// (or, FORCES_ONLY, the forces written out by particle); returns the rebuild
+// trigger.
 template <bool NL16, bool FORCES_ONLY, bool CUBIC, bool CAP>
 __device__ __forceinline__ bool step_one(const Sys& S, Ctl* ctl, const SoA& B,
                                          const uint4* __restrict__ P, uint4* __restrict__ Pn,
@@ -327,10 +336,7 @@ __device__ __forceinline__ bool step_one(const Sys& S, Ctl* ctl, const SoA& B,
   }
   if (!ok) set_status(ctl, PRX_EOVERSTRETCH);
   if constexpr (FORCES_ONLY) {
-    S.fout[3 * (size_t)i + 0] = (double)fx;
-    S.fout[3 * (size_t)i + 1] = (double)fy;
-    S.fout[3 * (size_t)i + 2] = (double)fz;
-    S.eout[i] = (double)e;
+    store_force(S, __ldg(B.id + i), (double)fx, (double)fy, (double)fz, (double)e);
     return false;
   } else {
     const double xi = B.x[i], yi = B.y[i], zi = B.z[i];

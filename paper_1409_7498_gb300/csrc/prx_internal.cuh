@@ -383,9 +383,10 @@ void launch_rx(const Sys& S, cudaStream_t st, long long step_arg,
 void launch_observables(const Sys& S, cudaStream_t st, int nblocks);
 // Counts the populations per (type, state) into S.pop (creation).
 void launch_pop_init(const Sys& S, cudaStream_t st);
-void launch_pair_hist(const Sys& S, cudaStream_t st, const PairClass& a, const PairClass& b,
-                      const double* e2, int nbins, unsigned long long* counts,
-                      unsigned long long* nab);
+void launch_pair_hist(const Sys& S, cudaStream_t st, const PairClass& a, const PairClass& b, double r_max, double* e2,
+                      int nbins, unsigned long long* counts);
+// Sum of eout (after a forces-only launch); where the device value will be.
+const double* launch_energy_sum(const Sys& S, cudaStream_t st);
 int rebin_kernel_count(const Sys& S);
 int rx_kernel_count(int rule);
 int step_kernel_count(int fp64);
@@ -395,6 +396,8 @@ size_t build_tile_smem(const Sys& S);
 // into the box, ids and types checked) or velocities (which = 1), copied to
 // the device; errors land in ctl->input_err.
 void launch_stage_input(const Sys& S, cudaStream_t st, const double* buf, int which);
+// The first m records of a bond list in canonical order (bonds.cu).
+BondRec* launch_sort_bonds(BondRec* list, BondRec* scratch, uint32_t m, cudaStream_t st);
 // Per-particle arrays in particle (id) order into device buffer `out`:
 // 0 states, 1 types, 2 positions wrapped into the box, 3 velocities.
 void launch_gather_by_id(const Sys& S, cudaStream_t st, int what, void* out);

@@ -34,6 +34,7 @@ constexpr double kDefaultSkin = 0.3;
 constexpr uint32_t kHistCap = 8192;
 constexpr uint64_t kCkptMagic = 0x31305850594C4F50ull;  // "POLYRX01"
 constexpr int kNoRxChunk = 10;
+constexpr uint32_t kMaxBins = 2048;  // of a pair histogram
 
 struct ProfEvent {
   std::string name;
@@ -81,6 +82,11 @@ struct prx_system {
   EngPlan eng;
   bool eng_planned = false;
   uint64_t eng_launches = 0;
+  size_t bond_scratch = 0;  // bytes of fout and eout together
+  // pair histogram: squared bin edges, counts and class sizes; a pinned copy of
+  // the latter
+  double* hist_dev = nullptr;
+  unsigned long long* hist_host = nullptr;
   bool profiling = false;
   std::vector<ProfEvent> prof;
   std::string err;
@@ -755,8 +761,11 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
     return bail(fail(sys, PRX_ECUDA, "capture stream creation failed"));
   if (cudaMallocHost(&sys->ctl_host, sizeof(Ctl)) != cudaSuccess)
     return bail(fail(sys, PRX_ENOMEM, "pinned control block"));
-  if (cudaMallocHost(&sys->obs_host, sizeof(*sys->obs_host) * (PRX_OBS_SLOTS + 1)) != cudaSuccess)
+  const size_t obs_bytes = sizeof(*sys->obs_host) * (PRX_OBS_SLOTS + 1);
+  if (cudaMallocHost(&sys->obs_host, obs_bytes + 8 * (size_t)(kMaxBins + 2)) != cudaSuccess)
     return bail(fail(sys, PRX_ENOMEM, "pinned observables block"));
+  static_assert(sizeof(*sys->obs_host) % 8 == 0, "the histogram's counts follow the observables");
+  sys->hist_host = (unsigned long long*)((char*)sys->obs_host + obs_bytes);
   memset(sys->ctl_host, 0, sizeof(Ctl));
 
   DevArena A;
@@ -772,9 +781,10 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   A.add(&S.hist, (size_t)S.hist_cap + 2), A.add(&S.ctl, 1);
   A.add(&S.pop, (size_t)POP_REPLICAS * PRX_MAX_TYPES * PRX_MAX_STATES);
   A.add(&S.red, 4 * ((size_t)(n + RX_THREADS - 1) / RX_THREADS + 1));
-  A.add(&S.fout, 3 * (size_t)n), A.add(&S.eout, (size_t)n);
-  A.add(&sys->eng_bar, 64);
+  A.add(&S.fout, 3 * (size_t)n), A.add(&S.eout, (size_t)n);  // (one after the other: the bond sort's scratch)
+  A.add(&sys->eng_bar, 64), A.add(&sys->hist_dev, 2 * (size_t)kMaxBins + 3);
   if ((rc = A.commit(sys, sys->dev_allocs))) return bail(rc);
+  sys->bond_scratch = (size_t)((char*)S.eout - (char*)S.fout) + 8 * (size_t)n;
   if ((rc = setup_grid(sys, grid_rc > rc_w ? grid_rc : rc_w))) return bail(rc);
 
   const SoA& B = S.s0;
@@ -1155,7 +1165,7 @@ uint64_t estimate_bytes(const prx_system_desc& d, double r_react) {
   const uint64_t allocs = 40;  // separate cudaMalloc calls, each rounded up
   return 2 * per_set + n * (2 * 16 + 4 * 4) + (n * cap / 2 + 1) * sizeof(prx_bond) +
            (kHistCap + 2ull) * sizeof(prx_history_record) + sizeof(Ctl) + 32 * (n / RX_THREADS + 2) +
-           32 * n + ncell * 12 + (ncell <= ENG_CELLS ? ncell * 4 * ENG_BUCKET : 0) + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + allocs * 4096;
+           32 * n + ncell * 12 + (ncell <= ENG_CELLS ? ncell * 4 * ENG_BUCKET : 0) + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + 8 * (2 * kMaxBins + 3) + allocs * 4096;
 }
 
 
@@ -1405,25 +1415,16 @@ int prx_compute_forces(prx_system* sys, double* f_out, double* epot_out) {
     if (epot_out) *epot_out = 0.0;
     return PRX_OK;
   }
+  // the forces by particle, as the kernel writes them, and the energies' sum
   launch_step(sys->S, sys->stream, sys->d.force_precision == PRX_FORCE_FP64, 1, 0, 0);
   sys->other_launches++;
   CK(cudaGetLastError());
-  std::vector<double> f(3 * n), e(n);
-  CK(cudaMemcpyAsync(f.data(), sys->S.fout, 24 * n, cudaMemcpyDeviceToHost, sys->stream));
-  CK(cudaMemcpyAsync(e.data(), sys->S.eout, 8 * n, cudaMemcpyDeviceToHost, sys->stream));
-  HostSlots h;
-  int rc = fetch_slots(sys, h, 0u);
-  if (rc) return rc;
-  std::vector<double> e_by_id(n);
-  for (size_t s = 0; s < n; ++s) {
-    const uint32_t p = h.id[s];
-    for (int k = 0; k < 3; ++k) f_out[3 * (size_t)p + k] = f[3 * s + k];
-    e_by_id[p] = e[s];
-  }
+  CK(cudaMemcpyAsync(f_out, sys->S.fout, 24 * n, cudaMemcpyDeviceToHost, sys->stream));
   if (epot_out) {
-    double t = 0.0;
-    for (size_t p = 0; p < n; ++p) t += e_by_id[p];
-    *epot_out = t;
+    const double* sum = launch_energy_sum(sys->S, sys->stream);
+    sys->other_launches += 2;
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(epot_out, sum, 8, cudaMemcpyDeviceToHost, sys->stream));
   }
   return sync_status(sys);
 }
@@ -1472,6 +1473,16 @@ int prx_get_bonds(prx_system* sys, prx_bond* out, uint64_t cap, uint64_t* n_out)
   *n_out = nb;
   const uint64_t m = std::min(cap, nb);
   if (!m || !out) {  // the count alone
+    rc = sync_status(sys);
+    if (rc) return rc;
+    return cap < nb ? fail(sys, PRX_ECAPACITY, "bond buffer too small") : PRX_OK;
+  }
+  // in canonical order on the device (the force scratch arrays, free outside
+  // a step, take the other half of the merge), unless they are too short
+  if (24ull * nb <= sys->bond_scratch) {
+    const BondRec* sorted = launch_sort_bonds(sys->S.bonds, (BondRec*)sys->S.fout, (uint32_t)nb, sys->stream);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(out, sorted, sizeof(prx_bond) * m, cudaMemcpyDeviceToHost, sys->stream));
     rc = sync_status(sys);
     if (rc) return rc;
     return cap < nb ? fail(sys, PRX_ECAPACITY, "bond buffer too small") : PRX_OK;
@@ -1850,42 +1861,21 @@ int prx_load(const char* path, void* cuda_stream, prx_system** out) {
 
 int prx_pair_histogram(prx_system* sys, const prx_class* a, const prx_class* b, double r_max,
                        uint32_t nbins, uint64_t* counts, uint64_t* n_a, uint64_t* n_b) {
-  if (!sys || !a || !b || !counts || nbins < 1 || nbins > 2048) return PRX_EINVAL;
+  if (!sys || !a || !b || !counts || nbins < 1 || nbins > kMaxBins) return PRX_EINVAL;
   if (!(r_max > 0.0) || r_max > sys->grid_rcut)
     return fail(sys, PRX_EINVAL, "r_max beyond the cutoff the Verlet lists guarantee");
-  std::vector<double> e2(nbins + 1);
-  for (uint32_t k = 0; k <= nbins; ++k) {
-    const double e = r_max * (double)k / (double)nbins;
-    e2[k] = e * e;
-  }
-  double* d_e2 = nullptr;
-  unsigned long long* d_c = nullptr;
-  CK(cudaMalloc(&d_e2, sizeof(double) * (nbins + 1)));
-  if (cudaMalloc(&d_c, sizeof(unsigned long long) * (nbins + 2)) != cudaSuccess) {
-    cudaFree(d_e2);
-    return fail(sys, PRX_ENOMEM, "histogram buffers");
-  }
-  std::vector<unsigned long long> h(nbins + 2, 0ull);
-  cudaError_t e = cudaMemcpyAsync(d_e2, e2.data(), sizeof(double) * (nbins + 1), cudaMemcpyHostToDevice,
-                                  sys->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d_c, 0, sizeof(unsigned long long) * (nbins + 2), sys->stream);
-  if (e == cudaSuccess && sys->S.n) {
-    launch_pair_hist(sys->S, sys->stream, PairClass{a->type_mask, a->s_lo, a->s_hi},
-                     PairClass{b->type_mask, b->s_lo, b->s_hi}, d_e2, (int)nbins, d_c, d_c + nbins);
-    sys->other_launches++;
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h.data(), d_c, sizeof(unsigned long long) * (nbins + 2), cudaMemcpyDeviceToHost,
-                        sys->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(sys->stream);
-  cudaFree(d_e2);
-  cudaFree(d_c);
-  if (e != cudaSuccess) return fail(sys, PRX_ECUDA, std::string("pair histogram: ") + cudaGetErrorString(e));
-  for (uint32_t k = 0; k < nbins; ++k) counts[k] = h[k];
-  if (n_a) *n_a = h[nbins];
-  if (n_b) *n_b = h[nbins + 1];
-  return sync_status(sys);
+  double* d_e2 = sys->hist_dev;
+  unsigned long long* d_c = (unsigned long long*)(d_e2 + kMaxBins + 1);
+  launch_pair_hist(sys->S, sys->stream, PairClass{a->type_mask, a->s_lo, a->s_hi},
+                   PairClass{b->type_mask, b->s_lo, b->s_hi}, r_max, d_e2, (int)nbins, d_c);
+  sys->other_launches += 2;
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(sys->hist_host, d_c, 8 * (size_t)(nbins + 2), cudaMemcpyDeviceToHost, sys->stream));
+  const int rc = sync_status(sys);  // (one wait for the counts and the control block)
+  for (uint32_t k = 0; k < nbins; ++k) counts[k] = sys->hist_host[k];
+  if (n_a) *n_a = sys->hist_host[nbins];
+  if (n_b) *n_b = sys->hist_host[nbins + 1];
+  return rc;
 }
 
 // ---- autotuner -------------------------------------------------------------------
