@@ -674,7 +674,7 @@ __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA
   };
   for (uint32_t o = g; o < S.n; o += stride) eng_permute_one(S, A, B, P, o, new_slot);
   if (bar.sync(false) == 2) return 2;
-  for (uint32_t c = g; c < ncell; c += stride) S.count[c] = 0u;  // for the next rebuild
+  for (uint32_t c = g; c < ncell; c += stride) S.count[c] = 0u;  // (zero outside rebuilds)
   const uint32_t nt = (uint32_t)(S.eng_tiles_y * S.nc[2]);
   for (uint32_t t = b; t < nt; t += nb) {
     eng_build_tile<NL16>(S, P, S.win, t, smem);
@@ -769,8 +769,6 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
   // share its L1; FP32: one chunk per warp, its slots in the lanes' registers
   const uint32_t c0 = (uint32_t)((unsigned long long)chunks * b / bar.nb);
   const uint32_t c1 = (uint32_t)((unsigned long long)chunks * (b + 1u) / bar.nb);
-  for (uint32_t c = b * ENG_THREADS + threadIdx.x; c < (((uint32_t)S.ncell + 3u) & ~3u); c += bar.nb * ENG_THREADS)
-    S.count[c] = 0u;
   [[maybe_unused]] Resident r;
   const uint32_t ri = (c0 + warp) * 32u + (threadIdx.x & 31u);
   const bool rv = !F64 && c0 + warp < c1 && ri < S.n;

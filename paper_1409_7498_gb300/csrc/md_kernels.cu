@@ -562,6 +562,8 @@ __device__ __forceinline__ void rebin_cellsort_body(const Sys& S, const Blk blk)
   const uint32_t c = blk.b * blockDim.x + threadIdx.x;
   if (c >= (uint32_t)S.ncell) return;
   const uint32_t s0 = S.cell_start[c], s1 = S.cell_start[c + 1];
+  S.count[c] = 0u;  // for the next rebuild
+  S.fill[c] = 0u;
   if (s1 - s0 <= 8u) {
     // the common case: an 8-input sorting network in registers (absent
     // members padded with the largest key)
@@ -995,8 +997,6 @@ void launch_rebin(const Sys& S, cudaStream_t st, int mode, void (*hook)(void*, c
   auto H = [&](const char* nm, int p) {
     if (hook) hook(ctx, nm, p);
   };
-  cudaMemsetAsync(S.count, 0, sizeof(uint32_t) * S.ncell, st);
-  cudaMemsetAsync(S.fill, 0, sizeof(uint32_t) * S.ncell, st);
   H(mode == 2 ? "count_keys" : "rebin_keys", 0);
   if (mode == 2) k_count_keys<<<gp, 256, 0, st>>>(S);
   else if (mode == 1) k_rebin_keys_x<<<gp, 256, 0, st>>>(S);

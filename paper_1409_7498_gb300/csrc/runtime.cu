@@ -344,6 +344,9 @@ int setup_grid(prx_system* sys, double rc) {
   A.add(&S.nn, (size_t)S.n);
   A.add(&S.bucket, ncell <= (long long)ENG_CELLS ? (size_t)ncell * ENG_BUCKET : 0);
   if ((rc2 = A.commit(sys, sys->grid_allocs))) return rc2;
+  // the cell counters are zero outside rebuilds
+  CK(cudaMemsetAsync(S.count, 0, sizeof(uint32_t) * (((size_t)ncell + 3) & ~(size_t)3), sys->stream));
+  CK(cudaMemsetAsync(S.fill, 0, sizeof(uint32_t) * (size_t)ncell, sys->stream));
   {
     // list-build tiling: the rows per tile (the rows of a layer shared out
     // evenly) that keep most of the passes of 256 threads busy and restage
