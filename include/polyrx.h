@@ -455,7 +455,9 @@ typedef struct {
   uint64_t steps;           /* steps run by the batch */
   uint64_t rebuilds;        /* steps after which some member rebuilt its lists */
   uint64_t reactions;       /* reaction steps run */
-  uint64_t kernel_launches; /* kernels launched by the batch */
+  uint64_t kernel_launches; /* kernels of the batch's work: one per step and variant (and the
+                               device-driven run's own), ten per rebuild, five per reaction step;
+                               merged kernels count as those they stand for */
   uint64_t graph_launches;  /* CUDA graph replays */
   uint32_t max_slots;       /* as given to prx_batch_create (0: no limit) */
   uint32_t slots_used;      /* admitted systems not yet reported by prx_batch_poll */

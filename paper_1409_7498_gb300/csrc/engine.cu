@@ -300,61 +300,6 @@ __device__ __forceinline__ bool eng_step64(const Sys& S, Ctl* ctl, const SoA& B,
   return moved;
 }
 
-// Cell of a fixed-point position.
-__device__ __forceinline__ uint32_t eng_cell(const Sys& S, const uint4 q) {
-  const uint32_t cx = __umulhi(q.x, (uint32_t)S.nc[0]);
-  const uint32_t cy = __umulhi(q.y, (uint32_t)S.nc[1]);
-  const uint32_t cz = __umulhi(q.z, (uint32_t)S.nc[2]);
-  return (cz * (uint32_t)S.nc[1] + cy) * (uint32_t)S.nc[0] + cx;
-}
-
-// Old slot o goes to its new slot: every per-particle array into the other
-// set, bond partners renamed, a fresh displacement reference, and the slot's
-// cell (into win, read by the list build).  new_slot(j, cell of j) gives a
-// slot's new place.
-template <class F>
-__device__ __forceinline__ void eng_permute_one(const Sys& S, const SoA& A, const SoA& B, uint4* P, uint32_t o,
-                                                F new_slot) {
-  double x = A.x[o], y = A.y[o], z = A.z[o];
-  const double vx = A.vx[o], vy = A.vy[o], vz = A.vz[o];
-  const uint32_t pid = A.id[o];
-  const uint8_t ty = A.type[o];
-  const int8_t st = A.state[o];
-  const uint32_t nb = A.nadj[o];
-  const uint32_t key = S.key[o];
-  const uint32_t* from = A.adj + (size_t)o * S.cap;
-  // the first two bonds' chains beside the slot's own
-  const uint32_t e0 = from[0], e1 = S.cap > 1 ? from[1] : 0u;
-  const uint32_t k0 = nb > 0u ? S.key[e0 & SLOT_MASK] : 0u, k1 = nb > 1u ? S.key[e1 & SLOT_MASK] : 0u;
-  const uint32_t s = new_slot(o, key);
-  uint32_t* to = B.adj + (size_t)s * S.cap;
-  if (nb > 0u) to[0] = new_slot(e0 & SLOT_MASK, k0) | (e0 & ~SLOT_MASK);
-  if (nb > 1u) to[1] = new_slot(e1 & SLOT_MASK, k1) | (e1 & ~SLOT_MASK);
-#pragma unroll 1
-  for (uint32_t b = 2; b < nb; ++b) {
-    const uint32_t f = from[b];
-    to[b] = new_slot(f & SLOT_MASK, S.key[f & SLOT_MASK]) | (f & ~SLOT_MASK);
-  }
-  x = wrap_into_box(x, S.L[0]);
-  y = wrap_into_box(y, S.L[1]);
-  z = wrap_into_box(z, S.L[2]);
-  B.x[s] = x;
-  B.y[s] = y;
-  B.z[s] = z;
-  B.vx[s] = vx;
-  B.vy[s] = vy;
-  B.vz[s] = vz;
-  B.id[s] = pid;
-  B.type[s] = ty;
-  B.state[s] = st;
-  B.nadj[s] = (uint8_t)nb;
-  const uint32_t X = periodic_fx(x, S.Lfx[0], S.M64[0]);
-  const uint32_t Y = periodic_fx(y, S.Lfx[1], S.M64[1]);
-  const uint32_t Z = periodic_fx(z, S.Lfx[2], S.M64[2]);
-  P[s] = make_uint4(X, Y, Z, coarse_ref(X, Y, Z, S.wshift));
-  S.win[s] = key;
-}
-
 // Entry k of slot i's list.
 template <bool NL16>
 __device__ __forceinline__ void nl_put(const Sys& S, int k, uint32_t i, uint32_t j) {
@@ -600,7 +545,7 @@ __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA
   const uint32_t ncell = (uint32_t)S.ncell;
   bool over = false;
   for (uint32_t i = g; i < S.n; i += stride) {
-    const uint32_t k = eng_cell(S, P[i]);
+    const uint32_t k = cell_of_pos(S, P[i]);
     S.key[i] = k;
     const uint32_t rank = atomicAdd(&S.count[k], 1u);
     S.new_of_old[i] = rank;
@@ -672,7 +617,7 @@ __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA
     for (uint32_t q = 0; q < c; ++q) r += row[q] < j ? 1u : 0u;
     return r;
   };
-  for (uint32_t o = g; o < S.n; o += stride) eng_permute_one(S, A, B, P, o, new_slot);
+  for (uint32_t o = g; o < S.n; o += stride) permute_old<false>(S, A, B, P, S.win, o, new_slot);
   if (bar.sync(false) == 2) return 2;
   for (uint32_t c = g; c < ncell; c += stride) S.count[c] = 0u;  // (zero outside rebuilds)
   const uint32_t nt = (uint32_t)(S.eng_tiles_y * S.nc[2]);
@@ -929,7 +874,7 @@ static unsigned engine_resident(const void* k, size_t sm) {
 // as do boxes with more cells or longer rows than the rebuild holds.
 EngPlan engine_plan(const Sys& S, int fp64) {
   EngPlan p;
-  if (!S.n || S.ncell > (int)ENG_CELLS || !S.eng_ty || S.fcapf > 0.f || S.step_lanes != 1) return p;
+  if (!S.n || !S.bucket || S.ncell > (int)ENG_CELLS || !S.eng_ty || S.fcapf > 0.f || S.step_lanes != 1) return p;
   if (fp64 && S.n > ENG_F64_MAX) return p;
   p.smem = engine_smem(S);
   const unsigned warps = ENG_THREADS / 32;

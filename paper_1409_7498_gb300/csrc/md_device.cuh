@@ -636,6 +636,61 @@ __device__ __forceinline__ void build_tile(const Sys& S, const float4* F, const 
   }
 }
 
+// Cell of a fixed-point position.
+__device__ __forceinline__ uint32_t cell_of_pos(const Sys& S, const uint4 q) {
+  const uint32_t cx = __umulhi(q.x, (uint32_t)S.nc[0]);
+  const uint32_t cy = __umulhi(q.y, (uint32_t)S.nc[1]);
+  const uint32_t cz = __umulhi(q.z, (uint32_t)S.nc[2]);
+  return (cz * (uint32_t)S.nc[1] + cy) * (uint32_t)S.nc[0] + cx;
+}
+
+// Old slot o goes to its new slot: every per-particle array into the other
+// set, bond partners renamed, a fresh displacement reference, and the slot's
+// cell (into cell_of, read by the list build).  new_slot(j, cell of j) gives a
+// slot's new place.  XYZ: also the list build's coordinates.
+template <bool XYZ, class F>
+__device__ __forceinline__ void permute_old(const Sys& S, const SoA& A, const SoA& B, uint4* P, uint32_t* cell_of,
+                                            uint32_t o, F new_slot) {
+  double x = A.x[o], y = A.y[o], z = A.z[o];
+  const double vx = A.vx[o], vy = A.vy[o], vz = A.vz[o];
+  const uint32_t pid = A.id[o];
+  const uint8_t ty = A.type[o];
+  const int8_t st = A.state[o];
+  const uint32_t nb = A.nadj[o];
+  const uint32_t key = S.key[o];
+  const uint32_t* from = A.adj + (size_t)o * S.cap;
+  // the first two bonds' chains beside the slot's own
+  const uint32_t e0 = from[0], e1 = S.cap > 1 ? from[1] : 0u;
+  const uint32_t k0 = nb > 0u ? S.key[e0 & SLOT_MASK] : 0u, k1 = nb > 1u ? S.key[e1 & SLOT_MASK] : 0u;
+  const uint32_t s = new_slot(o, key);
+  uint32_t* to = B.adj + (size_t)s * S.cap;
+  if (nb > 0u) to[0] = new_slot(e0 & SLOT_MASK, k0) | (e0 & ~SLOT_MASK);
+  if (nb > 1u) to[1] = new_slot(e1 & SLOT_MASK, k1) | (e1 & ~SLOT_MASK);
+#pragma unroll 1
+  for (uint32_t b = 2; b < nb; ++b) {
+    const uint32_t f = from[b];
+    to[b] = new_slot(f & SLOT_MASK, S.key[f & SLOT_MASK]) | (f & ~SLOT_MASK);
+  }
+  x = wrap_into_box(x, S.L[0]);
+  y = wrap_into_box(y, S.L[1]);
+  z = wrap_into_box(z, S.L[2]);
+  B.x[s] = x;
+  B.y[s] = y;
+  B.z[s] = z;
+  B.vx[s] = vx;
+  B.vy[s] = vy;
+  B.vz[s] = vz;
+  B.id[s] = pid;
+  B.type[s] = ty;
+  B.state[s] = st;
+  B.nadj[s] = (uint8_t)nb;
+  const uint32_t X = periodic_fx(x, S.Lfx[0], S.M64[0]);
+  const uint32_t Y = periodic_fx(y, S.Lfx[1], S.M64[1]);
+  const uint32_t Z = periodic_fx(z, S.Lfx[2], S.M64[2]);
+  P[s] = make_uint4(X, Y, Z, coarse_ref(X, Y, Z, S.wshift));
+  if constexpr (XYZ) reinterpret_cast<float4*>(S.fout)[s] = build_xyz(S, X, Y, Z, key, s);
+  cell_of[s] = key;
+}
 }  // namespace
 
 }  // namespace prx

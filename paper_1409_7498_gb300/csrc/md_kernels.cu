@@ -207,8 +207,9 @@ __global__ void __launch_bounds__(BT, 1536 / BT)
 template <bool NL16, bool CUBIC, bool CAP>
 __global__ void __launch_bounds__(256, 6)
     kb_step_nl(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t n,
-               cudaGraphConditionalHandle cond, int use_cond, uint32_t* __restrict__ act_n) {
-  if (blockIdx.x == 0 && threadIdx.x < 5) act_n[threadIdx.x] = 0u;  // for this step's rebuild plan
+               cudaGraphConditionalHandle cond, int use_cond, uint32_t* act_n, BlkMap* act, uint4 act_off) {
+  __shared__ int need;
+  if (!act && blockIdx.x == 0 && threadIdx.x < 5) act_n[threadIdx.x] = 0u;  // for this step's rebuild plan
   __shared__ __align__(16) unsigned char sbuf[sizeof(Sys)];
   const Sys& S = *reinterpret_cast<const Sys*>(sbuf);
   static_assert(sizeof(Sys) % 8 == 0, "Sys is copied in 8-byte words");
@@ -234,7 +235,27 @@ __global__ void __launch_bounds__(256, 6)
     __syncthreads();  // the block's work on the member is done (and its parameters read)
     if (threadIdx.x == 0) {
       __threadfence();
-      if (atomicAdd(&ctl->done_step, cnt) + cnt == m.nb) step_done(S, ph, step, cond, use_cond);
+      need = 0;
+      if (atomicAdd(&ctl->done_step, cnt) + cnt == m.nb) {
+        need = act && atomicAdd(&ctl->rebin_flag, 0) ? 1 : 0;
+        if (!need) step_done(S, ph, step, cond, use_cond);
+      }
+    }
+    __syncthreads();
+    if (need) {  // the member's last block lists its blocks for the rebuild's kernels
+      __shared__ uint32_t at[3];
+      const uint32_t nb[3] = {m.nb, ((uint32_t)S.ncell + SCAN_TILE - 1) / SCAN_TILE, (uint32_t)(S.tiles_y * S.nc[2])};
+      if (threadIdx.x == 0) {
+        at[0] = act_off.x + atomicAdd(&act_n[0], nb[0]);
+        atomicAdd(&act_n[1], nb[0]);
+        at[1] = act_off.y + atomicAdd(&act_n[2], nb[1]);
+        at[2] = act_off.z + atomicAdd(&act_n[3], nb[2]);
+      }
+      __syncthreads();
+      for (int f = 0; f < 3; ++f)
+        for (uint32_t q = threadIdx.x; q < nb[f]; q += blockDim.x) act[at[f] + q] = BlkMap{m.sys, q, nb[f], 0u};
+      __syncthreads();
+      if (threadIdx.x == 0) step_done(S, ph, step, cond, use_cond);
     }
     e += cnt;
     if (e < e1) __syncthreads();
@@ -520,7 +541,8 @@ __global__ void __launch_bounds__(256) kb_scan_down(const Sys* __restrict__ T, c
   }
 }
 
-// Batched rebuilds clear the cell counters in a kernel (a single system uses memsets).
+// Cell counters of a batch's members cleared before its launch-by-launch
+// rebuild.
 __global__ void __launch_bounds__(256) kb_rebin_clear(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
   for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
     const BlkMap m = M[e];
@@ -687,6 +709,107 @@ __global__ void __launch_bounds__(256) kb_rebin_permute(const Sys* __restrict__ 
   }
 }
 
+// ---------------------------------------------------------------------------
+// Rebuild of a batch's members through buckets (all of them with at most
+// BUCKET_CELLS cells that hold few particles): the keys' atomics give each
+// slot's arrival rank in its cell, under which it is noted in the cell's
+// bucket; a scan of the counts gives the cells' first slots, and a slot's new
+// place is its cell's first slot plus the number of the cell's members with a
+// smaller old slot.  With the plan's work done by the step kernel, four
+// kernels instead of ten: 256 replicas 377 -> 366 us per step.  (A single
+// system keeps the seven kernels of launch_rebin: at a million beads the
+// permutation by old slot, whose stores are scattered, takes 67 us instead of
+// the 57 of scatter, sort and permutation.)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void keys_bucket_body(const Sys& S, const Blk blk) {
+  Ctl* ctl = S.ctl;
+  const uint4* P = ctl->phase ? S.P1 : S.P0;
+  const uint32_t i = blk.b * blockDim.x + threadIdx.x;
+  if (i >= S.n) return;
+  const uint32_t k = cell_of_pos(S, P[i]);
+  S.key[i] = k;
+  const uint32_t rank = atomicAdd(&S.count[k], 1u);
+  if (rank < ENG_BUCKET) S.bucket[(size_t)k * ENG_BUCKET + rank] = i;
+}
+
+// Scan tile blk.b with the counts before it summed by the block itself.
+__device__ __forceinline__ void scan_direct_body(const Sys& S, const Blk blk) {
+  const uint32_t n = (uint32_t)S.ncell, base = blk.b * SCAN_TILE;
+  uint32_t part = 0, off;
+#pragma unroll 4
+  for (uint32_t c = threadIdx.x * 4u; c < base; c += 1024u) {
+    const uint4 v = *reinterpret_cast<const uint4*>(S.count + c);
+    part += v.x + v.y + v.z + v.w;
+  }
+  (void)block_exclusive_scan_256(part, off);
+  const uint32_t c0 = base + threadIdx.x * (SCAN_TILE / 256);
+  uint32_t loc[SCAN_TILE / 256];
+  uint32_t s = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_TILE / 256; ++k) {
+    loc[k] = c0 + k < n ? S.count[c0 + k] : 0u;
+    s += loc[k];
+  }
+  uint32_t total;
+  uint32_t run = off + block_exclusive_scan_256(s, total);
+  if (blk.b == 0 && threadIdx.x == 0) S.cell_start[0] = 0u;
+#pragma unroll
+  for (int k = 0; k < SCAN_TILE / 256; ++k) {
+    run += loc[k];
+    if (c0 + k < n) S.cell_start[c0 + k + 1] = run;
+  }
+}
+
+// Old slots of block blk of 256, and the block's share of the counters back to
+// zero.  A cell with more members than a bucket holds (rare where buckets are
+// used) has them counted from the keys.
+__device__ __forceinline__ void permute_bucket_body(const Sys& S, const Blk blk) {
+  Ctl* ctl = S.ctl;
+  const SoA A = ctl->set ? S.s1 : S.s0, B = ctl->set ? S.s0 : S.s1;
+  uint4* P = ctl->phase ? S.P1 : S.P0;
+  auto new_slot = [&](uint32_t j, uint32_t k) {
+    const uint32_t s0 = S.cell_start[k], c = S.cell_start[k + 1] - s0;
+    uint32_t r = s0;
+    if (c <= ENG_BUCKET) {
+      const uint4* row = reinterpret_cast<const uint4*>(S.bucket + (size_t)k * ENG_BUCKET);
+      for (uint32_t q = 0; q < c; q += 4u) {
+        const uint4 v = row[q >> 2];
+        r += (v.x < j ? 1u : 0u) + (q + 1u < c && v.y < j ? 1u : 0u) + (q + 2u < c && v.z < j ? 1u : 0u) +
+             (q + 3u < c && v.w < j ? 1u : 0u);
+      }
+    } else {
+      for (uint32_t i = 0; i < j; ++i) r += S.key[i] == k ? 1u : 0u;
+    }
+    return r;
+  };
+  const uint32_t o = blk.b * 256u + threadIdx.x;
+  if (o < S.n) permute_old<true>(S, A, B, P, S.tmp, o, new_slot);
+  for (uint32_t c = o; c < (uint32_t)S.ncell; c += blk.nb * 256u) S.count[c] = 0u;
+}
+
+// The kernels over the members that need a rebuild.  Their blocks were listed
+// by the step kernel as each member finished: act_n[0 .. 3] count the entries
+// of the keys, the permutation, the scan and the list build.  A count is reset
+// once its kernel is done: the keys' by the scan, the scan's by the
+// permutation, the other two by the list build's last block.
+__global__ void __launch_bounds__(256) kb_keys_bucket(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t* act_n) {
+  const uint32_t n = act_n[0];
+  for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) keys_bucket_body(T[M[e].sys], Blk{M[e].b, M[e].nb});
+}
+__global__ void __launch_bounds__(256) kb_scan_direct(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t* act_n) {
+  const uint32_t n = act_n[2];
+  if (blockIdx.x == 0 && threadIdx.x == 0) act_n[0] = 0u;
+  for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
+    scan_direct_body(T[M[e].sys], Blk{M[e].b, M[e].nb});
+    __syncthreads();
+  }
+}
+__global__ void __launch_bounds__(256, 4) kb_permute_bucket(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t* act_n) {
+  const uint32_t n = act_n[1];
+  if (blockIdx.x == 0 && threadIdx.x == 0) act_n[2] = 0u;
+  for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) permute_bucket_body(T[M[e].sys], Blk{M[e].b, M[e].nb});
+}
+
 // One tile per block; the last warp of the system's tiles flips the SoA set
 // and clears the flag (a warp count, not a block barrier: warps that finish
 // early leave).
@@ -710,14 +833,21 @@ __global__ void __launch_bounds__(256) k_build_nlist(Sys S) {
   build_nlist_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, smem_b);
 }
 __global__ void __launch_bounds__(256, 4)
-    kb_build_nlist(const Sys* __restrict__ T, const BlkMap* __restrict__ M, const uint32_t* __restrict__ C) {
+    kb_build_nlist(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t* C, uint32_t* act_n) {
   extern __shared__ __align__(16) unsigned char smem_b[];
-  for (uint32_t e = blockIdx.x; e < *C; e += gridDim.x) {
+  const uint32_t n = *C;
+  for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
     const BlkMap m = M[e];
     const Sys& S = T[m.sys];
     if (S.nl16) build_nlist_body<true>(S, Blk{m.b, m.nb}, smem_b);
     else build_nlist_body<false>(S, Blk{m.b, m.nb}, smem_b);
     __syncthreads();  // the buffers and the warp count are used again
+  }
+  // bucket rebuilds: the last block resets the counts still set (every block
+  // has read C by then)
+  if (act_n && threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&act_n[4], 1u) == gridDim.x - 1u) act_n[1] = act_n[3] = act_n[4] = 0u;
   }
 }
 
@@ -978,7 +1108,7 @@ int raise_smem_limit(int which, size_t bytes) {
 
 int configure_build_kernel(size_t smem_bytes) { return raise_smem_limit(0, smem_bytes); }
 
-constexpr unsigned kScanSelfTiles = 1024;  // tiles up to which the scan has two passes
+constexpr unsigned kScanSelfTiles = 1024;   // tiles up to which the scan has two passes
 
 int rebin_kernel_count(const Sys& S) {
   return (S.ncell + SCAN_TILE - 1) / SCAN_TILE <= (int)kScanSelfTiles ? 7 : 8;
@@ -996,6 +1126,14 @@ void launch_rebin(const Sys& S, cudaStream_t st, int mode, void (*hook)(void*, c
   const unsigned tiles = blocks_for(S.ncell, SCAN_TILE);
   auto H = [&](const char* nm, int p) {
     if (hook) hook(ctx, nm, p);
+  };
+  auto build = [&] {
+    const unsigned gt = (unsigned)(S.tiles_y * S.nc[2]);
+    const size_t sm = build_tile_smem(S);
+    H("build_nlist", 0);
+    if (S.nl16) k_build_nlist<true><<<gt, S.tile_threads, sm, st>>>(S);
+    else k_build_nlist<false><<<gt, S.tile_threads, sm, st>>>(S);
+    H("build_nlist", 1);
   };
   H(mode == 2 ? "count_keys" : "rebin_keys", 0);
   if (mode == 2) k_count_keys<<<gp, 256, 0, st>>>(S);
@@ -1029,12 +1167,7 @@ void launch_rebin(const Sys& S, cudaStream_t st, int mode, void (*hook)(void*, c
     k_rebin_permute<<<(gp < r ? gp : r), 256, 0, st>>>(S, mode != 2);
   }
   H("rebin_permute", 1);
-  const unsigned gt = (unsigned)(S.tiles_y * S.nc[2]);
-  const size_t sm = build_tile_smem(S);
-  H("build_nlist", 0);
-  if (S.nl16) k_build_nlist<true><<<gt, S.tile_threads, sm, st>>>(S);
-  else k_build_nlist<false><<<gt, S.tile_threads, sm, st>>>(S);
-  H("build_nlist", 1);
+  build();
 }
 
 void launch_batch_step(const BatchLaunch& L, cudaStream_t st, cudaGraphConditionalHandle h,
@@ -1045,8 +1178,9 @@ void launch_batch_step(const BatchLaunch& L, cudaStream_t st, cudaGraphCondition
     if (!L.step_n[v]) return;
     auto* kern = kb_step_nl<N16, CU, CA>;
     const unsigned r = resident_blocks(128 + v, (const void*)kern, 256);
-    kern<<<L.step_n[v] < r ? L.step_n[v] : r, 256, 0, st>>>(L.T, L.part + L.step_off[v], L.step_n[v], h, use_cond,
-                                                            L.act_n);
+    kern<<<L.step_n[v] < r ? L.step_n[v] : r, 256, 0, st>>>(
+        L.T, L.part + L.step_off[v], L.step_n[v], h, use_cond, L.act_n, L.buckets ? L.act : nullptr,
+        make_uint4(0u, L.n_part + L.n_cell, L.n_part + L.n_cell + L.n_tile + L.n_one, 0u));
   };
   using T_ = std::true_type;
   using F_ = std::false_type;
@@ -1059,18 +1193,35 @@ void launch_batch_step(const BatchLaunch& L, cudaStream_t st, cudaGraphCondition
 // its family in turn.  (A block per entry of the full map, returning at once
 // beyond the compacted count, costs ~18 us per kernel at 13,400 entries, most
 // of what a rebuild of the few members that need one takes.)
+//
+// Where every member's cells have buckets the step kernel lists the blocks and
+// four kernels follow; else the plan and nine.
 void launch_batch_rebuild(const BatchLaunch& L, cudaStream_t st) {
+  auto grid = [](int v, const void* k, unsigned n) {
+    const unsigned r = resident_blocks(v, k, 256);
+    return n < r ? n : r;
+  };
+  int per = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kb_build_nlist, L.build_threads, L.build_smem) != cudaSuccess ||
+      per < 1) {
+    cudaGetLastError();
+    per = 1;
+  }
+  const unsigned rb = device_sms() * (unsigned)per, gb = L.n_build < rb ? L.n_build : rb;
+  if (L.buckets) {
+    const BlkMap *tile = L.act + L.n_part + L.n_cell, *build = tile + L.n_tile + L.n_one;
+    kb_keys_bucket<<<grid(144, (const void*)kb_keys_bucket, L.n_part), 256, 0, st>>>(L.T, L.act, L.act_n);
+    kb_scan_direct<<<grid(145, (const void*)kb_scan_direct, L.n_tile), 256, 0, st>>>(L.T, tile, L.act_n);
+    kb_permute_bucket<<<grid(146, (const void*)kb_permute_bucket, L.n_part), 256, 0, st>>>(L.T, L.act, L.act_n);
+    kb_build_nlist<<<gb, L.build_threads, L.build_smem, st>>>(L.T, build, L.act_n + 3, L.act_n);
+    return;
+  }
   const uint32_t o1 = L.n_part, o2 = o1 + L.n_cell, o3 = o2 + L.n_tile, o4 = o3 + L.n_one;
   const uint32_t n_all = o4 + L.n_build;
   kb_rebuild_plan<<<blocks_for(n_all, 256), 256, 0, st>>>(L.T, L.part, make_uint4(o1, o2, o3, o4), n_all,
                                                            L.act, L.act_n);
   const BlkMap *part = L.act, *cell = L.act + o1, *tile = L.act + o2, *one = L.act + o3, *build = L.act + o4;
-  const uint32_t *c_part = L.act_n, *c_cell = L.act_n + 1, *c_tile = L.act_n + 2, *c_one = L.act_n + 3,
-                 *c_build = L.act_n + 4;
-  auto grid = [](int v, const void* k, unsigned n) {
-    const unsigned r = resident_blocks(v, k, 256);
-    return n < r ? n : r;
-  };
+  const uint32_t *c_part = L.act_n, *c_cell = L.act_n + 1, *c_tile = L.act_n + 2, *c_one = L.act_n + 3;
   kb_rebin_clear<<<grid(136, (const void*)kb_rebin_clear, L.n_cell), 256, 0, st>>>(L.T, cell, c_cell);
   kb_rebin_keys<<<grid(137, (const void*)kb_rebin_keys, L.n_part), 256, 0, st>>>(L.T, part, c_part);
   kb_scan_tiles<<<grid(138, (const void*)kb_scan_tiles, L.n_tile), 256, 0, st>>>(L.T, tile, c_tile);
@@ -1079,14 +1230,7 @@ void launch_batch_rebuild(const BatchLaunch& L, cudaStream_t st) {
   kb_rebin_scatter<<<grid(141, (const void*)kb_rebin_scatter, L.n_part), 256, 0, st>>>(L.T, part, c_part);
   kb_rebin_cellsort<<<grid(142, (const void*)kb_rebin_cellsort, L.n_cell), 256, 0, st>>>(L.T, cell, c_cell);
   kb_rebin_permute<<<grid(143, (const void*)kb_rebin_permute, L.n_part), 256, 0, st>>>(L.T, part, c_part);
-  int per = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kb_build_nlist, L.build_threads, L.build_smem) != cudaSuccess ||
-      per < 1) {
-    cudaGetLastError();
-    per = 1;
-  }
-  const unsigned r = device_sms() * (unsigned)per;
-  kb_build_nlist<<<L.n_build < r ? L.n_build : r, L.build_threads, L.build_smem, st>>>(L.T, build, c_build);
+  kb_build_nlist<<<gb, L.build_threads, L.build_smem, st>>>(L.T, build, L.act_n + 4, nullptr);
 }
 
 int batch_rebuild_kernel_count() { return 10; }

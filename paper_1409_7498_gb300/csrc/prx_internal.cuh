@@ -39,7 +39,8 @@ constexpr uint32_t SLOT_MASK = 0x7FFFFFFFu;
 constexpr int STEP_THREADS = 128;
 constexpr int RX_THREADS = 256;
 constexpr int TILE_Y_MAX = 8;  // cell rows per tile of the list build
-constexpr unsigned ENG_BUCKET = 16;    // slots per cell bucket of the persistent runs
+constexpr unsigned ENG_BUCKET = 16;    // slots per cell bucket
+constexpr unsigned BUCKET_CELLS = 131072;  // cells up to which a system has buckets
 constexpr unsigned ENG_CELLS = 32768;  // cells up to which a block scans all counts itself
 constexpr int SCAN_TILE = 2048;  // elements per scan tile (256 threads x 8)
 
@@ -183,8 +184,8 @@ struct Sys {
   float rv2_build;                // (r_c + skin + rounding margin)^2, list build test (FP32)
   // list-build tiling (cells of edge >= r_c + skin)
   int tile_y, tiles_y, tile_threads, tile_cap;
-  // persistent runs of small systems: buckets of the cells (ENG_BUCKET slots
-  // each), tiles of their list build (rows, staged entries, slots)
+  // buckets of the cells (ENG_BUCKET slots each; nullptr: rebuilds sort without
+  // them); tiles of the persistent runs' list build (rows, staged entries, slots)
   uint32_t* bucket;
   int eng_ty, eng_tiles_y, eng_cap, eng_slots;
   unsigned long long inv_nc64[2];  // ceil(2^64 / nc) for y and z
@@ -364,6 +365,7 @@ struct BatchLaunch {
   // force cap; the blocks of variant v are part[step_off[v] .. + step_n[v])
   unsigned step_off[8], step_n[8];
   bool any_nearest;  // a member has the nearest-partner rule
+  bool buckets;      // every member rebuilds through buckets
 };
 
 // ---- host-side launchers (defined in the kernel translation units) ----------

@@ -277,6 +277,14 @@ void free_list(std::vector<void*>& l) {
   l.clear();
 }
 
+// Entries of the cells' buckets: none where cells hold so many particles that
+// buckets would overflow, where there are far more cells than particles, or
+// more cells than the paths that use buckets take.
+uint64_t bucket_slots(uint64_t n, uint64_t ncell) {
+  return (double)n <= 6.0 * (double)ncell && ncell <= std::min<uint64_t>(2 * n + ENG_CELLS, BUCKET_CELLS)
+             ? ncell * ENG_BUCKET : 0;
+}
+
 // Grid, fixed-point constants and Verlet-list layout for list cutoff rc
 // (the larger of the WCA and reaction cutoffs):
 //   list radius r_v = rc + skin; cells of edge >= r_v (only used to build the
@@ -342,8 +350,10 @@ int setup_grid(prx_system* sys, double rc) {
   S.nl16 = S.n <= 65535 ? 1 : 0;
   A.add((uint8_t**)&S.nl, (size_t)S.list_cap * S.n * (S.nl16 ? 2 : 4));
   A.add(&S.nn, (size_t)S.n);
-  A.add(&S.bucket, ncell <= (long long)ENG_CELLS ? (size_t)ncell * ENG_BUCKET : 0);
+  const size_t nbucket = bucket_slots(S.n, (uint64_t)ncell);
+  A.add(&S.bucket, nbucket);
   if ((rc2 = A.commit(sys, sys->grid_allocs))) return rc2;
+  if (!nbucket) S.bucket = nullptr;
   // the cell counters are zero outside rebuilds
   CK(cudaMemsetAsync(S.count, 0, sizeof(uint32_t) * (((size_t)ncell + 3) & ~(size_t)3), sys->stream));
   CK(cudaMemsetAsync(S.fill, 0, sizeof(uint32_t) * (size_t)ncell, sys->stream));
@@ -1082,6 +1092,8 @@ int batch_prepare(prx_batch* b) {
   L.act = b->maps + nmaps;
   L.act_n = b->act_n;
   L.any_nearest = false;
+  L.buckets = true;
+  for (const Sys& m : table) L.buckets = L.buckets && m.bucket;
   for (const Sys& m : table) L.any_nearest = L.any_nearest || (m.has_rx && m.R.rule == PRX_SELECT_NEAREST);
   for (int v = 0; v < 8; ++v) {
     L.step_off[v] = step_off[v];
@@ -1168,7 +1180,7 @@ uint64_t estimate_bytes(const prx_system_desc& d, double r_react) {
   const uint64_t allocs = 40;  // separate cudaMalloc calls, each rounded up
   return 2 * per_set + n * (2 * 16 + 4 * 4) + (n * cap / 2 + 1) * sizeof(prx_bond) +
            (kHistCap + 2ull) * sizeof(prx_history_record) + sizeof(Ctl) + 32 * (n / RX_THREADS + 2) +
-           32 * n + ncell * 12 + (ncell <= ENG_CELLS ? ncell * 4 * ENG_BUCKET : 0) + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + 8 * (2 * kMaxBins + 3) + allocs * 4096;
+           32 * n + ncell * 12 + 4 * bucket_slots(n, ncell) + 8 * nblk + list_cap * n * nl_bytes + 2 * n + 16384 + 8 * (2 * kMaxBins + 3) + allocs * 4096;
 }
 
 
