@@ -663,27 +663,36 @@ __device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4
   long long unused = 0;
   if (R.rule != PRX_SELECT_NEAREST && R.nr <= 1) {
     rx_find_random4<NL16>(S, Blk{0u, 1u}, B, P, step, list, nact, unused, unused);
-  } else if (R.rule == PRX_SELECT_NEAREST) {
-    for (uint32_t w = threadIdx.x; w < nact; w += ENG_THREADS)
-      S.win[list[w]] = nearest_partner<NL16>(S, B, P, list[w], true, unused);
-    for (uint32_t i = lo + threadIdx.x; i < hi; i += ENG_THREADS)
-      if (in_window(R.mask_T, R.t_lo, R.t_hi, B.type[i], B.state[i]))
-        S.win[i] = nearest_partner<NL16>(S, B, P, i, false, unused);
   } else {
-    for (uint32_t w = threadIdx.x; w < nact; w += ENG_THREADS) {
-      uint32_t ch = 0u;
-      const uint32_t i = list[w];
-      S.win[i] = rx_find_multi<NL16>(S, B, P, step, i, unused, unused, ch);
-      S.wch[i] = (uint8_t)ch;
+    for (uint32_t wb = (threadIdx.x & ~31u) / RX_GROUP; wb < nact; wb += ENG_THREADS / RX_GROUP) {
+      const uint32_t w = wb + (uint32_t)lane / RX_GROUP;
+      const bool valid = w < nact;
+      const uint32_t i = valid ? list[w] : 0u;
+      uint32_t best = NONE, ch = 0u;
+      if (R.rule == PRX_SELECT_NEAREST) best = nearest_partner<NL16, RX_GROUP>(S, B, P, i, valid, true, unused);
+      else best = rx_find_multi<NL16>(S, B, P, step, i, valid, unused, unused, ch);
+      if (valid && lane % RX_GROUP == 0) {
+        if (R.nr > 1) S.wch[i] = (uint8_t)ch;
+        S.win[i] = best;
+      }
+    }
+    if (R.rule == PRX_SELECT_NEAREST) {
+      for (uint32_t wb = lo + (threadIdx.x & ~31u) / RX_GROUP; wb < hi; wb += ENG_THREADS / RX_GROUP) {
+        const uint32_t i = wb + (uint32_t)lane / RX_GROUP;
+        const bool valid = i < hi && in_window(R.mask_T, R.t_lo, R.t_hi, B.type[i], B.state[i]);
+        if (!__any_sync(0xFFFFFFFFu, valid)) continue;
+        const uint32_t best = nearest_partner<NL16, RX_GROUP>(S, B, P, i, valid, false, unused);
+        if (valid && lane % RX_GROUP == 0) S.win[i] = best;
+      }
     }
   }
   if (bar.sync(false) == 2) return 2;
-  for (uint32_t base = 0; base < nact; base += ENG_THREADS) {
-    const uint32_t w = base + threadIdx.x;
+  for (uint32_t wb = (threadIdx.x & ~31u) / RX_GROUP; wb < nact; wb += ENG_THREADS / RX_GROUP) {
+    const uint32_t w = wb + (uint32_t)lane / RX_GROUP;
+    const uint32_t i = w < nact ? list[w] : 0u;
     bool unused_w;
-    const uint32_t i = w < nact ? list[w] : NONE;
-    const uint32_t T = w < nact ? rx_decide<NL16>(S, B, step, i, unused_w) : NONE;
-    (void)rx_form(S, B, step, i, T, dpop);
+    const uint32_t T = rx_decide<NL16>(S, B, step, i, w < nact, unused_w);
+    (void)rx_form(S, B, step, i, lane % RX_GROUP == 0 ? T : NONE, dpop);
   }
   __syncthreads();
   int32_t* rep = S.pop + (size_t)(b % POP_REPLICAS) * (PRX_MAX_TYPES * PRX_MAX_STATES);

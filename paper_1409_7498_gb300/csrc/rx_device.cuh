@@ -32,17 +32,23 @@ __device__ __forceinline__ uint32_t nl_get_rx(const Sys& S, int k, uint32_t i) {
 // LAMMPS rule (Sec. IV.A): the eligible partner of the other kind (a T when
 // want_T, else an A) within r_react of slot i, not bonded to it, of smallest
 // exact r^2 (ties to the smaller id); `in_range` counts the pairs in range.
-template <bool NL16>
+// The G lanes of a group share a slot, lane q its list entries q, q + G, ...:
+// with RX_GROUP lanes the chain of dependent loads (entry -> position -> type)
+// runs once per slot instead of once per entry.  Called by whole warps unless
+// G = 1; lanes of a group without a slot pass valid = false.
+constexpr int RX_GROUP = 16;
+template <bool NL16, int G>
 __device__ __forceinline__ uint32_t nearest_partner(const Sys& S, const SoA& B, const uint4* P,
-                                                    uint32_t i, bool want_T, long long& in_range) {
+                                                    uint32_t i, bool valid, bool want_T, long long& in_range) {
   const RxParams& R = S.R;
+  i = valid ? i : 0u;
   const uint4 pi = P[i];
   const double xi = B.x[i], yi = B.y[i], zi = B.z[i];
   const uint32_t nb = B.nadj[i];
   uint32_t best = NONE, bestid = 0u;
   double best_r2 = 0.0;
-  const int cnt = S.nn[i];
-  for (int k = 0; k < cnt; ++k) {
+  const int cnt = valid ? S.nn[i] : 0;
+  for (int k = (int)(threadIdx.x & (G - 1)); k < cnt; k += G) {
     const uint32_t j = nl_get_rx<NL16>(S, k, i);
     // distance prefilter first (as in the random rule's search)
     const uint4 pj = P[j];
@@ -67,6 +73,16 @@ __device__ __forceinline__ uint32_t nearest_partner(const Sys& S, const SoA& B, 
       best = j;
       best_r2 = r2;
       bestid = idj;
+    }
+  }
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) {
+    const double r2 = __shfl_xor_sync(0xFFFFFFFFu, best_r2, o);
+    const uint32_t id = __shfl_xor_sync(0xFFFFFFFFu, bestid, o), j = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+    if (j != NONE && (best == NONE || r2 < best_r2 || (r2 == best_r2 && id < bestid))) {
+      best = j;
+      best_r2 = r2;
+      bestid = id;
     }
   }
   return best;
@@ -96,20 +112,21 @@ __device__ __forceinline__ void rx_accept_and_key(const Sys& S, const SoA& B,
 // reaction's windows, exact FP64 r^2 below the reaction's cutoff, not
 // bonded), one acceptance draw against the cumulative bounds of m, and the
 // retained pair of smallest selection key.  `ch` receives the chosen pair's
-// reaction.
+// reaction.  A group of RX_GROUP lanes per A, as in nearest_partner.
 template <bool NL16>
 __device__ __forceinline__ uint32_t rx_find_multi(const Sys& S, const SoA& B, const uint4* P,
-                                                  unsigned long long step, uint32_t i,
+                                                  unsigned long long step, uint32_t i, bool valid,
                                                   long long& ncand, long long& nret, uint32_t& ch) {
   const RxParams& R = S.R;
+  i = valid ? i : 0u;
   const uint32_t elA = rx_elig_A(R, B.type[i], B.state[i]);
   const uint4 pi = P[i];
   const uint32_t idi = B.id[i];
   const uint32_t nb = B.nadj[i];
   uint32_t best = NONE, bestid = 0u;
   unsigned long long bestkey = 0ull;
-  const int cnt = S.nn[i];
-  for (int k = 0; k < cnt; ++k) {
+  const int cnt = valid ? S.nn[i] : 0;
+  for (int k = (int)(threadIdx.x & (RX_GROUP - 1)); k < cnt; k += RX_GROUP) {
     const uint32_t j = nl_get_rx<NL16>(S, k, i);
     const uint4 pj = P[j];
     const float ex = __int2float_rn(pdiff(pj.x, pi.x)) * S.scale[0];
@@ -147,6 +164,18 @@ __device__ __forceinline__ uint32_t rx_find_multi(const Sys& S, const SoA& B, co
       bestkey = key;
       bestid = idj;
       ch = (uint32_t)c;
+    }
+  }
+#pragma unroll
+  for (int o = RX_GROUP / 2; o > 0; o >>= 1) {
+    const unsigned long long key = __shfl_xor_sync(0xFFFFFFFFu, bestkey, o);
+    const uint32_t id = __shfl_xor_sync(0xFFFFFFFFu, bestid, o), j = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+    const uint32_t c = __shfl_xor_sync(0xFFFFFFFFu, ch, o);
+    if (j != NONE && (best == NONE || key < bestkey || (key == bestkey && id < bestid))) {
+      best = j;
+      bestkey = key;
+      bestid = id;
+      ch = c;
     }
   }
   return best;
@@ -253,46 +282,47 @@ __device__ __forceinline__ void rx_find_random4(const Sys& S, const Blk blk, con
   }
 }
 
-// Steps 6-7 for one eligible A: the T it keeps (NONE: none); `winner` tells
-// whether it had picked one (random rule) or its choice was mutual (nearest).
+// Steps 6-7 for one eligible A (a group of RX_GROUP lanes, as in
+// nearest_partner): the T it keeps (NONE: none), the same in every lane of the
+// group; `winner` tells whether it had picked one (random rule) or its choice
+// was mutual (nearest).
 template <bool NL16>
 __device__ __forceinline__ uint32_t rx_decide(const Sys& S, const SoA& B, unsigned long long step,
-                                              uint32_t i, bool& winner) {
+                                              uint32_t i, bool valid, bool& winner) {
   const RxParams& R = S.R;
-  const uint32_t T = S.win[i];
+  const uint32_t T = valid ? S.win[i] : NONE;
   winner = false;
-  if (T == NONE) return NONE;
   if (R.rule == PRX_SELECT_NEAREST) {
     // LAMMPS rule: an A and the T it picked react when the T picked it too
     // and u < k dt Theta, drawn with the pair's smaller id first
-    if (S.win[T] != i) return NONE;
+    if (T == NONE || S.win[T] != i) return NONE;
     winner = true;
     const uint32_t ida = B.id[i], idt = B.id[T];
     const uint4 w = keyed_draw(S.seed, step, min(ida, idt), max(ida, idt), TAG_NEAREST);
     return u53_below(w.x, w.y, R.p53) ? T : NONE;
   }
-  winner = true;
-  const uint32_t idi = B.id[i], idT = B.id[T];
-  const unsigned long long mine = key64(keyed_draw(S.seed, step, idT, idi, TAG_SEL_T));
-  bool keep = true;
-  const int cnt = S.nn[T];
-  // four list entries of T at a time (independent loads go out together)
-  for (int k0 = 0; k0 < cnt && keep; k0 += 4) {
-    uint32_t aa[4], wa[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) aa[u] = k0 + u < cnt ? nl_get_rx<NL16>(S, k0 + u, T) : i;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) wa[u] = S.win[aa[u]];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint32_t a = aa[u];
-      if (!keep || k0 + u >= cnt || a == i || wa[u] != T) continue;
-      const uint32_t ida = B.id[a];
-      const unsigned long long other = key64(keyed_draw(S.seed, step, idT, ida, TAG_SEL_T));
-      if (other < mine || (other == mine && ida < idi)) keep = false;
+  winner = T != NONE;
+  // the other A's that picked T are in T's list
+  bool lost = false;
+  const int cnt = winner ? S.nn[T] : 0;
+  uint32_t idi = 0u, idT = 0u;
+  unsigned long long mine = 0ull;
+  bool drawn = false;
+  for (int k = (int)(threadIdx.x & (RX_GROUP - 1)); k < cnt; k += RX_GROUP) {
+    const uint32_t a = nl_get_rx<NL16>(S, k, T);
+    if (a == i || S.win[a] != T) continue;
+    if (!drawn) {
+      idi = B.id[i], idT = B.id[T];
+      mine = key64(keyed_draw(S.seed, step, idT, idi, TAG_SEL_T));
+      drawn = true;
     }
+    const uint32_t ida = B.id[a];
+    const unsigned long long other = key64(keyed_draw(S.seed, step, idT, ida, TAG_SEL_T));
+    lost |= other < mine || (other == mine && ida < idi);
   }
-  return keep ? T : NONE;
+  const unsigned any = __ballot_sync(0xFFFFFFFFu, lost);
+  const unsigned group = ((1u << RX_GROUP) - 1u) << ((threadIdx.x & 31u) & ~(RX_GROUP - 1u));
+  return winner && !(any & group) ? T : NONE;
 }
 
 // Step 9 for the pairs (i, T) of a warp (T = NONE: none), called by the whole

@@ -132,25 +132,27 @@ __device__ __forceinline__ void rx_find_body(const Sys& S, const Blk blk, long l
   const SoA B = ctl->set ? S.s1 : S.s0;
   const uint4* P = ctl->phase ? S.P1 : S.P0;
   const uint32_t nact = ctl->n_active;
-  // four lanes per eligible A (random rule) or one: blocks past them have nothing to do
+  // four lanes per eligible A (random rule) or a group: blocks past them have nothing to do
   const bool four = R.rule != PRX_SELECT_NEAREST && R.nr <= 1;
-  if (blk.b * (four ? blockDim.x / 4u : blockDim.x) >= nact) return;
+  if (blk.b * (blockDim.x / (four ? 4u : (unsigned)RX_GROUP)) >= nact) return;
   long long ncand = 0, nret = 0;
   if (four) {
     rx_find_random4<NL16>(S, blk, B, P, step, S.tmp, nact, ncand, nret);
   } else {
-    // the nearest rule and concurrent reactions: one thread per eligible A
-    for (uint32_t w = blk.b * blockDim.x + threadIdx.x; w < nact; w += blk.nb * blockDim.x) {
-      const uint32_t i = S.tmp[w];
-      uint32_t best = NONE;
-      if (R.rule == PRX_SELECT_NEAREST) {
-        best = nearest_partner<NL16>(S, B, P, i, true, ncand);
-      } else {
-        uint32_t ch = 0u;
-        best = rx_find_multi<NL16>(S, B, P, step, i, ncand, nret, ch);
-        S.wch[i] = (uint8_t)ch;
+    // the nearest rule and concurrent reactions: a group of lanes per eligible A
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t wb = (blk.b * blockDim.x + (threadIdx.x & ~31u)) / RX_GROUP; wb < nact;
+         wb += blk.nb * blockDim.x / RX_GROUP) {
+      const uint32_t w = wb + lane / RX_GROUP;
+      const bool valid = w < nact;
+      const uint32_t i = valid ? S.tmp[w] : 0u;
+      uint32_t best = NONE, ch = 0u;
+      if (R.rule == PRX_SELECT_NEAREST) best = nearest_partner<NL16, RX_GROUP>(S, B, P, i, valid, true, ncand);
+      else best = rx_find_multi<NL16>(S, B, P, step, i, valid, ncand, nret, ch);
+      if (valid && lane % RX_GROUP == 0u) {
+        if (R.nr > 1) S.wch[i] = (uint8_t)ch;
+        S.win[i] = best;
       }
-      S.win[i] = best;
     }
   }
   const long long c = block_sum_ll(ncand);
@@ -186,7 +188,7 @@ __device__ __forceinline__ void rx_find_T_body(const Sys& S, const Blk blk) {
   const uint32_t i = blk.b * blockDim.x + threadIdx.x;
   if (i >= S.n || !in_window(R.mask_T, R.t_lo, R.t_hi, B.type[i], B.state[i])) return;
   long long unused = 0;
-  S.win[i] = nearest_partner<NL16>(S, B, P, i, false, unused);
+  S.win[i] = nearest_partner<NL16, 1>(S, B, P, i, true, false, unused);
 }
 
 template <bool NL16>
@@ -221,24 +223,24 @@ __device__ __forceinline__ void rx_select_apply_body(const Sys& S, const Blk blk
   const uint32_t nact = ctl->n_active;
   // blocks past the eligible A's have nothing to do; the last of the others
   // (of the first, when there is no A) writes the record
-  const uint32_t busy = max(1u, min(blk.nb, (nact + blockDim.x - 1u) / blockDim.x));
+  const uint32_t per = blockDim.x / RX_GROUP;  // A's per block and pass
+  const uint32_t busy = max(1u, min(blk.nb, (nact + per - 1u) / per));
   if (blk.b >= busy) return;
   long long nwin = 0, nfin = 0;
   // population changes of this block's bonds, per (type, state)
   __shared__ int32_t dpop[PRX_MAX_TYPES * PRX_MAX_STATES];
   for (int k = threadIdx.x; k < PRX_MAX_TYPES * PRX_MAX_STATES; k += blockDim.x) dpop[k] = 0;
   __syncthreads();
-  // block-strided over the eligible A's, warp-uniform trip count
-  for (uint32_t base = blk.b * blockDim.x; base < nact; base += blk.nb * blockDim.x) {
-    const uint32_t w = base + threadIdx.x;
-    uint32_t i = NONE, T = NONE;
-    if (w < nact) {
-      i = S.tmp[w];
-      bool winner;
-      T = rx_decide<NL16>(S, B, step, i, winner);
-      nwin += winner ? 1 : 0;
-    }
-    nfin += rx_form(S, B, step, i, T, dpop) ? 1 : 0;
+  // block-strided over the eligible A's (a group of lanes each), warp-uniform
+  // trip count
+  for (uint32_t base = blk.b * per; base < nact; base += blk.nb * per) {
+    const uint32_t w = base + threadIdx.x / RX_GROUP;
+    const bool first = threadIdx.x % RX_GROUP == 0u;
+    const uint32_t i = w < nact ? S.tmp[w] : 0u;
+    bool winner;
+    const uint32_t T = rx_decide<NL16>(S, B, step, i, w < nact, winner);
+    nwin += winner && first ? 1 : 0;
+    nfin += rx_form(S, B, step, i, first ? T : NONE, dpop) ? 1 : 0;
   }
   const long long cw = block_sum_ll(nwin);
   const long long cf = block_sum_ll(nfin);
