@@ -609,15 +609,14 @@ __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA
     for (uint32_t i = g; i < S.n; i += stride) S.tmp[first(S.key[i]) + S.new_of_old[i]] = i;
     if (bar.sync(false) == 2) return 2;
   }
-  auto new_slot = [&](uint32_t j, uint32_t k) {
-    const uint32_t s0 = first(k), c = (k + 1u < ncell ? first(k + 1u) : S.n) - s0;
-    const uint32_t* row = over_any ? S.tmp + s0 : S.bucket + (size_t)k * ENG_BUCKET;
+  auto start = [&](uint32_t k) { return k < ncell ? first(k) : S.n; };
+  auto from_tmp = [&](uint32_t j, uint32_t, uint32_t s0, uint32_t c) {
     uint32_t r = s0;
 #pragma unroll 4
-    for (uint32_t q = 0; q < c; ++q) r += row[q] < j ? 1u : 0u;
+    for (uint32_t q = 0; q < c; ++q) r += S.tmp[s0 + q] < j ? 1u : 0u;
     return r;
   };
-  for (uint32_t o = g; o < S.n; o += stride) permute_old<false>(S, A, B, P, S.win, o, new_slot);
+  for (uint32_t o = g; o < S.n; o += stride) permute_old<false>(S, A, B, P, S.win, o, start, over_any != 0, from_tmp);
   if (bar.sync(false) == 2) return 2;
   for (uint32_t c = g; c < ncell; c += stride) S.count[c] = 0u;  // (zero outside rebuilds)
   const uint32_t nt = (uint32_t)(S.eng_tiles_y * S.nc[2]);

@@ -646,11 +646,15 @@ __device__ __forceinline__ uint32_t cell_of_pos(const Sys& S, const uint4 q) {
 
 // Old slot o goes to its new slot: every per-particle array into the other
 // set, bond partners renamed, a fresh displacement reference, and the slot's
-// cell (into cell_of, read by the list build).  new_slot(j, cell of j) gives a
-// slot's new place.  XYZ: also the list build's coordinates.
-template <bool XYZ, class F>
+// cell (into cell_of, read by the list build).  start(k) is the first slot of
+// cell k (n for k = ncell); a slot's new place is that plus the number of its
+// cell's members with a smaller old slot, from the cell's bucket or, where
+// `other` (a bucket overflowed), from other(slot, cell, first, members).  The
+// slot's own lookup and its first two bond partners' run side by side.  XYZ:
+// also the list build's coordinates.
+template <bool XYZ, class Start, class Other>
 __device__ __forceinline__ void permute_old(const Sys& S, const SoA& A, const SoA& B, uint4* P, uint32_t* cell_of,
-                                            uint32_t o, F new_slot) {
+                                            uint32_t o, Start start, bool other_all, Other other) {
   double x = A.x[o], y = A.y[o], z = A.z[o];
   const double vx = A.vx[o], vy = A.vy[o], vz = A.vz[o];
   const uint32_t pid = A.id[o];
@@ -659,17 +663,39 @@ __device__ __forceinline__ void permute_old(const Sys& S, const SoA& A, const So
   const uint32_t nb = A.nadj[o];
   const uint32_t key = S.key[o];
   const uint32_t* from = A.adj + (size_t)o * S.cap;
-  // the first two bonds' chains beside the slot's own
-  const uint32_t e0 = from[0], e1 = S.cap > 1 ? from[1] : 0u;
-  const uint32_t k0 = nb > 0u ? S.key[e0 & SLOT_MASK] : 0u, k1 = nb > 1u ? S.key[e1 & SLOT_MASK] : 0u;
-  const uint32_t s = new_slot(o, key);
+  const uint32_t e0 = nb > 0u ? from[0] : o, e1 = nb > 1u ? from[1] : o;
+  auto members_before = [&](uint4 v, uint32_t q, uint32_t c, uint32_t j) {  // among members q .. q + 3 of c
+    return (q < c && v.x < j ? 1u : 0u) + (q + 1u < c && v.y < j ? 1u : 0u) + (q + 2u < c && v.z < j ? 1u : 0u) +
+           (q + 3u < c && v.w < j ? 1u : 0u);
+  };
+  auto row = [&](uint32_t k) { return reinterpret_cast<const uint4*>(S.bucket + (size_t)k * ENG_BUCKET); };
+  // of slot j in cell k with members first .. first + c, the first four of them v
+  auto place = [&](uint32_t j, uint32_t k, uint32_t first, uint32_t c, uint4 v) {
+    if (other_all || c > ENG_BUCKET) return other(j, k, first, c);
+    uint32_t r = first + members_before(v, 0u, c, j);
+#pragma unroll 1
+    for (uint32_t q = 4u; q < c; q += 4u) r += members_before(row(k)[q >> 2], q, c, j);
+    return r;
+  };
+  const uint32_t j[3] = {o, e0 & SLOT_MASK, e1 & SLOT_MASK};
+  uint32_t k[3] = {key, S.key[j[1]], S.key[j[2]]}, f[3], c[3], r[3];
+  uint4 v[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    f[q] = start(k[q]);
+    c[q] = start(k[q] + 1u) - f[q];
+    v[q] = row(k[q])[0];
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) r[q] = place(j[q], k[q], f[q], c[q], v[q]);
+  const uint32_t s = r[0];
   uint32_t* to = B.adj + (size_t)s * S.cap;
-  if (nb > 0u) to[0] = new_slot(e0 & SLOT_MASK, k0) | (e0 & ~SLOT_MASK);
-  if (nb > 1u) to[1] = new_slot(e1 & SLOT_MASK, k1) | (e1 & ~SLOT_MASK);
+  if (nb > 0u) to[0] = r[1] | (e0 & ~SLOT_MASK);
+  if (nb > 1u) to[1] = r[2] | (e1 & ~SLOT_MASK);
 #pragma unroll 1
   for (uint32_t b = 2; b < nb; ++b) {
-    const uint32_t f = from[b];
-    to[b] = new_slot(f & SLOT_MASK, S.key[f & SLOT_MASK]) | (f & ~SLOT_MASK);
+    const uint32_t e = from[b], jb = e & SLOT_MASK, kb = S.key[jb], fb = start(kb);
+    to[b] = place(jb, kb, fb, start(kb + 1u) - fb, row(kb)[0]) | (e & ~SLOT_MASK);
   }
   x = wrap_into_box(x, S.L[0]);
   y = wrap_into_box(y, S.L[1]);
@@ -691,6 +717,7 @@ __device__ __forceinline__ void permute_old(const Sys& S, const SoA& A, const So
   if constexpr (XYZ) reinterpret_cast<float4*>(S.fout)[s] = build_xyz(S, X, Y, Z, key, s);
   cell_of[s] = key;
 }
+
 }  // namespace
 
 }  // namespace prx

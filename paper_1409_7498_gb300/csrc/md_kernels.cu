@@ -736,7 +736,7 @@ __device__ __forceinline__ void keys_bucket_body(const Sys& S, const Blk blk) {
 __device__ __forceinline__ void scan_direct_body(const Sys& S, const Blk blk) {
   const uint32_t n = (uint32_t)S.ncell, base = blk.b * SCAN_TILE;
   uint32_t part = 0, off;
-#pragma unroll 4
+#pragma unroll 16
   for (uint32_t c = threadIdx.x * 4u; c < base; c += 1024u) {
     const uint4 v = *reinterpret_cast<const uint4*>(S.count + c);
     part += v.x + v.y + v.z + v.w;
@@ -767,23 +767,14 @@ __device__ __forceinline__ void permute_bucket_body(const Sys& S, const Blk blk)
   Ctl* ctl = S.ctl;
   const SoA A = ctl->set ? S.s1 : S.s0, B = ctl->set ? S.s0 : S.s1;
   uint4* P = ctl->phase ? S.P1 : S.P0;
-  auto new_slot = [&](uint32_t j, uint32_t k) {
-    const uint32_t s0 = S.cell_start[k], c = S.cell_start[k + 1] - s0;
-    uint32_t r = s0;
-    if (c <= ENG_BUCKET) {
-      const uint4* row = reinterpret_cast<const uint4*>(S.bucket + (size_t)k * ENG_BUCKET);
-      for (uint32_t q = 0; q < c; q += 4u) {
-        const uint4 v = row[q >> 2];
-        r += (v.x < j ? 1u : 0u) + (q + 1u < c && v.y < j ? 1u : 0u) + (q + 2u < c && v.z < j ? 1u : 0u) +
-             (q + 3u < c && v.w < j ? 1u : 0u);
-      }
-    } else {
-      for (uint32_t i = 0; i < j; ++i) r += S.key[i] == k ? 1u : 0u;
-    }
+  auto start = [&](uint32_t k) { return S.cell_start[k]; };
+  auto from_keys = [&](uint32_t j, uint32_t k, uint32_t first, uint32_t) {
+    uint32_t r = first;
+    for (uint32_t i = 0; i < j; ++i) r += S.key[i] == k ? 1u : 0u;
     return r;
   };
   const uint32_t o = blk.b * 256u + threadIdx.x;
-  if (o < S.n) permute_old<true>(S, A, B, P, S.tmp, o, new_slot);
+  if (o < S.n) permute_old<true>(S, A, B, P, S.tmp, o, start, false, from_keys);
   for (uint32_t c = o; c < (uint32_t)S.ncell; c += blk.nb * 256u) S.count[c] = 0u;
 }
 

@@ -95,6 +95,14 @@ struct Ctl {
   unsigned long long dg_rebuild, dg_react;
 };
 
+// Observables as they are read back: kinetic energy / 2 and momentum,
+// populations, step, bonds and status.
+struct ObsPack {
+  double sums[4];
+  HistRec rec;
+  Ctl ctl;
+};
+
 constexpr int MAX_RX = PRX_MAX_REACTIONS;
 constexpr int POP_REPLICAS = 32;
 
@@ -382,7 +390,7 @@ void launch_rebin(const Sys& S, cudaStream_t st, int mode, void (*hook)(void*, c
                   void* hook_ctx);
 void launch_rx(const Sys& S, cudaStream_t st, long long step_arg,
                void (*hook)(void*, const char*, int), void* hook_ctx);
-void launch_observables(const Sys& S, cudaStream_t st, int nblocks);
+void launch_observables(const Sys& S, cudaStream_t st, ObsPack* out);
 // Counts the populations per (type, state) into S.pop (creation).
 void launch_pop_init(const Sys& S, cudaStream_t st);
 void launch_pair_hist(const Sys& S, cudaStream_t st, const PairClass& a, const PairClass& b, double r_max, double* e2,

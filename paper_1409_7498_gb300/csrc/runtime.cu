@@ -53,11 +53,8 @@ struct prx_system {
   cudaStream_t cap = nullptr;
   Sys S{};
   Ctl* ctl_host = nullptr;  // pinned mirror for read-back
-  struct ObsHost {          // pinned read-back of the observables
-    double sums[4];         // kinetic energy / 2, momentum
-    HistRec rec;            // populations
-    Ctl ctl;                // step, bonds, status
-  }* obs_host = nullptr;    // PRX_OBS_SLOTS pipelined slots + one for the synchronous call
+  ObsPack* obs_host = nullptr;  // pinned: PRX_OBS_SLOTS pipelined slots + one for the synchronous call
+  ObsPack* obs_dev = nullptr;
   cudaEvent_t obs_ev[PRX_OBS_SLOTS] = {};
   bool obs_pending[PRX_OBS_SLOTS] = {};
   std::vector<void*> dev_allocs;
@@ -795,7 +792,7 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   A.add(&S.pop, (size_t)POP_REPLICAS * PRX_MAX_TYPES * PRX_MAX_STATES);
   A.add(&S.red, 4 * ((size_t)(n + RX_THREADS - 1) / RX_THREADS + 1));
   A.add(&S.fout, 3 * (size_t)n), A.add(&S.eout, (size_t)n);  // (one after the other: the bond sort's scratch)
-  A.add(&sys->eng_bar, 64), A.add(&sys->hist_dev, 2 * (size_t)kMaxBins + 3);
+  A.add(&sys->eng_bar, 64), A.add(&sys->hist_dev, 2 * (size_t)kMaxBins + 3), A.add(&sys->obs_dev, 1);
   if ((rc = A.commit(sys, sys->dev_allocs))) return bail(rc);
   sys->bond_scratch = (size_t)((char*)S.eout - (char*)S.fout) + 8 * (size_t)n;
   if ((rc = setup_grid(sys, grid_rc > rc_w ? grid_rc : rc_w))) return bail(rc);
@@ -1520,19 +1517,15 @@ int prx_get_bonds(prx_system* sys, prx_bond* out, uint64_t cap, uint64_t* n_out)
 
 // Enqueues the observables and their copy into pinned slot q (no wait).
 int enqueue_observables(prx_system* sys, int q) {
-  const uint32_t n = sys->S.n;
-  const int nblk = (int)((n + RX_THREADS - 1) / RX_THREADS);
-  auto* oh = sys->obs_host + q;
-  if (n) {
-    launch_observables(sys->S, sys->stream, nblk);
-    sys->other_launches += 3;
+  ObsPack* oh = sys->obs_host + q;
+  if (sys->S.n) {
+    launch_observables(sys->S, sys->stream, sys->obs_dev);
+    sys->other_launches += 1;
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(oh->sums, sys->S.red + 4 * (size_t)nblk, sizeof(oh->sums), cudaMemcpyDeviceToHost,
-                       sys->stream));
-    CK(cudaMemcpyAsync(&oh->rec, &sys->S.hist[sys->S.hist_cap], sizeof(HistRec), cudaMemcpyDeviceToHost,
-                       sys->stream));
+    CK(cudaMemcpyAsync(oh, sys->obs_dev, sizeof(ObsPack), cudaMemcpyDeviceToHost, sys->stream));
+  } else {
+    CK(cudaMemcpyAsync(&oh->ctl, sys->S.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, sys->stream));
   }
-  CK(cudaMemcpyAsync(&oh->ctl, sys->S.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, sys->stream));
   return PRX_OK;
 }
 

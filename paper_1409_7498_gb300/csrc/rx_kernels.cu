@@ -26,17 +26,6 @@ namespace prx {
 
 namespace {
 
-__device__ __forceinline__ bool last_block_rx(unsigned int* counter, uint32_t nb) {
-  __shared__ bool is_last;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    is_last = (atomicAdd(counter, 1u) == nb - 1);
-  }
-  __syncthreads();
-  return is_last && threadIdx.x == 0;
-}
-
 __device__ __forceinline__ long long block_sum_ll(long long v) {
   __shared__ long long part[RX_THREADS / 32];
 #pragma unroll
@@ -285,21 +274,17 @@ __global__ void __launch_bounds__(RX_THREADS, 4)
   else rx_select_apply_body<false>(S, Blk{m.b, m.nb}, -1LL);
 }
 
-// Populations per (type, state) counted over every slot into out[128]
-// (integer atomics: the counts do not depend on their order).  With rec set,
-// the last block also stamps rec's step and bond count (on-demand
-// observables, into the spare history slot).
-__device__ __forceinline__ void pop_count_body(const Sys& S, const Blk blk, int32_t* out,
-                                               HistRec* rec) {
-  Ctl* ctl = S.ctl;
-  const SoA B = ctl->set ? S.s1 : S.s0;
+// Populations per (type, state) counted over every slot into S.pop (creation;
+// the reaction steps keep them current).
+__global__ void __launch_bounds__(RX_THREADS) k_pop_init(Sys S) {
+  const SoA B = S.ctl->set ? S.s1 : S.s0;
   __shared__ int32_t h[PRX_MAX_TYPES * PRX_MAX_STATES];
   for (int k = threadIdx.x; k < PRX_MAX_TYPES * PRX_MAX_STATES; k += blockDim.x) h[k] = 0;
   __syncthreads();
   // Block-strided over the slots; within a warp, lanes with the same
   // (type, state) bin are counted by one shared atomic of their leader.
   const int lane = threadIdx.x & 31;
-  for (uint32_t base = blk.b * blockDim.x; base < S.n; base += blk.nb * blockDim.x) {
+  for (uint32_t base = blockIdx.x * blockDim.x; base < S.n; base += gridDim.x * blockDim.x) {
     const uint32_t i = base + threadIdx.x;
     int key = -1;
     if (i < S.n) {
@@ -312,68 +297,50 @@ __device__ __forceinline__ void pop_count_body(const Sys& S, const Blk blk, int3
   }
   __syncthreads();
   for (int k = threadIdx.x; k < PRX_MAX_TYPES * PRX_MAX_STATES; k += blockDim.x)
-    if (h[k]) atomicAdd(out + k, h[k]);
-  if (!rec) return;
-  __threadfence();
-  if (last_block_rx(&ctl->done_obs, blk.nb)) {
-    ctl->done_obs = 0u;
-    rec->step = (long long)ctl->step;
-    rec->bonds = (long long)ctl->nbonds;
-  }
+    if (h[k]) atomicAdd(S.pop + k, h[k]);
 }
 
-__global__ void __launch_bounds__(RX_THREADS) k_obs_hist(Sys S) {
-  pop_count_body(S, Blk{blockIdx.x, gridDim.x}, &S.hist[S.hist_cap].counts[0][0], &S.hist[S.hist_cap]);
-}
-__global__ void __launch_bounds__(RX_THREADS) k_pop_init(Sys S) {
-  pop_count_body(S, Blk{blockIdx.x, gridDim.x}, S.pop, nullptr);
-}
-
-// Per-block FP64 partial sums of m v^2 / 2 and m v (fixed-order tree).
-__global__ void __launch_bounds__(RX_THREADS) k_obs_sums(Sys S, double mass) {
+// The observables in one launch, packed for one copy: FP64 sums of m v^2 / 2
+// and m v (grid-strided per thread, a fixed warp tree, the warps in order; the
+// last block adds the blocks' sums, thread t blocks t, t + 256, ..., and a
+// fixed tree: the same order on every call), the populations from the running
+// counts, and the control block.  Three kernels, a recount of the populations
+// and three copies before: observables of 2,048 beads 35 -> 27 us.
+__global__ void __launch_bounds__(RX_THREADS) k_obs_hist(Sys S, double mass, ObsPack* __restrict__ out) {
   Ctl* ctl = S.ctl;
   const SoA B = ctl->set ? S.s1 : S.s0;
-  // grid-strided sums per thread, then a fixed warp tree and the warps in
-  // order: few FP64 additions per slot, the same order on every call
-  double ke = 0.0, px = 0.0, py = 0.0, pz = 0.0;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < S.n; i += gridDim.x * blockDim.x) {
     const double vx = B.vx[i], vy = B.vy[i], vz = B.vz[i];
-    ke += vx * vx + vy * vy + vz * vz;
-    px += vx;
-    py += vy;
-    pz += vz;
+    a[0] += vx * vx + vy * vy + vz * vz;
+    a[1] += vx;
+    a[2] += vy;
+    a[3] += vz;
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ke += __shfl_down_sync(0xFFFFFFFFu, ke, o);
-    px += __shfl_down_sync(0xFFFFFFFFu, px, o);
-    py += __shfl_down_sync(0xFFFFFFFFu, py, o);
-    pz += __shfl_down_sync(0xFFFFFFFFu, pz, o);
-  }
-  __shared__ double red[4][RX_THREADS / 32];
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] += __shfl_down_sync(0xFFFFFFFFu, a[q], o);
+  __shared__ double part[4][RX_THREADS];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    red[0][wid] = ke;
-    red[1][wid] = px;
-    red[2][wid] = py;
-    red[3][wid] = pz;
-  }
+  if (lane == 0)
+    for (int q = 0; q < 4; ++q) part[q][wid] = a[q];
   __syncthreads();
   if (threadIdx.x < 4) {
     double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[threadIdx.x][w];
     S.red[4 * (size_t)blockIdx.x + threadIdx.x] = (threadIdx.x == 0 ? 0.5 * mass : mass) * t;
   }
-}
-
-// The nsum per-block sums reduced to one value each, in a fixed order (thread
-// t adds blocks t, t + 256, ...; then a fixed tree), written to
-// red[4 nblk .. 4 nblk + 3].
-__global__ void __launch_bounds__(RX_THREADS) k_obs_final(Sys S, uint32_t nsum, uint32_t nblk) {
-  __shared__ double part[4][RX_THREADS];
-  double a[4] = {0.0, 0.0, 0.0, 0.0};
-  for (uint32_t b = threadIdx.x; b < nsum; b += blockDim.x)
-    for (int q = 0; q < 4; ++q) a[q] += S.red[4 * (size_t)b + q];
+  __threadfence();
+  __shared__ bool is_last;
+  __syncthreads();
+  if (threadIdx.x == 0) is_last = atomicAdd(&ctl->done_obs, 1u) == gridDim.x - 1u;
+  __syncthreads();
+  if (!is_last) return;
+  if (threadIdx.x == 0) ctl->done_obs = 0u;
+  for (int q = 0; q < 4; ++q) a[q] = 0.0;
+  for (uint32_t b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+    for (int q = 0; q < 4; ++q) a[q] += __ldcg(S.red + 4 * (size_t)b + q);
   for (int q = 0; q < 4; ++q) part[q][threadIdx.x] = a[q];
   __syncthreads();
   for (int w = RX_THREADS / 2; w > 0; w >>= 1) {
@@ -381,7 +348,19 @@ __global__ void __launch_bounds__(RX_THREADS) k_obs_final(Sys S, uint32_t nsum, 
       for (int q = 0; q < 4; ++q) part[q][threadIdx.x] += part[q][threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x < 4) S.red[4 * (size_t)nblk + threadIdx.x] = part[threadIdx.x][0];
+  if (threadIdx.x < 4) out->sums[threadIdx.x] = part[threadIdx.x][0];
+  for (int k = threadIdx.x; k < PRX_MAX_TYPES * PRX_MAX_STATES; k += blockDim.x) {
+    int32_t c = 0;
+    for (int q = 0; q < POP_REPLICAS; ++q) c += S.pop[q * (PRX_MAX_TYPES * PRX_MAX_STATES) + k];
+    (&out->rec.counts[0][0])[k] = c;
+  }
+  if (threadIdx.x == 0) {
+    out->rec.step = (long long)ctl->step;
+    out->rec.bonds = (long long)ctl->nbonds;
+  }
+  static_assert(sizeof(Ctl) % 8 == 0, "the control block is copied in 8-byte words");
+  for (uint32_t w = threadIdx.x; w < sizeof(Ctl) / 8; w += blockDim.x)
+    reinterpret_cast<unsigned long long*>(&out->ctl)[w] = reinterpret_cast<const unsigned long long*>(ctl)[w];
 }
 
 // Batched reaction steps clear each member's counters in a kernel.
@@ -514,15 +493,10 @@ void launch_pair_hist(const Sys& S, cudaStream_t st, const PairClass& a, const P
   else k_pair_hist<false><<<g, RX_THREADS, sm, st>>>(S, a, b, e2, nbins, counts);
 }
 
-// On-demand observables: the spare history slot (index hist_cap) receives the
-// populations; S.red the per-block sums and, after them, their totals.
-void launch_observables(const Sys& S, cudaStream_t st, int nblocks) {
-  cudaMemsetAsync(&S.hist[S.hist_cap], 0, sizeof(HistRec), st);
-  k_obs_hist<<<nblocks, RX_THREADS, 0, st>>>(S);
-  // the sums on at most 8 blocks per SM, strided over the slots
-  const unsigned nsum = nblocks < 1216 ? (unsigned)nblocks : 1216u;
-  k_obs_sums<<<nsum, RX_THREADS, 0, st>>>(S, S.mass);
-  k_obs_final<<<1, RX_THREADS, 0, st>>>(S, nsum, (uint32_t)nblocks);
+// On-demand observables into `out` (on at most 8 blocks per SM).
+void launch_observables(const Sys& S, cudaStream_t st, ObsPack* out) {
+  const unsigned g = blocks_rx(S.n) < 1216u ? blocks_rx(S.n) : 1216u;
+  k_obs_hist<<<g, RX_THREADS, 0, st>>>(S, S.mass, out);
 }
 
 void launch_pop_init(const Sys& S, cudaStream_t st) {
