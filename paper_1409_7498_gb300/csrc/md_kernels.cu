@@ -58,8 +58,17 @@ __device__ __forceinline__ void step_done(const Sys& S, int ph, unsigned long lo
   ctl->phase = ph ^ 1;
   ctl->step = step;
   if (!S.in_batch) {
+    const int dg = ctl->dg_on;  // (loads side by side)
+    const unsigned long long left = ctl->steps_left - 1ull;
+    const unsigned int until = S.has_rx ? ctl->until_rx - 1u : 1u;
     const int flag = atomicAdd(&ctl->rebin_flag, 0);
     if (use_cond) cudaGraphSetConditional(cond, flag ? 1u : 0u);
+    if (dg) {  // device-driven run (dg.cu): whether another step may follow at once
+      ctl->steps_left = left;
+      ctl->until_rx = until ? until : S.theta;
+      ctl->rx_due = !until;
+      ctl->hold = flag || !until || !left;
+    }
   } else {
     __threadfence();
     if (atomicAdd(&S.batch->done_step, 1u) == S.n_members - 1) {
@@ -87,11 +96,12 @@ template <bool NL16, bool FORCES_ONLY, bool CUBIC, bool CAP, int BT>
 __global__ void __launch_bounds__(BT, 1536 / BT)
     k_step_nl(Sys S, cudaGraphConditionalHandle cond, int use_cond) {
   __shared__ unsigned int warps_left;
+  Ctl* ctl = S.ctl;
+  const int hold = ctl->hold, ph = ctl->phase;
+  const unsigned long long step = ctl->step + 1ull;
+  if (hold) return;  // (dg.cu; the same for every block)
   if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
   __syncthreads();
-  Ctl* ctl = S.ctl;
-  const int ph = ctl->phase;
-  const unsigned long long step = ctl->step + 1ull;
   const uint4* __restrict__ P = ph ? S.P1 : S.P0;
   uint4* __restrict__ Pn = ph ? S.P0 : S.P1;
   const uint32_t W = gridDim.x * (blockDim.x >> 5);
@@ -120,11 +130,12 @@ template <bool NL16, bool FORCES_ONLY, bool CUBIC, int BT>
 __global__ void __launch_bounds__(BT, 1536 / BT)
     k_step_nl4(Sys S, cudaGraphConditionalHandle cond, int use_cond) {
   __shared__ unsigned int warps_left;
+  Ctl* ctl = S.ctl;
+  const int hold = ctl->hold, ph = ctl->phase;
+  const unsigned long long step = ctl->step + 1ull;
+  if (hold) return;  // (dg.cu; the same for every block)
   if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
   __syncthreads();
-  Ctl* ctl = S.ctl;
-  const int ph = ctl->phase;
-  const unsigned long long step = ctl->step + 1ull;
   const uint4* __restrict__ P = ph ? S.P1 : S.P0;
   uint4* __restrict__ Pn = ph ? S.P0 : S.P1;
   const uint32_t W = gridDim.x * (blockDim.x >> 5);
@@ -279,7 +290,9 @@ constexpr int F64_LANES = 4;
 template <bool NL16, bool ENERGY>
 __global__ void __launch_bounds__(32) k_forces64(Sys S) {
   Ctl* ctl = S.ctl;
-  const SoA B = ctl->set ? S.s1 : S.s0;
+  const int hold = ctl->hold, set = ctl->set;
+  if (hold) return;  // (dg.cu)
+  const SoA B = set ? S.s1 : S.s0;
   const int lane = threadIdx.x & 31, q = lane & (F64_LANES - 1);
   const uint32_t i = blockIdx.x * (32 / F64_LANES) + (uint32_t)(lane / F64_LANES);
   double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
@@ -329,12 +342,12 @@ __global__ void __launch_bounds__(32) k_forces64(Sys S) {
 __global__ void __launch_bounds__(STEP_THREADS)
     k_integrate64(Sys S, cudaGraphConditionalHandle cond, int use_cond) {
   __shared__ unsigned int warps_left;
+  Ctl* ctl = S.ctl;
+  const int hold = ctl->hold, set = ctl->set, ph = ctl->phase;
+  const unsigned long long step = ctl->step + 1ull;
+  if (hold) return;  // (dg.cu; the same for every block)
   if (threadIdx.x == 0) warps_left = blockDim.x >> 5;
   __syncthreads();
-  Ctl* ctl = S.ctl;
-  const int set = ctl->set;
-  const int ph = ctl->phase;
-  const unsigned long long step = ctl->step + 1ull;
   const SoA B = set ? S.s1 : S.s0;
   const uint4* __restrict__ P = ph ? S.P1 : S.P0;
   uint4* __restrict__ Pn = ph ? S.P0 : S.P1;

@@ -74,12 +74,15 @@ static_assert(sizeof(HistRec) == sizeof(prx_history_record), "history record lay
 struct Ctl {
   int set;                  // current SoA set
   int phase;                // current off buffer
+  int hold;                 // (dg.cu) further steps of this graph return at once: a rebuild
+                            // or a reaction step comes first, or the run is done
   int rebin_flag;           // a particle left its extended cell
   int status;               // sticky PRX_E* status (0 = ok)
   unsigned int done_step;   // last-block counters
   unsigned int done_rebin;
   unsigned int done_rx;
   unsigned int done_obs;
+  int dg_on;                // a device-driven run (dg.cu) is in progress
   unsigned long long step;  // completed MD steps
   unsigned long long rebins;
   unsigned long long reactions;
@@ -89,10 +92,12 @@ struct Ctl {
   unsigned int n_active;       // eligible A's of the current reaction step
   unsigned int input_err;      // creation: first bad input kind (1 non-finite
                                // position, 2 outside the box, 3 type >= 8)
-  // device-driven runs (dg.cu): steps left in the run, and the device graphs
-  // k_dg_next launches (as cudaGraphExec_t values)
+  // device-driven runs (dg.cu): steps left in the run, the device graphs
+  // k_dg_next launches (as cudaGraphExec_t values), and the k_dg_next run so far
   unsigned long long steps_left;
-  unsigned long long dg_rebuild, dg_react;
+  unsigned long long dg_rebuild, dg_react, dg_runs;
+  int rx_due;                  // a reaction step follows
+  unsigned int until_rx;       // steps to the next one
 };
 
 // Observables as they are read back: kinetic energy / 2 and momentum,
@@ -230,6 +235,7 @@ struct Sys {
   // reaction scheme (has_rx = 0: none)
   RxParams R;
   int has_rx;
+  unsigned int theta;       // its reaction interval
   // batch membership: in_batch = 1 inside a batched launch; batch = the
   // batch's control block
   int in_batch;
@@ -428,7 +434,7 @@ cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint3
 // last kernel of the step's device graph, tail-launches what follows.
 void launch_dg_arm(const Sys& S, cudaStream_t st, unsigned long long steps,
                    unsigned long long rebuild, unsigned long long react);
-void launch_dg_next(const Sys& S, cudaStream_t st, unsigned int theta);
+void launch_dg_next(const Sys& S, cudaStream_t st);
 // The same for a batch: k_dgb_next follows the batch's step kernels.
 void launch_dgb_arm(BatchCtl* c, cudaStream_t st, unsigned long long steps, unsigned long long phase,
                     unsigned long long theta, int any_rx, unsigned long long rebuild,

@@ -68,9 +68,11 @@ struct prx_system {
   cudaGraphExec_t g_step = nullptr, g_chunk = nullptr, g_react = nullptr;
   cudaGraphExec_t g_chunk1 = nullptr;  // one interval, when g_chunk holds several
   uint32_t chunk_m = 1;                // reaction intervals per g_chunk replay
-  // device graphs of device-driven runs (dg.cu): one step (+ k_dg_next), the
-  // rebuild, the reaction; dg_ok when all three instantiated
-  cudaGraphExec_t dg_step = nullptr, dg_rebuild = nullptr, dg_react = nullptr;
+  // device graphs of device-driven runs (dg.cu): the steps (+ k_dg_next), the
+  // rebuild, the reaction; dg_ok when all three instantiated.  dg_one holds
+  // one step, for runs shorter than dg_step's (made when first needed).
+  cudaGraphExec_t dg_step = nullptr, dg_rebuild = nullptr, dg_react = nullptr, dg_one = nullptr;
+  uint32_t dg_steps = 1;  // steps in dg_step
   bool dg_ok = false;
   bool graphs_valid = false;
   // persistent runs (engine.cu): the barrier words, the plan (once asked
@@ -264,7 +266,8 @@ void destroy_graphs(prx_system* s) {
   if (s->dg_step) cudaGraphExecDestroy(s->dg_step);
   if (s->dg_rebuild) cudaGraphExecDestroy(s->dg_rebuild);
   if (s->dg_react) cudaGraphExecDestroy(s->dg_react);
-  s->dg_step = s->dg_rebuild = s->dg_react = nullptr;
+  if (s->dg_one) cudaGraphExecDestroy(s->dg_one);
+  s->dg_step = s->dg_rebuild = s->dg_react = s->dg_one = nullptr;
   s->dg_ok = false;
   s->graphs_valid = false;
 }
@@ -536,15 +539,33 @@ cudaError_t capture_device_graph(cudaStream_t cap, F body, cudaGraphExec_t* out)
   return cudaGraphUpload(*out, cap);
 }
 
+// The step graph of a device-driven run, holding `steps` steps.
+cudaError_t build_dg_step(prx_system* sys, uint32_t steps, cudaGraphExec_t* out) {
+  return capture_device_graph(sys->cap, [&] {
+    for (uint32_t q = 0; q < steps; ++q)
+      launch_step(sys->S, sys->cap, sys->d.force_precision == PRX_FORCE_FP64, 0, 0, 0);
+    launch_dg_next(sys->S, sys->cap);
+  }, out);
+}
+
 // The device graphs of device-driven runs; on any failure the system keeps
 // the host-replayed graphs (the same kernels).
 void build_device_graphs(prx_system* sys) {
-  const bool fp64 = sys->d.force_precision == PRX_FORCE_FP64;
-  const unsigned theta = sys->has_rx ? (unsigned)sys->rxd.theta : 1u;
-  cudaError_t e = capture_device_graph(sys->cap, [&] {
-    launch_step(sys->S, sys->cap, fp64, 0, 0, 0);
-    launch_dg_next(sys->S, sys->cap, theta);
-  }, &sys->dg_step);
+  // Up to four steps per graph, so that the reaction interval divides into
+  // graphs of nearly equal length (10: 4 + 4 + 2; 5: 3 + 2; 1: one step, since
+  // every step is followed by a reaction step).  us per step with 1 / 2 / 3 /
+  // 4 / 8 steps per graph: 100,000 beads 22.98 / 21.33 / 20.75 / 20.76 / 20.61,
+  // 250,007 (reactions every 10 steps) 33.80 / 31.87 / 31.48 / 31.46 / 31.44,
+  // 1,000,000 (every 10) 87.32 / 85.36 / 84.82 / 84.48 / 84.42; longer graphs
+  // add more kernels that a rebuild in their middle turns into empty ones.
+  // In FP64 mode an empty force kernel costs ~1.4 us per 1,000 of its blocks of
+  // 8 slots: 20,000 beads 54.1 -> 52.2, but 100,000 188.1 -> 189.5, so that
+  // systems above 65,536 keep one step per graph.
+  const uint64_t most = sys->d.force_precision == PRX_FORCE_FP64 && sys->S.n > 65536 ? 1 : 4;
+  const uint64_t theta = sys->has_rx ? sys->S.theta : most;
+  const uint64_t graphs = (theta + most - 1) / most;
+  sys->dg_steps = (uint32_t)((theta + graphs - 1) / graphs);
+  cudaError_t e = build_dg_step(sys, sys->dg_steps, &sys->dg_step);
   if (e == cudaSuccess)
     e = capture_device_graph(sys->cap, [&] { launch_rebin(sys->S, sys->cap, 0, nullptr, nullptr); },
                              &sys->dg_rebuild);
@@ -1326,6 +1347,7 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
   }
   sys->has_rx = 1;
   sys->S.has_rx = 1;
+  sys->S.theta = rx->theta;
   destroy_graphs(sys);
   const double need = std::max(wca_rc(sys->d), rmax);
   if (need > sys->grid_rcut) {
@@ -1357,16 +1379,28 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
     // one device-driven chain of nsteps steps (with the rebuilds and the
     // reaction steps it decides on) behind one host launch
     if (nsteps == 0) return PRX_OK;
+    // a run shorter than the graph would end in empty step kernels (~2 us
+    // each): it takes the graph of one step
+    cudaGraphExec_t first = sys->dg_step;
+    if (nsteps < sys->dg_steps) {
+      if (!sys->dg_one && (build_dg_step(sys, 1, &sys->dg_one) != cudaSuccess ||
+                           cudaStreamSynchronize(sys->cap) != cudaSuccess)) {
+        cudaGetLastError();
+        if (sys->dg_one) cudaGraphExecDestroy(sys->dg_one);
+        sys->dg_one = nullptr;
+      }
+      if (sys->dg_one) first = sys->dg_one;
+    }
     launch_dg_arm(sys->S, sys->stream, nsteps, (unsigned long long)sys->dg_rebuild,
                   (unsigned long long)sys->dg_react);
-    CK(cudaGraphLaunch(sys->dg_step, sys->stream));
+    CK(cudaGraphLaunch(first, sys->stream));
     if (sys->has_rx) {
       const uint64_t th = sys->rxd.theta;
       sys->graph_rx_launches += (sys->host_step + nsteps) / th - sys->host_step / th;
     }
     sys->host_step += nsteps;
     sys->step_launches += nsteps;
-    sys->other_launches += 1 + nsteps;  // the arm kernel, one k_dg_next per step
+    sys->other_launches += 1;  // the arm kernel (k_dg_next counts itself)
     return PRX_OK;
   }
   const uint64_t theta = sys->has_rx ? sys->rxd.theta : (uint64_t)kNoRxChunk;
@@ -1644,7 +1678,8 @@ int prx_get_stats(prx_system* sys, prx_stats* out) {
   // sequence of kernels and increments the device counter once
   out->kernel_launches = sys->step_launches * (uint64_t)step_kernel_count(sys->d.force_precision) +
                          sys->ctl_host->rebins * (uint64_t)rebin_kernel_count(sys->S) +
-                         sys->graph_rx_launches * (uint64_t)rx_kernel_count(sys->S.R.rule) + sys->other_launches;
+                         sys->graph_rx_launches * (uint64_t)rx_kernel_count(sys->S.R.rule) + sys->ctl_host->dg_runs +
+                         sys->other_launches;
   for (int k = 0; k < 3; ++k) {
     out->cells[k] = (uint32_t)sys->S.nc[k];
     out->cell_edge[k] = sys->d.box[k] / sys->S.nc[k];
