@@ -149,7 +149,9 @@ typedef struct {
   uint64_t rebins;        /* neighbour-list rebuilds (sort + lists), including the first */
   uint64_t step_launches; /* step kernels run */
   uint64_t kernel_launches; /* all kernels run by this system so far; a phase of a
-                               persistent run counts as the kernel it stands for */
+                               persistent run counts as the kernel it stands for, and a
+                               step kernel that a device-driven run turned into an empty
+                               one (a rebuild or reaction step came first) not at all */
   uint32_t cells[3];      /* cell grid */
   double cell_edge[3];
 } prx_stats;
@@ -215,9 +217,9 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
  * system's stream and returns without waiting.  A run of a small system is
  * a few launches of a persistent kernel, each of some hundred steps with
  * their rebuilds and reaction steps; otherwise the run is one device-driven
- * chain: after each step a kernel on the GPU launches the list rebuild when
- * a particle moved more than skin/2, the reaction step when it is due, and
- * the next step (device graph launches); where device graphs are not
+ * chain of graphs of up to four steps, each ended by a kernel on the GPU that
+ * launches the list rebuild when a particle moved more than skin/2, the
+ * reaction step when it is due, and the next steps; where device graphs are not
  * available the library replays host-launched CUDA graphs with a
  * conditional rebuild node after each step instead, with the same kernels
  * and the same result. */
