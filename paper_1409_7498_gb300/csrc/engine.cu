@@ -42,6 +42,11 @@ constexpr int ENG_UNITS = 1024;  // (slot, layer) pairs per tile of the list bui
 // block reaches the word's next use only after every block has left the
 // other word's barrier, hence this one, so a count beyond the target cannot
 // be seen.  The words start a launch at zero.
+//
+// The arrival releases at GPU scope and every poll acquires, so that the wait
+// ends with the load that sees the target: 8.95 -> 8.52 us per step (33,096
+// beads), against relaxed polls with a fence after them (a second round trip),
+// whether that fence is __threadfence or fence.acq_rel.
 struct GroupBar {
   unsigned long long* w;
   int* res;  // shared: thread 0's verdict for the block
@@ -54,15 +59,13 @@ struct GroupBar {
     if (nb == 1u) return any;
     if (threadIdx.x == 0) {
       unsigned long long* p = w + (e & 1u) * 16u;
-      __threadfence();
-      atomicAdd(p, any ? 0x100000001ull : 1ull);
+      asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(any ? 0x100000001ull : 1ull) : "memory");
       const uint32_t target = (e / 2u + 1u) * nb;
       unsigned long long v;
       unsigned left = ENG_POLLS;
       do {
-        v = *(volatile unsigned long long*)p;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
       } while ((uint32_t)v != target && --left);
-      __threadfence();
       const uint32_t fl = (uint32_t)(v >> 32);
       const uint32_t before = (e & 1u) ? flags1 : flags0;
       *res = left ? (fl != before ? 1 : 0) : 2;
