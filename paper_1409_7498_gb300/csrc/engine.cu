@@ -876,11 +876,12 @@ static unsigned engine_resident(const void* k, size_t sm) {
 
 // Which runs go through the persistent kernel, by size (us per step, launch
 // chain -> persistent, step growth at density 0.85 on a GB300):
-//   FP32: 1,024 beads 18.8 -> 7.3, 16,384 21.1 -> 8.9, 33,000 21.3 -> 9.6,
-//   60,000 23.7 -> 13.4, 77,000 24.3 -> 16.1: up to one resident slot per
-//   thread of the GPU (77,824 with 152 SMs).
-//   FP64: 1,250 beads 30.1 -> 12.3, 5,000 34.5 -> 20.7, 10,000 40.2 -> 36.3,
-//   20,000 56.5 -> 58.5 (by then the FP64 pipe bounds both): up to 16,384.
+//   FP32: 1,024 beads 18.8 -> 6.5, 16,384 21.1 -> 7.7, 33,000 21.3 -> 9.1,
+//   60,000 23.7 -> 12.1, 77,000 24.3 -> 14.6 (the chain with four steps per
+//   graph takes 20.0 at 100,000): up to one resident slot per thread of the
+//   GPU (77,824 with 152 SMs).
+//   FP64: 1,250 beads 30.1 -> 11.3, 5,000 34.5 -> 19.6, 10,000 40.2 -> 35.2,
+//   20,000 53 -> 58 (by then the FP64 pipe bounds both): up to 16,384.
 // Runs with a force cap (warm-ups) and four-lane runs keep the launch chain,
 // as do boxes with more cells or longer rows than the rebuild holds.
 EngPlan engine_plan(const Sys& S, int fp64) {
