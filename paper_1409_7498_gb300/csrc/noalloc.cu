@@ -93,6 +93,10 @@ __device__ __forceinline__ bool na_bonded(const NaArgs& a, uint32_t i, uint32_t 
 // The particles a block searches for: NA_BLOCKS blocks share them in ranges.
 constexpr int NA_BLOCKS = 128, NA_THREADS = 1024, NA_WARPS = NA_THREADS / 32;
 constexpr int NA_RANGE = (PRX_NOALLOC_MAX_N + NA_BLOCKS - 1) / NA_BLOCKS;
+// strips of one particle per thread that a whole block takes in turn, a batch
+// of them at a time
+constexpr int NA_STRIPS = (PRX_NOALLOC_MAX_N + NA_THREADS - 1) / NA_THREADS, NA_BATCH = 4;
+static_assert(NA_STRIPS <= 32 && NA_STRIPS % NA_BATCH == 0 && NA_BATCH % 2 == 0, "strip masks");
 
 // binary64 -> binary32 towards zero on the integer pipe (error below 2^-23
 // of the value; values below 2^-126 become 0, beyond 2^128 or not finite a
@@ -113,7 +117,7 @@ __device__ __forceinline__ float na_f32(double x) {
 // of particles; the warps are shared out over the block's particles, so that
 // a few A's among many T's still keep all of them busy.  Bound by the FP32
 // instructions of the pair test (16 per pair) and the staging: a call with
-// 8,192 particles, 11% of them A, takes 102 us (one thread per particle and
+// 8,192 particles, 11% of them A, takes 92 us (one thread per particle and
 // FP64 tests of every pair: 11,900 us).  A coordinate more than a box edge outside the
 // box sends every pair to the exact test.
 __global__ void __launch_bounds__(NA_THREADS, 1) k_na_find(NaArgs a) {
@@ -138,20 +142,44 @@ __global__ void __launch_bounds__(NA_THREADS, 1) k_na_find(NaArgs a) {
     __syncthreads();
     if (threadIdx.x == 0) nstaged = nown = 0u, far = 0;
     __syncthreads();
-    for (uint32_t base = 0; base < a.n; base += NA_THREADS) {
-      const uint32_t j = base + threadIdx.x;
-      const bool el = j < a.n && (pass ? is_A(j) : is_T(j));
-      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, el);
+    // which of this thread's particles are of the partner's kind (types and
+    // states of four strips on their way at once), then their positions, two
+    // strips at a time
+    uint32_t kind = 0u;
+#pragma unroll 1
+    for (uint32_t u = 0; u * NA_THREADS < a.n; u += NA_BATCH) {
+#pragma unroll
+      for (int q = 0; q < NA_BATCH; ++q) {
+        const uint32_t j = (u + q) * NA_THREADS + threadIdx.x, jc = min(j, a.n - 1u);
+        const bool is = pass ? is_A(jc) : is_T(jc);
+        if (j < a.n && is) kind |= 1u << (u + q);
+      }
+    }
+#pragma unroll 1
+    for (uint32_t u = 0; u * NA_THREADS < a.n; u += 2) {
+      const bool el[2] = {((kind >> u) & 1u) != 0u, ((kind >> (u + 1u)) & 1u) != 0u};
+      double x[2][3];
+      uint32_t bal[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const double* pj = a.pos + 3 * (size_t)((u + q) * NA_THREADS + threadIdx.x);
+        if (el[q]) x[q][0] = pj[0], x[q][1] = pj[1], x[q][2] = pj[2];
+        bal[q] = __ballot_sync(0xFFFFFFFFu, el[q]);
+      }
       uint32_t at = 0u;
-      if (lane == 0 && bal) at = atomicAdd(&nstaged, (uint32_t)__popc(bal));
-      at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(bal & ((1u << lane) - 1u));
-      if (el) {
-        const double x = a.pos[3 * (size_t)j], y = a.pos[3 * (size_t)j + 1], z = a.pos[3 * (size_t)j + 2];
-        sx[at] = na_f32(x), sy[at] = na_f32(y), sz[at] = na_f32(z);
-        sid[at] = (uint16_t)j;
-        // (also true for values that are not numbers)
-        if (!(fabsf(sx[at]) <= 2.f * a.Lf[0] && fabsf(sy[at]) <= 2.f * a.Lf[1] && fabsf(sz[at]) <= 2.f * a.Lf[2]))
-          far = 1;
+      if (lane == 0 && (bal[0] | bal[1])) at = atomicAdd(&nstaged, (uint32_t)(__popc(bal[0]) + __popc(bal[1])));
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (el[q]) {
+          const uint32_t e = at + __popc(bal[q] & ((1u << lane) - 1u));
+          sx[e] = na_f32(x[q][0]), sy[e] = na_f32(x[q][1]), sz[e] = na_f32(x[q][2]);
+          sid[e] = (uint16_t)((u + q) * NA_THREADS + threadIdx.x);
+          // (also true for values that are not numbers)
+          if (!(fabsf(sx[e]) <= 2.f * a.Lf[0] && fabsf(sy[e]) <= 2.f * a.Lf[1] && fabsf(sz[e]) <= 2.f * a.Lf[2]))
+            far = 1;
+        }
+        at += __popc(bal[q]);
       }
     }
     for (uint32_t i = lo + threadIdx.x; i < hi; i += NA_THREADS)
@@ -266,69 +294,93 @@ __global__ void __launch_bounds__(256) k_na_select(NaArgs a) {
   }
 }
 
-// Step 9 in one block: bonds appended in ascending id of A (a running count
-// over the ids, no atomics), adjacency rows and states updated.  A pair that
-// would exceed a particle's valence forms no bond and takes no place in the
+// Step 9 in one block: bonds appended in ascending id of A (counts per strip
+// and warp, then their prefix sums), adjacency rows and states updated.  A pair
+// that would exceed a particle's valence forms no bond and takes no place in the
 // bond list (status PRX_ECAPACITY); the surviving pairs are all counted in
 // the trace, as prx_react_once counts them.  Each A and each T is in at most
 // one pair, so the valence reads see the rows as they were before this step.
-__global__ void k_na_apply(NaArgs a) {
-  __shared__ uint32_t wtot[32];
-  __shared__ uint32_t carry, surv;
-  if (threadIdx.x == 0) carry = surv = 0u;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (uint32_t base = 0; base < a.n; base += blockDim.x) {
-    const uint32_t i = base + threadIdx.x;
-    const uint32_t T = i < a.n ? a.sc->fin[i] : NONE;
-    bool has = false;
-    uint32_t na = 0, nt = 0;
-    if (T != NONE) {
-      const uint32_t ta = a.type[i], tt = a.type[T];
+// Bound by latency: strip by strip, each with its loads and three barriers, it
+// took 23.4 us for 8,192 particles; with the loads of four strips in flight and
+// one scan for them 12.7 us (all sixteen strips unrolled: 11.0, and 3 us
+// more for 1,000 particles, which only fetch the longer code).
+__global__ void __launch_bounds__(NA_THREADS, 1) k_na_apply(NaArgs a) {
+  __shared__ uint32_t before[NA_BATCH][NA_WARPS], total[NA_BATCH], pairs[NA_WARPS];
+  static_assert((PRX_MAX_TYPES & (PRX_MAX_TYPES - 1)) == 0, "a mask keeps the type in range");
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t np = 0u, carry = 0u;
+#pragma unroll 1
+  for (uint32_t base = 0; base < a.n; base += NA_BATCH * NA_THREADS) {
+    uint32_t T[NA_BATCH];
+    uint32_t bond[NA_BATCH];  // bit 31: forms; rank in the warp, the rows' lengths
+#pragma unroll
+    for (int u = 0; u < NA_BATCH; ++u) {
+      const uint32_t i = base + u * NA_THREADS + threadIdx.x;
+      T[u] = i < a.n ? a.sc->fin[i] : NONE;
+    }
+#pragma unroll
+    for (int u = 0; u < NA_BATCH; ++u) {
+      const bool pair = T[u] != NONE;
+      const uint32_t i = min(base + u * NA_THREADS + threadIdx.x, a.n - 1u), j = pair ? T[u] : i;
+      // (a pair's types are below 8; the others' values are not used)
+      const uint32_t ta = a.type[i] & (PRX_MAX_TYPES - 1), tt = a.type[j] & (PRX_MAX_TYPES - 1);
+      const uint32_t na = a.nadj[i], nt = a.nadj[j];
       const uint32_t capA = a.R.maxval[ta] < a.cap ? a.R.maxval[ta] : a.cap;
       const uint32_t capT = a.R.maxval[tt] < a.cap ? a.R.maxval[tt] : a.cap;
-      na = a.nadj[i];
-      nt = a.nadj[T];
-      has = na < capA && nt < capT;
-      if (!has) atomicCAS(&a.sc->status, 0, PRX_ECAPACITY);
+      const bool has = pair && na < capA && nt < capT;
+      if (pair && !has) atomicCAS(&a.sc->status, 0, PRX_ECAPACITY);
+      np += __popc(__ballot_sync(0xFFFFFFFFu, pair));
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, has);
+      bond[u] = has ? 0x80000000u | (uint32_t)__popc(bal & ((1u << lane) - 1u)) << 16 | nt << 8 | na : 0u;
+      if (lane == 0) before[u][wid] = __popc(bal);
     }
-    const uint32_t sbal = __ballot_sync(0xFFFFFFFFu, T != NONE);
-    if (lane == 0 && sbal) atomicAdd(&surv, __popc(sbal));
-    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, has);
-    if (lane == 0) wtot[wid] = __popc(bal);
     __syncthreads();
-    uint32_t before = carry;
-    for (int w = 0; w < wid; ++w) before += wtot[w];
-    const uint32_t pos = before + __popc(bal & ((1u << lane) - 1u));
-    if (has) {
-      if (pos >= a.bonds_cap) {
-        atomicCAS(&a.sc->status, 0, PRX_ECAPACITY);
-      } else {
-        const uint32_t sbit = a.R.style << 31;
-        a.adj[(size_t)i * a.cap + na] = T | sbit;
-        a.nadj[i] = (uint8_t)(na + 1);
-        a.adj[(size_t)T * a.cap + nt] = i | sbit;
-        a.nadj[T] = (uint8_t)(nt + 1);
-        a.state[i] = (int8_t)(a.state[i] + a.R.dA);
-        a.state[T] = (int8_t)(a.state[T] + a.R.dT);
-        prx_bond b;
-        b.a = i;
-        b.t = T;
-        b.step = (int64_t)a.step;
-        b.style = a.R.style;
-        b.reaction = 0u;
-        a.bonds[pos] = b;
+    if (wid < NA_BATCH) {
+      const uint32_t v = before[wid][lane];
+      uint32_t s = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t w = __shfl_up_sync(0xFFFFFFFFu, s, o);
+        if (lane >= o) s += w;
       }
+      before[wid][lane] = s - v;
+      if (lane == 31) total[wid] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t t = 0;
-      for (int w = 0; w < nw; ++w) t += wtot[w];
-      carry += t;
+#pragma unroll
+    for (int u = 0; u < NA_BATCH; ++u) {
+      if (bond[u]) {
+        const uint32_t i = base + u * NA_THREADS + threadIdx.x, j = T[u];
+        const uint32_t na = bond[u] & 0xFFu, nt = (bond[u] >> 8) & 0xFFu;
+        const uint32_t pos = carry + before[u][wid] + ((bond[u] >> 16) & 0x7FFFu);
+        if (pos >= a.bonds_cap) {
+          atomicCAS(&a.sc->status, 0, PRX_ECAPACITY);
+        } else {
+          const uint32_t sbit = a.R.style << 31;
+          a.adj[(size_t)i * a.cap + na] = j | sbit;
+          a.nadj[i] = (uint8_t)(na + 1);
+          a.adj[(size_t)j * a.cap + nt] = i | sbit;
+          a.nadj[j] = (uint8_t)(nt + 1);
+          a.state[i] = (int8_t)(a.state[i] + a.R.dA);
+          a.state[j] = (int8_t)(a.state[j] + a.R.dT);
+          prx_bond b;
+          b.a = i;
+          b.t = j;
+          b.step = (int64_t)a.step;
+          b.style = a.R.style;
+          b.reaction = 0u;
+          a.bonds[pos] = b;
+        }
+      }
+      carry += total[u];
     }
-    __syncthreads();
+    __syncthreads();  // (the counts' places serve the next batch)
   }
+  if (lane == 0) pairs[wid] = np;
+  __syncthreads();
   if (threadIdx.x == 0) {
+    uint32_t surv = 0u;
+    for (int w = 0; w < NA_WARPS; ++w) surv += pairs[w];
     const uint32_t formed = carry < a.bonds_cap ? carry : a.bonds_cap;
     a.sc->nbonds = formed;
     a.sc->trace[3] = surv;
@@ -442,7 +494,7 @@ extern "C" int prx_react_noalloc(const prx_reaction_desc* rx, const double* box,
     return PRX_ECUDA;
   k_na_find<<<NA_BLOCKS, NA_THREADS, (size_t)n * (3 * sizeof(float) + sizeof(uint16_t)), st>>>(a);
   k_na_select<<<NA_BLOCKS, 256, 0, st>>>(a);
-  k_na_apply<<<1, 1024, 0, st>>>(a);
+  k_na_apply<<<1, NA_THREADS, 0, st>>>(a);
   if (cudaGetLastError() != cudaSuccess) return PRX_ECUDA;
   if (cudaMemcpyAsync(&got, &sc->trace[0], sizeof(got), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
