@@ -30,7 +30,7 @@ __global__ void k_dg_arm(Ctl* ctl, unsigned long long steps, unsigned int theta,
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     ctl->steps_left = steps;
     ctl->until_rx = theta ? theta - (unsigned int)(ctl->step % theta) : 0u;
-    ctl->dg_on = 1;
+    ctl->dg_on = steps != 0ull;
     ctl->hold = ctl->rx_due = 0;
     ctl->dg_rebuild = rebuild;
     ctl->dg_react = react;

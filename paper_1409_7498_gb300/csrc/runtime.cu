@@ -1393,7 +1393,9 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
     }
     launch_dg_arm(sys->S, sys->stream, nsteps, (unsigned long long)sys->dg_rebuild,
                   (unsigned long long)sys->dg_react);
-    CK(cudaGraphLaunch(first, sys->stream));
+    const cudaError_t launched = cudaGraphLaunch(first, sys->stream);
+    if (launched != cudaSuccess) launch_dg_arm(sys->S, sys->stream, 0, 0, 0);  // no run in progress
+    CK(launched);
     if (sys->has_rx) {
       const uint64_t th = sys->rxd.theta;
       sys->graph_rx_launches += (sys->host_step + nsteps) / th - sys->host_step / th;
