@@ -31,9 +31,6 @@ namespace prx {
 namespace {
 
 constexpr int ENG_THREADS = 512;
-// polls of a barrier before it gives up (a few seconds): an error status
-// instead of a hang
-constexpr unsigned ENG_POLLS = 1u << 22;
 constexpr unsigned ENG_F64_MAX = 16384;  // particles of a persistent FP64 run
 constexpr int ENG_UNITS = 1024;  // (slot, layer) pairs per tile of the list build
 
@@ -51,6 +48,7 @@ struct GroupBar {
   unsigned long long* w;
   int* res;  // shared: thread 0's verdict for the block
   uint32_t nb, e, flags0, flags1;
+  uint32_t polls;  // of a barrier before it gives up
 
   // Waits for the whole group; 1 when a thread of any block raised `f`, 0
   // when none did, 2 when the wait ran out.
@@ -62,7 +60,7 @@ struct GroupBar {
       asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(any ? 0x100000001ull : 1ull) : "memory");
       const uint32_t target = (e / 2u + 1u) * nb;
       unsigned long long v;
-      unsigned left = ENG_POLLS;
+      unsigned left = polls;
       do {
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
       } while ((uint32_t)v != target && --left);
@@ -795,7 +793,9 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
       A.x[i] = B.x[i], A.y[i] = B.y[i], A.z[i] = B.z[i];
   }
   if (threadIdx.x == 0) {
-    if (bad) set_status(ctl, PRX_ETIMEOUT);
+    // over any earlier status: what a rebuild left half done (counters that are
+    // not zero, positions in the next set's order) must stop the later ones
+    if (bad) atomicExch(&ctl->status, PRX_ETIMEOUT);
     if (b == 0u) {
       ctl->set = set;
       ctl->phase = ph;
@@ -810,11 +810,17 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
 // follow one another on its stream).
 template <bool NL16, bool CUBIC, bool F64>
 __global__ void __launch_bounds__(ENG_THREADS, 1)
-    k_engine(Sys S, uint32_t nsteps, uint32_t theta, unsigned long long* bar, unsigned long long* bar_next) {
+    k_engine(Sys S, uint32_t nsteps, uint32_t theta, unsigned long long* bar, unsigned long long* bar_next,
+             uint32_t polls) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int res;
+  // a wait of an earlier launch ran out: nothing may build on what it left.
+  // (A block that reads the status of this launch's own timeout leaves early
+  // where the others already have.)
+  const int gone = S.ctl->status == PRX_ETIMEOUT;
+  if (__syncthreads_or(gone)) return;
   if (blockIdx.x == 0 && threadIdx.x < 2) bar_next[threadIdx.x * 16] = 0ull;
-  GroupBar gb{bar, &res, gridDim.x, 0u, 0u, 0u};
+  GroupBar gb{bar, &res, gridDim.x, 0u, 0u, 0u, polls};
   eng_run<NL16, CUBIC, F64>(S, blockIdx.x, gb, nsteps, theta, nullptr, smem);
 }
 
@@ -903,7 +909,8 @@ EngPlan engine_plan(const Sys& S, int fp64) {
 cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint32_t nsteps, uint32_t theta,
                           unsigned long long* bar, unsigned long long* bar_next) {
   Sys s = S;
-  void* args[] = {&s, &nsteps, &theta, &bar, &bar_next};
+  uint32_t polls = p.polls;
+  void* args[] = {&s, &nsteps, &theta, &bar, &bar_next, &polls};
   return cudaLaunchCooperativeKernel(p.kernel, dim3(p.blocks), dim3(ENG_THREADS), args, p.smem, st);
 }
 

@@ -41,8 +41,12 @@ __device__ __forceinline__ bool last_warp(unsigned int* counter, unsigned int* w
   return last;
 }
 
-// A particle moved more than skin/2: flag the system (and its batch).
+// A particle moved more than skin/2: flag the system (and its batch).  Not a
+// system whose persistent run timed out, which may have left its cell counters
+// and positions in the middle of a rebuild: its lists, old or new, name slots
+// below n and may be walked, but the next sort would place slots beyond n.
 __device__ __forceinline__ void raise_rebuild(const Sys& S) {
+  if (S.ctl->status == PRX_ETIMEOUT) return;
   atomicExch(&S.ctl->rebin_flag, 1);
   if (S.in_batch) atomicExch(&S.batch->any_rebuild, 1);
   __threadfence();

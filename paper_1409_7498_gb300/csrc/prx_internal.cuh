@@ -421,10 +421,14 @@ int configure_build_kernel(size_t smem_bytes);
 // Multiprocessors of the current device.
 unsigned device_sms();
 // Persistent runs (engine.cu).
+// Polls of a barrier before it gives up (a few seconds): an error status
+// instead of a hang.
+constexpr unsigned ENG_POLLS = 1u << 22;
 struct EngPlan {
   const void* kernel = nullptr;
   unsigned blocks = 0;  // 0: the system's runs do not go through a persistent kernel
   size_t smem = 0;
+  unsigned polls = 0;   // of a barrier before it gives up
 };
 EngPlan engine_plan(const Sys& S, int fp64);
 cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint32_t nsteps, uint32_t theta,
@@ -442,3 +446,10 @@ void launch_dgb_arm(BatchCtl* c, cudaStream_t st, unsigned long long steps, unsi
 void launch_dgb_next(BatchCtl* c, cudaStream_t st);
 
 }  // namespace prx
+
+// ---- for the tests only: exported, not part of the public interface ----------
+extern "C" {
+// Polls after which the barriers of the system's persistent runs give up
+// (at least 1; ENG_POLLS by default).
+int prx_test_wait_limit(prx_system* sys, uint32_t polls);
+}

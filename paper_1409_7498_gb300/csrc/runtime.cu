@@ -80,6 +80,7 @@ struct prx_system {
   unsigned long long* eng_bar = nullptr;
   EngPlan eng;
   bool eng_planned = false;
+  unsigned eng_polls = ENG_POLLS;
   uint64_t eng_launches = 0;
   size_t bond_scratch = 0;  // bytes of fout and eout together
   // pair histogram: squared bin edges, counts and class sizes; a pinned copy of
@@ -610,6 +611,7 @@ int ensure_graphs(prx_system* sys) {
 bool engine_fits(prx_system* sys) {
   if (!sys->eng_planned) {
     sys->eng = engine_plan(sys->S, sys->d.force_precision == PRX_FORCE_FP64);
+    sys->eng.polls = sys->eng_polls;
     sys->eng_planned = true;
   }
   return sys->eng.blocks > 0;
@@ -1204,6 +1206,12 @@ uint64_t estimate_bytes(const prx_system_desc& d, double r_react) {
 
 void free_slot(prx_batch* b, prx_system* sys);  // (defined with the batch entry points)
 
+// A system whose device wait ran out stays unusable (known once a call has
+// read its status; until then the kernels leave it as it is).
+int refuse_timed_out(prx_system* sys) {
+  return fail(sys, PRX_ETIMEOUT, "a device wait of this system timed out: its state is lost");
+}
+
 // Calls that would change a batch member on its own are refused.
 int refuse_member(prx_system* sys) {
   return fail(sys, PRX_EINVAL, "not allowed while the system is a member of a batch");
@@ -1361,6 +1369,7 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
 int prx_run(prx_system* sys, uint64_t nsteps) {
   if (!sys) return PRX_EINVAL;
   if (sys->batch) return refuse_member(sys);
+  if (sys->ctl_host->status == PRX_ETIMEOUT) return refuse_timed_out(sys);
   if (sys->S.n == 0) {
     sys->host_step += nsteps;
     return PRX_OK;
@@ -1427,6 +1436,13 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
       }
     }
   }
+  return PRX_OK;
+}
+
+int prx_test_wait_limit(prx_system* sys, uint32_t polls) {
+  if (!sys || polls < 1) return PRX_EINVAL;
+  sys->eng_polls = polls;
+  sys->eng_planned = false;
   return PRX_OK;
 }
 
@@ -2237,6 +2253,8 @@ int check_member(prx_batch* b, prx_system* sys) {
   if (sys->d.force_precision != PRX_FORCE_FP32)
     return bfail(b, PRX_EINVAL, "batches run PRX_FORCE_FP32 systems only");
   if (sys->profiling) return bfail(b, PRX_EINVAL, "system is being profiled");
+  if (sys->ctl_host->status == PRX_ETIMEOUT)
+    return bfail(b, PRX_ETIMEOUT, "a device wait of this system timed out: its state is lost");
   if (sys->S.step_lanes != 1)
     return bfail(b, PRX_EINVAL, "batch members run the one-lane step kernel (step_lanes 1)");
   if (sys->has_rx) {
