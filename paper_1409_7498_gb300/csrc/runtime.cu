@@ -1212,6 +1212,16 @@ int refuse_timed_out(prx_system* sys) {
   return fail(sys, PRX_ETIMEOUT, "a device wait of this system timed out: its state is lost");
 }
 
+// A run does not go into a caller's graph: what it queues (the device graphs,
+// the barrier words of a persistent launch, which the next launch clears) is
+// made for the one run that the host counts.
+int refuse_capture(prx_system* sys) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(sys->stream, &cs));
+  if (cs == cudaStreamCaptureStatusNone) return PRX_OK;
+  return fail(sys, PRX_ECUDA, "prx_run on a stream that is being captured into a CUDA graph");
+}
+
 // Calls that would change a batch member on its own are refused.
 int refuse_member(prx_system* sys) {
   return fail(sys, PRX_EINVAL, "not allowed while the system is a member of a batch");
@@ -1381,9 +1391,10 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
     }
     return PRX_OK;
   }
+  int rc;
+  if (nsteps && (rc = refuse_capture(sys))) return rc;
   if (engine_fits(sys)) return engine_run(sys, nsteps);
-  int rc = ensure_graphs(sys);
-  if (rc) return rc;
+  if ((rc = ensure_graphs(sys))) return rc;
   if (sys->dg_ok) {
     // one device-driven chain of nsteps steps (with the rebuilds and the
     // reaction steps it decides on) behind one host launch
