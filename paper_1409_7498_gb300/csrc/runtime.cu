@@ -360,14 +360,26 @@ int setup_grid(prx_system* sys, double rc) {
   CK(cudaMemsetAsync(S.fill, 0, sizeof(uint32_t) * (size_t)ncell, sys->stream));
   {
     // list-build tiling: the rows per tile (the rows of a layer shared out
-    // evenly) that keep most of the passes of 256 threads busy and restage
-    // few neighbour rows per particle, with four blocks per SM by shared
-    // memory.  us per list build with 1 / 2 / 3 / 4 / 5 / 8 rows: 130,000 beads
-    // 27.6 / 29.0 / 27.9 / 26.5 / 24.5 / 34.3, 500,000 beads 73.6 / 67.5 /
-    // 57.8 / 65.5 / 62.3 / 79.8, 1,048,576 beads 131 / 121 / 129 / 147 (1 to 4);
-    // the staging buffer holds all neighbour rows at once
+    // evenly).  While all tiles are resident at once or in two rounds, the build
+    // lasts as long as those rounds, each of as many passes as the fullest tiles'
+    // particles need (3% and six over the mean); with more rounds the tiles follow
+    // one another evenly, and restaging the neighbour rows counts as well.  The
+    // least rounds x passes + 0.00069 x (particles per SM) / rows is within 2% of
+    // the best of 1..8 rows on average over the twenty sizes measured (14% at
+    // worst; without a term for filling the SMs 17%, and 43% at 33,000 beads).
+    // us per list build with 1 / 2 / 3 / 4 / 5 / 8 rows: 33,000 beads 16.0 / 14.3 /
+    // 16.3 / 18.4 / 19.1 / 24.5, 80,000 20.4 / 20.4 / 22.5 / 22.5 / 22.8 / 26.3, 130,000
+    // 26.6 / 29.8 / 27.8 / 26.5 / 23.4 / 34.8, 500,000 beads 71.6 / 66.7 / 57.2 /
+    // 65.2 / 63.0 / 78.4, 1,048,576 beads 126 / 113 / 109 / 115 / 131 / 139; the
+    // staging buffer holds all neighbour rows at once
     const double per_row = (double)S.n / ((double)S.nc[1] * S.nc[2]);
     const double per_cell = (double)S.n / (double)ncell;
+    const double sms = (double)device_sms();
+    auto tile_threads = [&] {
+      const double mean = S.tile_y * per_row;
+      const int threads = (int)std::ceil((mean + 3.0 * std::sqrt(mean) + 16.0) / 32.0) * 32;
+      return std::max(64, std::min(256, threads));
+    };
     auto set_tiles = [&](int tiles) {
       S.tiles_y = tiles;
       S.tile_y = (S.nc[1] + tiles - 1) / tiles;  // the most rows of a tile
@@ -379,23 +391,26 @@ int setup_grid(prx_system* sys, double rc) {
       S.tile_cap = std::max(64, std::min(std::min(cap, 65535), (int)((budget - fixed) / 16)));
     };
     int best_tiles = S.nc[1];
-    double best_score = 0.0;
+    double best_cost = 0.0;
     for (int c = 1; c <= TILE_Y_MAX && c <= S.nc[1]; ++c) {
       set_tiles((S.nc[1] + c - 1) / c);
-      const double rows = (double)S.nc[1] / S.tiles_y;
-      const double passes = std::ceil((1.02 * S.tile_y * per_row + 4.0) / 256.0);
-      if (passes > 3.0 && c > 1) break;
-      const double blocks = std::min(4.0, std::floor(227.0 * 1024.0 / (double)(build_tile_smem(S) + 1024)));
-      const double score = rows * per_row / (256.0 * passes) * rows / (rows + 0.6) * blocks;
-      if (score > best_score) {
-        best_score = score;
+      const double rows = (double)S.nc[1] / S.tiles_y, threads = tile_threads();
+      // resident tiles of an SM (by shared memory, and by 64 registers a thread)
+      const double per_sm = std::max(1.0, std::min(std::floor(227.0 * 1024.0 / (double)(build_tile_smem(S) + 1024)),
+                                                   std::floor(1024.0 / threads)));
+      const double waves = (double)S.tiles_y * S.nc[2] / (sms * per_sm);
+      const bool few = waves <= 2.02;
+      const double rounds = few ? std::ceil(waves - 0.02) : waves + 0.3;
+      const double mean = S.tile_y * per_row;
+      const double passes = std::ceil((few ? 1.03 * mean + 6.0 : 1.01 * mean + 4.0) / threads);
+      const double cost = rounds * passes + 0.00069 * ((double)S.n / sms) / rows;
+      if (c == 1 || cost < best_cost) {
+        best_cost = cost;
         best_tiles = S.tiles_y;
       }
     }
     set_tiles(best_tiles);
-    const double mean_tile = S.tile_y * per_row;
-    const int threads = (int)std::ceil((mean_tile + 3.0 * std::sqrt(mean_tile) + 16.0) / 32.0) * 32;
-    S.tile_threads = std::max(64, std::min(256, threads));
+    S.tile_threads = tile_threads();
     // persistent runs: the rows per tile whose list build is shortest when one
     // block per SM takes the tiles in turn (a tile's staging costs about as
     // much as 1.6 rounds of its 512 threads over (slot, layer) pairs)
