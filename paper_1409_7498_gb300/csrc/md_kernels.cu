@@ -730,7 +730,8 @@ __global__ void __launch_bounds__(256) kb_rebin_permute(const Sys* __restrict__ 
 // Rebuild of a batch's members through buckets (all of them with at most
 // BUCKET_CELLS cells that hold few particles): the keys' atomics give each
 // slot's arrival rank in its cell, under which it is noted in the cell's
-// bucket; a scan of the counts gives the cells' first slots, and a slot's new
+// bucket, or, beyond ENG_BUCKET members, linked to the cell's further ones (fill
+// holds their heads, win the links; slots plus one, 0 the end); a scan of the counts gives the cells' first slots, and a slot's new
 // place is its cell's first slot plus the number of the cell's members with a
 // smaller old slot.  With the plan's work done by the step kernel, four
 // kernels instead of ten: 256 replicas 377 -> 366 us per step.  (A single
@@ -747,6 +748,7 @@ __device__ __forceinline__ void keys_bucket_body(const Sys& S, const Blk blk) {
   S.key[i] = k;
   const uint32_t rank = atomicAdd(&S.count[k], 1u);
   if (rank < ENG_BUCKET) S.bucket[(size_t)k * ENG_BUCKET + rank] = i;
+  else S.win[i] = atomicExch(&S.fill[k], i + 1u);  // (win is free outside reaction steps)
 }
 
 // Scan tile blk.b with the counts before it summed by the block itself.
@@ -778,20 +780,27 @@ __device__ __forceinline__ void scan_direct_body(const Sys& S, const Blk blk) {
 }
 
 // Old slots of block blk of 256, and the block's share of the counters back to
-// zero.  A cell with more members than a bucket holds (rare where buckets are
-// used) has them counted from the keys.
+// zero.  In a cell with more members than a bucket holds (one in 10,000 to 100
+// at four to six per cell on average) a lookup costs one load after another for
+// each further member.  Counted from the keys of all slots instead, it cost the
+// cell's every member and bond partner a walk over the system: two members of
+// 200,000 particles, 4.3 per cell, 304 us per step; with the links 72.
 __device__ __forceinline__ void permute_bucket_body(const Sys& S, const Blk blk) {
   Ctl* ctl = S.ctl;
   const SoA A = ctl->set ? S.s1 : S.s0, B = ctl->set ? S.s0 : S.s1;
   uint4* P = ctl->phase ? S.P1 : S.P0;
   auto start = [&](uint32_t k) { return S.cell_start[k]; };
-  auto from_keys = [&](uint32_t j, uint32_t k, uint32_t first, uint32_t) {
+  auto linked = [&](uint32_t j, uint32_t k, uint32_t first, uint32_t) {
+    const uint32_t* b = S.bucket + (size_t)k * ENG_BUCKET;
     uint32_t r = first;
-    for (uint32_t i = 0; i < j; ++i) r += S.key[i] == k ? 1u : 0u;
+#pragma unroll 4
+    for (uint32_t q = 0; q < ENG_BUCKET; ++q) r += b[q] < j ? 1u : 0u;
+#pragma unroll 1
+    for (uint32_t h = S.fill[k]; h; h = S.win[h - 1u]) r += h - 1u < j ? 1u : 0u;
     return r;
   };
   const uint32_t o = blk.b * 256u + threadIdx.x;
-  if (o < S.n) permute_old<true>(S, A, B, P, S.tmp, o, start, false, from_keys);
+  if (o < S.n) permute_old<true>(S, A, B, P, S.tmp, o, start, false, linked);
   for (uint32_t c = o; c < (uint32_t)S.ncell; c += blk.nb * 256u) S.count[c] = 0u;
 }
 
@@ -847,6 +856,8 @@ __global__ void __launch_bounds__(256, 4)
   for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
     const BlkMap m = M[e];
     const Sys& S = T[m.sys];
+    if (act_n)  // bucket rebuilds: the links' heads back to zero
+      for (uint32_t c = m.b * blockDim.x + threadIdx.x; c < (uint32_t)S.ncell; c += m.nb * blockDim.x) S.fill[c] = 0u;
     if (S.nl16) build_nlist_body<true>(S, Blk{m.b, m.nb}, smem_b);
     else build_nlist_body<false>(S, Blk{m.b, m.nb}, smem_b);
     __syncthreads();  // the buffers and the warp count are used again
