@@ -670,7 +670,7 @@ __device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4
       const uint32_t i = valid ? list[w] : 0u;
       uint32_t best = NONE, ch = 0u;
       if (R.rule == PRX_SELECT_NEAREST) best = nearest_partner<NL16, RX_GROUP>(S, B, P, i, valid, true, unused);
-      else best = rx_find_multi<NL16>(S, B, P, step, i, valid, unused, unused, ch);
+      else best = rx_find_multi<NL16, RX_GROUP>(S, B, P, step, i, valid, unused, unused, ch);
       if (valid && lane % RX_GROUP == 0) {
         if (R.nr > 1) S.wch[i] = (uint8_t)ch;
         S.win[i] = best;
@@ -691,7 +691,7 @@ __device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4
     const uint32_t w = wb + (uint32_t)lane / RX_GROUP;
     const uint32_t i = w < nact ? list[w] : 0u;
     bool unused_w;
-    const uint32_t T = rx_decide<NL16>(S, B, step, i, w < nact, unused_w);
+    const uint32_t T = rx_decide<NL16, RX_GROUP>(S, B, step, i, w < nact, unused_w);
     (void)rx_form(S, B, step, i, lane % RX_GROUP == 0 ? T : NONE, dpop);
   }
   __syncthreads();

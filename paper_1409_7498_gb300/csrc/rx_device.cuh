@@ -37,6 +37,21 @@ __device__ __forceinline__ uint32_t nl_get_rx(const Sys& S, int k, uint32_t i) {
 // runs once per slot instead of once per entry.  Called by whole warps unless
 // G = 1; lanes of a group without a slot pass valid = false.
 constexpr int RX_GROUP = 16;
+// Lanes per eligible A in the one-phase kernels.  While the groups fit the GPU
+// at once, more lanes shorten the chain; beyond, the slot's own loads and draws
+// of every group queue up.  us of the search with 16 / 4 / 1 lanes, nearest
+// rule: 2,200 A's 14.7 / 16.9 / 34, 20,000 29.7 / 24.6 / 39, 67,000 72 / 50 / 54,
+// 117,000 118 / 78 / 71; concurrent reactions: 11,000 22 / 25 / 46, 33,000 37 /
+// 32 / 56, 116,000 104 / 79 / 93.  Of the selection: nearest rule (which walks no
+// list), 2,200 A's 12.0 / 10.2 / 10.2, 117,000 30 / 21 / 14.3; random rule, 2,200
+// 13.6 / 12.6 / 11.4, 11,000 14.3 / 13.8 / 14.0, 67,000 22 / 17.7 / 15.6.
+__device__ __forceinline__ int rx_find_lanes(const RxParams& R, uint32_t nact) {
+  const bool several = R.nr > 1;
+  return nact <= (several ? 20000u : 5000u) ? RX_GROUP : nact <= (several ? 200000u : 90000u) ? 4 : 1;
+}
+__device__ __forceinline__ int rx_select_lanes(const RxParams& R, uint32_t nact) {
+  return R.rule == PRX_SELECT_NEAREST || nact > 32768u ? 1 : 4;
+}
 template <bool NL16, int G>
 __device__ __forceinline__ uint32_t nearest_partner(const Sys& S, const SoA& B, const uint4* P,
                                                     uint32_t i, bool valid, bool want_T, long long& in_range) {
@@ -112,8 +127,8 @@ __device__ __forceinline__ void rx_accept_and_key(const Sys& S, const SoA& B,
 // reaction's windows, exact FP64 r^2 below the reaction's cutoff, not
 // bonded), one acceptance draw against the cumulative bounds of m, and the
 // retained pair of smallest selection key.  `ch` receives the chosen pair's
-// reaction.  A group of RX_GROUP lanes per A, as in nearest_partner.
-template <bool NL16>
+// reaction.  A group of G lanes per A, as in nearest_partner.
+template <bool NL16, int G>
 __device__ __forceinline__ uint32_t rx_find_multi(const Sys& S, const SoA& B, const uint4* P,
                                                   unsigned long long step, uint32_t i, bool valid,
                                                   long long& ncand, long long& nret, uint32_t& ch) {
@@ -126,7 +141,7 @@ __device__ __forceinline__ uint32_t rx_find_multi(const Sys& S, const SoA& B, co
   uint32_t best = NONE, bestid = 0u;
   unsigned long long bestkey = 0ull;
   const int cnt = valid ? S.nn[i] : 0;
-  for (int k = (int)(threadIdx.x & (RX_GROUP - 1)); k < cnt; k += RX_GROUP) {
+  for (int k = (int)(threadIdx.x & (G - 1)); k < cnt; k += G) {
     const uint32_t j = nl_get_rx<NL16>(S, k, i);
     const uint4 pj = P[j];
     const float ex = __int2float_rn(pdiff(pj.x, pi.x)) * S.scale[0];
@@ -167,7 +182,7 @@ __device__ __forceinline__ uint32_t rx_find_multi(const Sys& S, const SoA& B, co
     }
   }
 #pragma unroll
-  for (int o = RX_GROUP / 2; o > 0; o >>= 1) {
+  for (int o = G / 2; o > 0; o >>= 1) {
     const unsigned long long key = __shfl_xor_sync(0xFFFFFFFFu, bestkey, o);
     const uint32_t id = __shfl_xor_sync(0xFFFFFFFFu, bestid, o), j = __shfl_xor_sync(0xFFFFFFFFu, best, o);
     const uint32_t c = __shfl_xor_sync(0xFFFFFFFFu, ch, o);
@@ -282,11 +297,12 @@ __device__ __forceinline__ void rx_find_random4(const Sys& S, const Blk blk, con
   }
 }
 
-// Steps 6-7 for one eligible A (a group of RX_GROUP lanes, as in
-// nearest_partner): the T it keeps (NONE: none), the same in every lane of the
-// group; `winner` tells whether it had picked one (random rule) or its choice
-// was mutual (nearest).
-template <bool NL16>
+// Steps 6-7 for one eligible A (a group of G lanes, as in nearest_partner):
+// the T it keeps (NONE: none), the same in every lane of the group; `winner`
+// tells whether it had picked one (random rule) or its choice was mutual
+// (nearest).  A lane alone takes four list entries of T at a time (independent
+// loads go out together).
+template <bool NL16, int G>
 __device__ __forceinline__ uint32_t rx_decide(const Sys& S, const SoA& B, unsigned long long step,
                                               uint32_t i, bool valid, bool& winner) {
   const RxParams& R = S.R;
@@ -308,21 +324,32 @@ __device__ __forceinline__ uint32_t rx_decide(const Sys& S, const SoA& B, unsign
   uint32_t idi = 0u, idT = 0u;
   unsigned long long mine = 0ull;
   bool drawn = false;
-  for (int k = (int)(threadIdx.x & (RX_GROUP - 1)); k < cnt; k += RX_GROUP) {
-    const uint32_t a = nl_get_rx<NL16>(S, k, T);
-    if (a == i || S.win[a] != T) continue;
-    if (!drawn) {
-      idi = B.id[i], idT = B.id[T];
-      mine = key64(keyed_draw(S.seed, step, idT, idi, TAG_SEL_T));
-      drawn = true;
+  constexpr int U = G == 1 ? 4 : 1;
+  for (int k = (int)(threadIdx.x & (G - 1)); k < cnt; k += G * U) {
+    uint32_t aa[U], wa[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) aa[u] = k + u * G < cnt ? nl_get_rx<NL16>(S, k + u * G, T) : i;
+#pragma unroll
+    for (int u = 0; u < U; ++u) wa[u] = S.win[aa[u]];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (aa[u] == i || wa[u] != T) continue;
+      if (!drawn) {
+        idi = B.id[i], idT = B.id[T];
+        mine = key64(keyed_draw(S.seed, step, idT, idi, TAG_SEL_T));
+        drawn = true;
+      }
+      const uint32_t ida = B.id[aa[u]];
+      const unsigned long long other = key64(keyed_draw(S.seed, step, idT, ida, TAG_SEL_T));
+      lost |= other < mine || (other == mine && ida < idi);
     }
-    const uint32_t ida = B.id[a];
-    const unsigned long long other = key64(keyed_draw(S.seed, step, idT, ida, TAG_SEL_T));
-    lost |= other < mine || (other == mine && ida < idi);
   }
-  const unsigned any = __ballot_sync(0xFFFFFFFFu, lost);
-  const unsigned group = ((1u << RX_GROUP) - 1u) << ((threadIdx.x & 31u) & ~(RX_GROUP - 1u));
-  return winner && !(any & group) ? T : NONE;
+  if constexpr (G > 1) {
+    const unsigned any = __ballot_sync(0xFFFFFFFFu, lost);
+    const unsigned group = ((1u << G) - 1u) << ((threadIdx.x & 31u) & ~(G - 1u));
+    lost = (any & group) != 0u;
+  }
+  return winner && !lost ? T : NONE;
 }
 
 // Step 9 for the pairs (i, T) of a warp (T = NONE: none), called by the whole

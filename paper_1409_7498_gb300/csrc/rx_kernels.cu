@@ -19,6 +19,8 @@
 //                the reaction's history record from them.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "prx_internal.cuh"
 #include "rx_device.cuh"
 
@@ -112,7 +114,10 @@ __global__ void __launch_bounds__(RX_THREADS)
   rx_compact_body(S, m.b >> 2);
 }
 
-template <bool NL16>
+// KIND 0: one reaction by the random rule; 1: the nearest rule or concurrent
+// reactions, with the lanes that suit their number of A's; 2: a batch's member,
+// either of these (four lanes: the other members fill the GPU too).
+template <bool NL16, int KIND>
 __device__ __forceinline__ void rx_find_body(const Sys& S, const Blk blk, long long step_arg) {
   const RxParams& R = S.R;
 
@@ -121,27 +126,35 @@ __device__ __forceinline__ void rx_find_body(const Sys& S, const Blk blk, long l
   const SoA B = ctl->set ? S.s1 : S.s0;
   const uint4* P = ctl->phase ? S.P1 : S.P0;
   const uint32_t nact = ctl->n_active;
-  // four lanes per eligible A (random rule) or a group: blocks past them have nothing to do
-  const bool four = R.rule != PRX_SELECT_NEAREST && R.nr <= 1;
-  if (blk.b * (blockDim.x / (four ? 4u : (unsigned)RX_GROUP)) >= nact) return;
+  // four lanes per eligible A (one reaction, random rule) or a group: blocks past them have nothing to do
+  const bool four = KIND == 0 || (KIND == 2 && R.rule != PRX_SELECT_NEAREST && R.nr <= 1);
+  const uint32_t lanes = KIND == 1 ? (uint32_t)rx_find_lanes(R, nact) : 4u;
+  if (blk.b * (blockDim.x / lanes) >= nact) return;
   long long ncand = 0, nret = 0;
   if (four) {
     rx_find_random4<NL16>(S, blk, B, P, step, S.tmp, nact, ncand, nret);
-  } else {
+  } else if constexpr (KIND != 0) {
     // the nearest rule and concurrent reactions: a group of lanes per eligible A
-    const uint32_t lane = threadIdx.x & 31u;
-    for (uint32_t wb = (blk.b * blockDim.x + (threadIdx.x & ~31u)) / RX_GROUP; wb < nact;
-         wb += blk.nb * blockDim.x / RX_GROUP) {
-      const uint32_t w = wb + lane / RX_GROUP;
-      const bool valid = w < nact;
-      const uint32_t i = valid ? S.tmp[w] : 0u;
-      uint32_t best = NONE, ch = 0u;
-      if (R.rule == PRX_SELECT_NEAREST) best = nearest_partner<NL16, RX_GROUP>(S, B, P, i, valid, true, ncand);
-      else best = rx_find_multi<NL16>(S, B, P, step, i, valid, ncand, nret, ch);
-      if (valid && lane % RX_GROUP == 0u) {
-        if (R.nr > 1) S.wch[i] = (uint8_t)ch;
-        S.win[i] = best;
+    auto groups = [&](auto g) {
+      constexpr int G = decltype(g)::value;
+      const uint32_t lane = threadIdx.x & 31u;
+      for (uint32_t wb = (blk.b * blockDim.x + (threadIdx.x & ~31u)) / G; wb < nact; wb += blk.nb * blockDim.x / G) {
+        const uint32_t w = wb + lane / G;
+        const bool valid = w < nact;
+        const uint32_t i = valid ? S.tmp[w] : 0u;
+        uint32_t best = NONE, ch = 0u;
+        if (R.rule == PRX_SELECT_NEAREST) best = nearest_partner<NL16, G>(S, B, P, i, valid, true, ncand);
+        else best = rx_find_multi<NL16, G>(S, B, P, step, i, valid, ncand, nret, ch);
+        if (valid && lane % G == 0u) {
+          if (R.nr > 1) S.wch[i] = (uint8_t)ch;
+          S.win[i] = best;
+        }
       }
+    };
+    if (KIND == 2 || lanes == 4u) groups(std::integral_constant<int, 4>{});
+    else if constexpr (KIND == 1) {
+      if (lanes == 1u) groups(std::integral_constant<int, 1>{});
+      else groups(std::integral_constant<int, RX_GROUP>{});
     }
   }
   const long long c = block_sum_ll(ncand);
@@ -152,17 +165,17 @@ __device__ __forceinline__ void rx_find_body(const Sys& S, const Blk blk, long l
   }
 }
 
-template <bool NL16>
-__global__ void __launch_bounds__(RX_THREADS) k_rx_find(Sys S, long long step_arg) {
-  rx_find_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, step_arg);
+template <bool NL16, int KIND>
+__global__ void __launch_bounds__(RX_THREADS, 4) k_rx_find(Sys S, long long step_arg) {
+  rx_find_body<NL16, KIND>(S, Blk{blockIdx.x, gridDim.x}, step_arg);
 }
 __global__ void __launch_bounds__(RX_THREADS, 4)
     kb_rx_find(const Sys* __restrict__ T, const BlkMap* __restrict__ M) {
   const BlkMap m = M[blockIdx.x];
   const Sys& S = T[m.sys];
   if (!S.has_rx) return;  // this member has no reaction scheme
-  if (S.nl16) rx_find_body<true>(S, Blk{m.b, m.nb}, -1LL);
-  else rx_find_body<false>(S, Blk{m.b, m.nb}, -1LL);
+  if (S.nl16) rx_find_body<true, 2>(S, Blk{m.b, m.nb}, -1LL);
+  else rx_find_body<false, 2>(S, Blk{m.b, m.nb}, -1LL);
 }
 
 // Steps 6-7 for one A winner: every other A that picked the same T lies
@@ -212,7 +225,8 @@ __device__ __forceinline__ void rx_select_apply_body(const Sys& S, const Blk blk
   const uint32_t nact = ctl->n_active;
   // blocks past the eligible A's have nothing to do; the last of the others
   // (of the first, when there is no A) writes the record
-  const uint32_t per = blockDim.x / RX_GROUP;  // A's per block and pass
+  const uint32_t lanes = (uint32_t)rx_select_lanes(R, nact);
+  const uint32_t per = blockDim.x / lanes;  // A's per block and pass
   const uint32_t busy = max(1u, min(blk.nb, (nact + per - 1u) / per));
   if (blk.b >= busy) return;
   long long nwin = 0, nfin = 0;
@@ -222,15 +236,20 @@ __device__ __forceinline__ void rx_select_apply_body(const Sys& S, const Blk blk
   __syncthreads();
   // block-strided over the eligible A's (a group of lanes each), warp-uniform
   // trip count
-  for (uint32_t base = blk.b * per; base < nact; base += blk.nb * per) {
-    const uint32_t w = base + threadIdx.x / RX_GROUP;
-    const bool first = threadIdx.x % RX_GROUP == 0u;
-    const uint32_t i = w < nact ? S.tmp[w] : 0u;
-    bool winner;
-    const uint32_t T = rx_decide<NL16>(S, B, step, i, w < nact, winner);
-    nwin += winner && first ? 1 : 0;
-    nfin += rx_form(S, B, step, i, first ? T : NONE, dpop) ? 1 : 0;
-  }
+  auto groups = [&](auto g) {
+    constexpr uint32_t G = decltype(g)::value;
+    for (uint32_t base = blk.b * per; base < nact; base += blk.nb * per) {
+      const uint32_t w = base + threadIdx.x / G;
+      const bool first = threadIdx.x % G == 0u;
+      const uint32_t i = w < nact ? S.tmp[w] : 0u;
+      bool winner;
+      const uint32_t T = rx_decide<NL16, (int)G>(S, B, step, i, w < nact, winner);
+      nwin += winner && first ? 1 : 0;
+      nfin += rx_form(S, B, step, i, first ? T : NONE, dpop) ? 1 : 0;
+    }
+  };
+  if (lanes == 4u) groups(std::integral_constant<uint32_t, 4>{});
+  else groups(std::integral_constant<uint32_t, 1>{});
   const long long cw = block_sum_ll(nwin);
   const long long cf = block_sum_ll(nfin);
   if (threadIdx.x == 0) {
@@ -468,8 +487,13 @@ void launch_rx(const Sys& S, cudaStream_t st, long long step_arg,
   H("rx_compact", 1);
   const unsigned gf = g < 1216u ? g : 1216u;
   H("rx_find", 0);
-  if (S.nl16) k_rx_find<true><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
-  else k_rx_find<false><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
+  if (S.R.rule != PRX_SELECT_NEAREST && S.R.nr <= 1) {
+    if (S.nl16) k_rx_find<true, 0><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
+    else k_rx_find<false, 0><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
+  } else {
+    if (S.nl16) k_rx_find<true, 1><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
+    else k_rx_find<false, 1><<<gf, RX_THREADS, 0, st>>>(S, step_arg);
+  }
   H("rx_find", 1);
   if (S.R.rule == PRX_SELECT_NEAREST) {
     H("rx_find_T", 0);
