@@ -1568,8 +1568,11 @@ int prx_get_bonds(prx_system* sys, prx_bond* out, uint64_t cap, uint64_t* n_out)
     return cap < nb ? fail(sys, PRX_ECAPACITY, "bond buffer too small") : PRX_OK;
   }
   // in canonical order on the device (the force scratch arrays, free outside
-  // a step, take the other half of the merge), unless they are too short
-  if (24ull * nb <= sys->bond_scratch) {
+  // a step, take the other half of the merge), unless they are too short or the
+  // records so few that the host sorts them sooner than a tile's network runs:
+  // us per call, host / device, 100 records 51 / 67, 1,000 63 / 76, 1,500 76 / 78,
+  // 2,000 99 / 78, 10,000 529 / 103
+  if (nb > 1536 && 24ull * nb <= sys->bond_scratch) {
     const BondRec* sorted = launch_sort_bonds(sys->S.bonds, (BondRec*)sys->S.fout, (uint32_t)nb, sys->stream);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(out, sorted, sizeof(prx_bond) * m, cudaMemcpyDeviceToHost, sys->stream));
