@@ -391,9 +391,10 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_256(uint32_t v, uint32_
 // neighbour rows are staged in shared memory (one pass in the common case) as
 // the FP32 coordinates that the permutation left in fout (build_xyz), each
 // row extended by one periodic image cell at both ends, so every particle's
-// 3 x 3 x 3 cell neighbourhood is 9 contiguous ranges.  Rows that are images
-// in y or z are met by shifting the particle's own coordinates.  A pair enters the list when its FP32 distance is below r_c + skin (widened by
-// the rounding bound).
+// 3 x 3 x 3 cell neighbourhood is 9 contiguous ranges.  y and z count from each
+// row's own lower edges: a candidate's row is one edge up or down or the same,
+// whether it is a periodic image or not.  A pair enters the list when its FP32
+// distance is below r_c + skin (widened by the rounding bound).
 //
 // Bound by instruction issue: ~15 instructions per candidate and lane, ~110
 // candidates.  Taking the coordinates from the permutation and describing the
@@ -408,23 +409,23 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// FP32 coordinates of a slot for the list build, in [0, L) per axis up to
-// rounding: a position that rounds across the box edge from the cell that the
-// sort put it in is kept on that cell's side.
-// .w holds the slot.
+// FP32 coordinates of a slot for the list build.  x in [0, L) up to rounding: a
+// position that rounds across the box edge from the cell that the sort put it
+// in is kept on that cell's side.  y and z from the lower edges of the cell row
+// that the sort put it in, so that they carry the rounding of a cell's edge, not
+// of the box's.  .w holds the slot.
 __device__ __forceinline__ float4 build_xyz(const Sys& S, uint32_t X, uint32_t Y, uint32_t Z, uint32_t key,
                                             uint32_t slot) {
-  const uint32_t nx = (uint32_t)S.nc[0], ny = (uint32_t)S.nc[1], nz = (uint32_t)S.nc[2];
-  const uint32_t row = key / nx, c[3] = {key - row * nx, row % ny, row / ny}, n[3] = {nx, ny, nz};
-  const uint32_t p[3] = {X, Y, Z};
-  float f[3];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    f[d] = __uint2float_rn(p[d]) * S.scale[d];
-    if (c[d] == 0u && p[d] >= 0xC0000000u) f[d] -= (float)S.L[d];
-    if (c[d] == n[d] - 1u && p[d] < 0x40000000u) f[d] += (float)S.L[d];
-  }
-  return make_float4(f[0], f[1], f[2], __uint_as_float(slot));
+  const uint32_t nx = (uint32_t)S.nc[0], ny = (uint32_t)S.nc[1];
+  const uint32_t row = key / nx, cx = key - row * nx, cz = row / ny, cy = row - cz * ny;
+  float x = __uint2float_rn(X) * S.scale[0];
+  if (cx == 0u && X >= 0xC0000000u) x -= (float)S.L[0];
+  if (cx == nx - 1u && X < 0x40000000u) x += (float)S.L[0];
+  // c 2^32 / nc to within one unit
+  const uint32_t y0 = (uint32_t)__umul64hi((unsigned long long)cy << 32, S.inv_nc64[0]);
+  const uint32_t z0 = (uint32_t)__umul64hi((unsigned long long)cz << 32, S.inv_nc64[1]);
+  return make_float4(x, __int2float_rn(pdiff(Y, y0)) * S.scale[1], __int2float_rn(pdiff(Z, z0)) * S.scale[2],
+                     __uint_as_float(slot));
 }
 
 struct BuildRow {
@@ -434,7 +435,6 @@ struct BuildRow {
   int tot;          // padL + cnt + particles of the right image cell (cell 0)
   int lo;           // first slot of the row
   int left;         // first slot of cell nx-1
-  float yoff, zoff; // image shift of the row
 };
 constexpr int TILE_ROWS_MAX = 3 * (TILE_Y_MAX + 2);
 
@@ -509,8 +509,6 @@ __device__ __forceinline__ void build_tile(const Sys& S, const float4* F, const 
       r.tot = r.padL + r.cnt + (int)(cs[1] - cs[0]);
       r.lo = (int)cs[0];
       r.left = (int)cs[nx - 1];
-      r.yoff = uy < 0 ? -(float)S.L[1] : (uy >= ny ? (float)S.L[1] : 0.f);
-      r.zoff = uz < 0 ? -(float)S.L[2] : (uz >= nz ? (float)S.L[2] : 0.f);
       ri[sr] = r;
     }
   }
@@ -603,8 +601,8 @@ __device__ __forceinline__ void build_tile(const Sys& S, const float4* F, const 
       for (int w = 0; w < 9; ++w) {
         const int lo = max((int)(win[w] & 0xFFFFu), c0) - c0;
         const int hi = min((int)(win[w] >> 16), c0 + cn) - c0;
-        const BuildRow& r = ri[(w / 3) * RY + yrel + (w % 3)];
-        const float y = fi.y - r.yoff, z = fi.z - r.zoff;
+        const float y = fi.y - (float)(w % 3 - 1) * S.cell_edge_f[0];
+        const float z = fi.z - (float)(w / 3 - 1) * S.cell_edge_f[1];
         auto walk = [&](int a, int b) {
 #pragma unroll 2
           for (int k = a; k < b; ++k) {

@@ -324,8 +324,9 @@ int setup_grid(prx_system* sys, double rc) {
   const double dmax = 0.5 * skin - 2.0 * std::sqrt(3.0) * wmax - 1e-6;
   if (!(dmax > 0.0)) return fail(sys, PRX_EINVAL, "skin too small for the displacement trigger");
   S.disp2_max = (float)(dmax * dmax);
-  // the list build compares FP32 tile-frame coordinates (~2e-7 L of rounding
-  // per coordinate): its radius is widened by more than that error
+  // the list build compares FP32 coordinates, x in the box (~2e-7 L of
+  // rounding), y and z from a cell row's edges (less than that): its radius is
+  // widened by more than that error
   {
     const double Lmax = std::max(sys->d.box[0], std::max(sys->d.box[1], sys->d.box[2]));
     const double rvb = rv * (1.0 + 1e-5) + 1e-6 * Lmax;
