@@ -570,53 +570,67 @@ __device__ __forceinline__ void build_tile(const Sys& S, const float4* F, const 
       yrel = 0;
       cx = 0;
     }
-    uint32_t win[9];
-#pragma unroll
-    for (int w = 0; w < 9; ++w) {
+    // staged entries [lo, hi) of window w
+    auto window = [&](int w, int& lo, int& hi) {
       const int sr = (w / 3) * RY + yrel + (w % 3);
       const uint32_t* cs = sCS + sr * (nx + 1);
       const BuildRow& r = ri[sr];
       const int off = r.base + r.padL - r.lo;  // slot -> staged entry
-      const int lo = cx == 0 ? r.base : off + (int)cs[cx - 1];
-      const int hi = cx + 2 > nx ? r.base + r.tot : off + (int)cs[cx + 2];
-      win[w] = (uint32_t)lo | ((uint32_t)hi << 16);
+      lo = cx == 0 ? r.base : off + (int)cs[cx - 1];
+      hi = cx + 2 > nx ? r.base + r.tot : off + (int)cs[cx + 2];
+    };
+    uint32_t win[9];  // (rows staged at once are at most CAP <= 65,535 entries)
+    if (one) {
+#pragma unroll
+      for (int w = 0; w < 9; ++w) {
+        int lo, hi;
+        window(w, lo, hi);
+        win[w] = (uint32_t)lo | ((uint32_t)hi << 16);
+      }
     }
     const int kself0 = ri[RY + yrel + 1].base + ri[RY + yrel + 1].padL + ((int)i - ri[RY + yrel + 1].lo);
     int cnt = 0;
     const int cap = S.list_cap;
     unsigned char* col = (unsigned char*)S.nl + (size_t)i * (NL16 ? 2 : 4);
     const uint32_t stride = S.n * (NL16 ? 2u : 4u);
-    for (int c0 = 0; c0 < TOT; c0 += CAP) {
-      const int cn = min(CAP, TOT - c0);
-      if (!one) {  // neighbour rows longer than the buffer: staged per chunk
+    // the staged entries [lo, hi) of window w; the particle itself is staged
+    // once (entry kself), in the centre row's window (w = 4), whose walk skips
+    // it: no candidate needs a self test
+    auto candidates = [&](int w, int lo, int hi, int kself) {
+      const float y = fi.y - (float)(w % 3 - 1) * S.cell_edge_f[0];
+      const float z = fi.z - (float)(w / 3 - 1) * S.cell_edge_f[1];
+      auto walk = [&](int a, int b) {
+#pragma unroll 2
+        for (int k = a; k < b; ++k) {
+          const float4 q = sX[k];
+          const float dx = q.x - fi.x, dy = q.y - y, dz = q.z - z;
+          list_candidate<NL16>(col, stride, fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rv2, __float_as_uint(q.w), cap,
+                               cnt);
+        }
+      };
+      if (w == 4) {
+        walk(lo, min(hi, max(lo, kself)));
+        walk(max(lo, kself + 1), hi);
+      } else {
+        walk(lo, hi);
+      }
+    };
+    if (one) {
+      if (act) {
+#pragma unroll
+        for (int w = 0; w < 9; ++w) candidates(w, (int)(win[w] & 0xFFFFu), (int)(win[w] >> 16), kself0);
+      }
+    } else {
+      for (int c0 = 0; c0 < TOT; c0 += CAP) {  // neighbour rows longer than the buffer: staged per chunk
+        const int cn = min(CAP, TOT - c0);
         __syncthreads();
         stage(c0, cn);
         __syncthreads();
-      }
-      if (!act) continue;
-      // the particle itself is staged once, in the centre row's window
-      // (w = 4), whose walk skips it: no candidate needs a self test
-      const int kself = kself0 - c0;
-#pragma unroll
-      for (int w = 0; w < 9; ++w) {
-        const int lo = max((int)(win[w] & 0xFFFFu), c0) - c0;
-        const int hi = min((int)(win[w] >> 16), c0 + cn) - c0;
-        const float y = fi.y - (float)(w % 3 - 1) * S.cell_edge_f[0];
-        const float z = fi.z - (float)(w / 3 - 1) * S.cell_edge_f[1];
-        auto walk = [&](int a, int b) {
-#pragma unroll 2
-          for (int k = a; k < b; ++k) {
-            const float4 q = sX[k];
-            const float dx = q.x - fi.x, dy = q.y - y, dz = q.z - z;
-            list_candidate<NL16>(col, stride, fmaf(dz, dz, fmaf(dy, dy, dx * dx)), rv2, __float_as_uint(q.w), cap,
-                                 cnt);
-          }
-        };
-        if (w == 4) {
-          walk(lo, min(hi, max(lo, kself)));
-          walk(max(lo, kself + 1), hi);
-        } else {
-          walk(lo, hi);
+#pragma unroll 1
+        for (int w = 0; act && w < 9; ++w) {
+          int lo, hi;
+          window(w, lo, hi);
+          candidates(w, max(lo, c0) - c0, min(hi, c0 + cn) - c0, kself0 - c0);
         }
       }
     }

@@ -396,7 +396,7 @@ int setup_grid(prx_system* sys, double rc) {
     for (int c = 1; c <= TILE_Y_MAX && c <= S.nc[1]; ++c) {
       set_tiles((S.nc[1] + c - 1) / c);
       const double rows = (double)S.nc[1] / S.tiles_y, threads = tile_threads();
-      // resident tiles of an SM (by shared memory, and by 64 registers a thread)
+      // resident tiles of an SM: by shared memory, and up to 1,024 threads
       const double per_sm = std::max(1.0, std::min(std::floor(227.0 * 1024.0 / (double)(build_tile_smem(S) + 1024)),
                                                    std::floor(1024.0 / threads)));
       const double waves = (double)S.tiles_y * S.nc[2] / (sms * per_sm);
