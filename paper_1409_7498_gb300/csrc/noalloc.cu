@@ -59,7 +59,7 @@ struct NaArgs {
   unsigned long long step;
   RxParams R;
   float Lf[3], invLf[3];
-  float near2;  // FP32 r^2 from which a pair is out of range for sure
+  float near2;  // FP32 r^2 from which a pair is out of range for sure (NaN: none is)
   NaScratch* sc;
 };
 
@@ -478,6 +478,9 @@ extern "C" int prx_react_noalloc(const prx_reaction_desc* rx, const double* box,
   const double Lmax = std::fmax(box[0], std::fmax(box[1], box[2]));
   const double reach = rx->r_react * (1.0 + 1e-5) + 4e-6 * Lmax;
   a.near2 = (float)(reach * reach * (1.0 + 1e-5));
+  // beyond these lengths a square leaves the FP32 range at either end: a bound
+  // that no distance is beyond sends every pair to the exact test
+  if (!(Lmax < 1e18 && reach > 1e-18)) a.near2 = NAN;
   for (int k = 0; k < 3; ++k) {
     a.Lf[k] = (float)box[k];
     a.invLf[k] = (float)(1.0 / box[k]);
