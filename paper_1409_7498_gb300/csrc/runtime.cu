@@ -69,8 +69,8 @@ struct prx_system {
   cudaGraphExec_t g_chunk1 = nullptr;  // one interval, when g_chunk holds several
   uint32_t chunk_m = 1;                // reaction intervals per g_chunk replay
   // device graphs of device-driven runs (dg.cu): the steps (+ k_dg_next), the
-  // rebuild, the reaction; dg_ok when all three instantiated.  dg_one holds
-  // one step, for runs shorter than dg_step's (made when first needed).
+  // rebuild, the reaction; dg_ok when they instantiated.  dg_one holds one step,
+  // for runs shorter than dg_step's (each of the two is made when first needed).
   cudaGraphExec_t dg_step = nullptr, dg_rebuild = nullptr, dg_react = nullptr, dg_one = nullptr;
   uint32_t dg_steps = 1;  // steps in dg_step
   bool dg_ok = false;
@@ -565,9 +565,25 @@ cudaError_t build_dg_step(prx_system* sys, uint32_t steps, cudaGraphExec_t* out)
   }, out);
 }
 
-// The device graphs of device-driven runs; on any failure the system keeps
-// the host-replayed graphs (the same kernels).
-void build_device_graphs(prx_system* sys) {
+// The step graph that suits a run of nsteps steps, made when first needed (the
+// other one where it cannot be made: both run any number of steps).  A run
+// shorter than the longer graph would end in empty step kernels (~2 us each).
+cudaGraphExec_t dg_graph(prx_system* sys, uint64_t nsteps) {
+  const bool one = nsteps < sys->dg_steps;
+  cudaGraphExec_t& want = one ? sys->dg_one : sys->dg_step;
+  if (!want && (build_dg_step(sys, one ? 1 : sys->dg_steps, &want) != cudaSuccess ||
+                cudaStreamSynchronize(sys->cap) != cudaSuccess)) {
+    cudaGetLastError();
+    if (want) cudaGraphExecDestroy(want);
+    want = nullptr;
+  }
+  return want ? want : one ? sys->dg_step : sys->dg_one;
+}
+
+// The device graphs of device-driven runs, with the step graph for a run of
+// nsteps steps; on any failure the system keeps the host-replayed graphs (the
+// same kernels).
+void build_device_graphs(prx_system* sys, uint64_t nsteps) {
   // Up to four steps per graph, so that the reaction interval divides into
   // graphs of nearly equal length (10: 4 + 4 + 2; 5: 3 + 2; 1: one step, since
   // every step is followed by a reaction step).  us per step with 1 / 2 / 3 /
@@ -582,28 +598,24 @@ void build_device_graphs(prx_system* sys) {
   const uint64_t theta = sys->has_rx ? sys->S.theta : most;
   const uint64_t graphs = (theta + most - 1) / most;
   sys->dg_steps = (uint32_t)((theta + graphs - 1) / graphs);
-  cudaError_t e = build_dg_step(sys, sys->dg_steps, &sys->dg_step);
-  if (e == cudaSuccess)
-    e = capture_device_graph(sys->cap, [&] { launch_rebin(sys->S, sys->cap, 0, nullptr, nullptr); },
-                             &sys->dg_rebuild);
+  cudaError_t e = capture_device_graph(
+      sys->cap, [&] { launch_rebin(sys->S, sys->cap, 0, nullptr, nullptr); }, &sys->dg_rebuild);
   if (e == cudaSuccess && sys->has_rx)
     e = capture_device_graph(sys->cap, [&] { launch_rx(sys->S, sys->cap, -1, nullptr, nullptr); },
                              &sys->dg_react);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(sys->cap);
-  sys->dg_ok = e == cudaSuccess;
+  sys->dg_ok = e == cudaSuccess && dg_graph(sys, nsteps);  // (waits for the uploads)
   if (!sys->dg_ok) {
     cudaGetLastError();
-    if (sys->dg_step) cudaGraphExecDestroy(sys->dg_step);
     if (sys->dg_rebuild) cudaGraphExecDestroy(sys->dg_rebuild);
     if (sys->dg_react) cudaGraphExecDestroy(sys->dg_react);
-    sys->dg_step = sys->dg_rebuild = sys->dg_react = nullptr;
+    sys->dg_rebuild = sys->dg_react = nullptr;
   }
 }
 
-int ensure_graphs(prx_system* sys) {
+int ensure_graphs(prx_system* sys, uint64_t nsteps) {
   if (sys->graphs_valid) return PRX_OK;
   destroy_graphs(sys);
-  build_device_graphs(sys);
+  build_device_graphs(sys, nsteps);
   if (sys->dg_ok) {
     sys->graphs_valid = true;
     return PRX_OK;
@@ -1410,23 +1422,12 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
   int rc;
   if (nsteps && (rc = refuse_capture(sys))) return rc;
   if (engine_fits(sys)) return engine_run(sys, nsteps);
-  if ((rc = ensure_graphs(sys))) return rc;
+  if ((rc = ensure_graphs(sys, nsteps))) return rc;
   if (sys->dg_ok) {
     // one device-driven chain of nsteps steps (with the rebuilds and the
     // reaction steps it decides on) behind one host launch
     if (nsteps == 0) return PRX_OK;
-    // a run shorter than the graph would end in empty step kernels (~2 us
-    // each): it takes the graph of one step
-    cudaGraphExec_t first = sys->dg_step;
-    if (nsteps < sys->dg_steps) {
-      if (!sys->dg_one && (build_dg_step(sys, 1, &sys->dg_one) != cudaSuccess ||
-                           cudaStreamSynchronize(sys->cap) != cudaSuccess)) {
-        cudaGetLastError();
-        if (sys->dg_one) cudaGraphExecDestroy(sys->dg_one);
-        sys->dg_one = nullptr;
-      }
-      if (sys->dg_one) first = sys->dg_one;
-    }
+    const cudaGraphExec_t first = dg_graph(sys, nsteps);
     launch_dg_arm(sys->S, sys->stream, nsteps, (unsigned long long)sys->dg_rebuild,
                   (unsigned long long)sys->dg_react);
     const cudaError_t launched = cudaGraphLaunch(first, sys->stream);
