@@ -2048,6 +2048,12 @@ namespace {
 std::mutex g_tune_mu;
 std::map<std::string, prx_tune_choice> g_tune_cache;
 
+// The kernels that a choice was timed with: counted up when a change moves the
+// times of the candidates against each other, so that a cache file's older
+// choices are no longer found (one with four lanes per slot, from before the
+// persistent runs, would keep a small system off them).
+constexpr int kTuneGeneration = 2;
+
 // The cache key: what the timing depends on.
 std::string tune_key(const prx_system_desc& d, const prx_reaction_desc* rx, uint32_t steps,
                      const double* skins, uint32_t n_skins, const uint32_t* threads,
@@ -2055,8 +2061,8 @@ std::string tune_key(const prx_system_desc& d, const prx_reaction_desc* rx, uint
                      const uint32_t* chunks, uint32_t n_chunks) {
   char buf[512];
   const double V = d.box[0] * d.box[1] * d.box[2];
-  snprintf(buf, sizeof(buf), "n=%u rho=%.4f cap=%u fp64=%d gamma=%.3g rx=%d rr=%.4g theta=%u k=%.4g steps=%u|",
-           d.n, d.n / V, d.adj_cap, d.force_precision, d.gamma, rx ? 1 : 0, rx ? rx->r_react : 0.0,
+  snprintf(buf, sizeof(buf), "g%d n=%u rho=%.4f cap=%u fp64=%d gamma=%.3g rx=%d rr=%.4g theta=%u k=%.4g steps=%u|",
+           kTuneGeneration, d.n, d.n / V, d.adj_cap, d.force_precision, d.gamma, rx ? 1 : 0, rx ? rx->r_react : 0.0,
            rx ? rx->theta : 0u, rx ? rx->k : 0.0, steps);
   std::string k(buf);
   for (uint32_t q = 0; q < n_skins; ++q) k += std::to_string(skins[q]) + ",";
