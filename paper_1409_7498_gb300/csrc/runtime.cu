@@ -449,12 +449,16 @@ int read_ctl(prx_system* sys) {
   return PRX_OK;
 }
 
-int sync_status(prx_system* sys) {
-  int rc = read_ctl(sys);
-  if (rc) return rc;
+// The sticky status that read_ctl brought.
+int status_read(prx_system* sys) {
   const int st = sys->ctl_host->status;
   if (st) return fail(sys, st, std::string("device reported ") + prx_status_string(st));
   return PRX_OK;
+}
+
+int sync_status(prx_system* sys) {
+  const int rc = read_ctl(sys);
+  return rc ? rc : status_read(sys);
 }
 
 // Event hook used while profiling: records an event before and after each launch.
@@ -1963,11 +1967,12 @@ int prx_pair_histogram(prx_system* sys, const prx_class* a, const prx_class* b, 
   sys->other_launches += 2;
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(sys->hist_host, d_c, 8 * (size_t)(nbins + 2), cudaMemcpyDeviceToHost, sys->stream));
-  const int rc = sync_status(sys);  // (one wait for the counts and the control block)
+  const int rc = read_ctl(sys);  // (one wait for the counts and the control block)
+  if (rc) return rc;
   for (uint32_t k = 0; k < nbins; ++k) counts[k] = sys->hist_host[k];
   if (n_a) *n_a = sys->hist_host[nbins];
   if (n_b) *n_b = sys->hist_host[nbins + 1];
-  return rc;
+  return status_read(sys);
 }
 
 // ---- autotuner -------------------------------------------------------------------

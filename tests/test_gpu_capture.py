@@ -43,3 +43,45 @@ def test_run_is_refused_while_capturing(n, fp64):
     for a, b in zip(*out):
         assert np.array_equal(a, b)
     assert out[0][2] == 40 and len(out[0][1]) > 0
+
+
+HISTOGRAM = """
+import ctypes as C, sys
+sys.path.insert(0, "tests")
+import numpy as np, torch
+import synth
+from helpers import gpu
+P = gpu()
+n = 2048
+inp = synth.step_growth(n - 200, 200, 4, 1)
+stream = torch.cuda.Stream()
+g = P.System(P.make_desc(n, inp.L, adj_cap=4), inp.x, inp.v, inp.type, inp.state, stream=stream.cuda_stream)
+a = P.prx_class(1, 0, 15)
+def histogram(counts):
+    k = C.c_uint64(99)
+    rc = P.lib().prx_pair_histogram(g.h, C.byref(a), C.byref(a), 1.1, len(counts), counts.ctypes.data, C.byref(k), C.byref(k))
+    return rc, k.value
+c = np.zeros(50, np.uint64)
+assert histogram(c) == (P.PRX_OK, n - 200) and c.sum() > 0
+graph = torch.cuda.CUDAGraph()
+c[:] = 7
+with torch.cuda.stream(stream):
+    graph.capture_begin(capture_error_mode="thread_local")
+    rc, k = histogram(c)  # its wait is refused, which also ends the capture
+assert rc == P.PRX_ECUDA and k == 99 and (c == 7).all(), (rc, k, c)
+print("untouched", flush=True)
+import os
+os._exit(0)
+"""
+
+
+def test_a_failed_histogram_writes_nothing():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", HISTOGRAM], cwd=root, capture_output=True, text=True, timeout=240)
+    assert r.returncode == 0 and "untouched" in r.stdout, r.stdout + r.stderr
