@@ -799,6 +799,7 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
     if (b == 0u) {
       ctl->set = set;
       ctl->phase = ph;
+      ctl->eng_steps += step - ctl->step;
       ctl->step = step;
       ctl->rebins += rebins;
     }

@@ -98,6 +98,7 @@ struct Ctl {
   unsigned long long dg_rebuild, dg_react, dg_runs;
   int rx_due;                  // a reaction step follows
   unsigned int until_rx;       // steps to the next one
+  unsigned long long eng_steps;  // steps that persistent kernels took
 };
 
 // Observables as they are read back: kinetic energy / 2 and momentum,
@@ -452,4 +453,6 @@ extern "C" {
 // Polls after which the barriers of the system's persistent runs give up
 // (at least 1; ENG_POLLS by default).
 int prx_test_wait_limit(prx_system* sys, uint32_t polls);
+// Steps of the system that went through the persistent kernel.  Synchronises.
+int prx_test_persistent_steps(prx_system* sys, uint64_t* steps);
 }

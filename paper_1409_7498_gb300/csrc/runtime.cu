@@ -1478,6 +1478,13 @@ int prx_test_wait_limit(prx_system* sys, uint32_t polls) {
   return PRX_OK;
 }
 
+int prx_test_persistent_steps(prx_system* sys, uint64_t* steps) {
+  if (!sys || !steps) return PRX_EINVAL;
+  const int rc = sync_status(sys);
+  *steps = sys->ctl_host->eng_steps;
+  return rc;
+}
+
 int prx_sync(prx_system* sys) {
   if (!sys) return PRX_EINVAL;
   return sync_status(sys);
