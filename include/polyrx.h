@@ -220,8 +220,9 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
 
 /* Queues nsteps MD steps (with the reaction every Theta steps) on the
  * system's stream and returns without waiting.  A run of a small system is
- * a few launches of a persistent kernel, each of some hundred steps with
- * their rebuilds and reaction steps; otherwise the run is one device-driven
+ * launches of a persistent kernel, each of up to 512 steps with their rebuilds
+ * and reaction steps (queued as one graph that launches itself again, when
+ * there are several); otherwise the run is one device-driven
  * chain of graphs of up to four steps, each ended by a kernel on the GPU that
  * launches the list rebuild when a particle moved more than skin/2, the
  * reaction step when it is due, and the next steps; where device graphs are not

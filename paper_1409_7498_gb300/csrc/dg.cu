@@ -67,6 +67,26 @@ __global__ void k_dgb_arm(BatchCtl* c, unsigned long long steps, unsigned long l
   }
 }
 
+// Persistent runs (engine.cu) of more than one launch: the graph is one launch
+// and k_eng_next, so that the host queues one graph however long the run is.
+// Queued one by one, the launches of two long runs filled the stream's queue
+// (1,024 entries) and prx_run waited for the device.
+__global__ void k_eng_arm(Ctl* ctl, unsigned long long steps) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) ctl->steps_left = steps;
+}
+__global__ void k_eng_next(Ctl* ctl, unsigned long long* bar) {
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  const unsigned long long left = ctl->steps_left;
+  const int status = ctl->status;
+  bar[0] = bar[16] = 0ull;  // the launch's barrier words
+  const unsigned long long rest = status == PRX_ETIMEOUT || left <= ENG_STEPS ? 0ull : left - ENG_STEPS;
+  ctl->steps_left = rest;
+  if (rest && cudaGraphLaunch(cudaGetCurrentGraphExec(), cudaStreamGraphTailLaunch) != cudaSuccess) {
+    ctl->steps_left = 0ull;
+    atomicCAS(&ctl->status, 0, PRX_ECUDA);
+  }
+}
+
 // After a batch step (the last member's epilogue left its decision in
 // rebuild_now): the rebuild of the members that need one, the reaction step
 // when the batch's phase wraps, the next step.
@@ -101,6 +121,10 @@ void launch_dg_arm(const Sys& S, cudaStream_t st, unsigned long long steps,
                    unsigned long long rebuild, unsigned long long react) {
   k_dg_arm<<<1, 32, 0, st>>>(S.ctl, steps, S.has_rx ? S.theta : 0u, rebuild, react);
 }
+
+void launch_eng_arm(const Sys& S, cudaStream_t st, unsigned long long steps) { k_eng_arm<<<1, 32, 0, st>>>(S.ctl, steps); }
+
+void launch_eng_next(const Sys& S, cudaStream_t st, unsigned long long* bar) { k_eng_next<<<1, 32, 0, st>>>(S.ctl, bar); }
 
 void launch_dg_next(const Sys& S, cudaStream_t st) { k_dg_next<<<1, 32, 0, st>>>(S.ctl); }
 

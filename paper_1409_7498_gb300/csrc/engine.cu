@@ -808,7 +808,8 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
 
 // One system, every block of the grid in its group.  bar: this launch's two
 // words; bar_next: the next launch's, cleared here (launches of a system
-// follow one another on its stream).
+// follow one another on its stream).  nsteps = 0: a launch of a run that the
+// device drives (dg.cu), which has steps_left to go and clears the words itself.
 template <bool NL16, bool CUBIC, bool F64>
 __global__ void __launch_bounds__(ENG_THREADS, 1)
     k_engine(Sys S, uint32_t nsteps, uint32_t theta, unsigned long long* bar, unsigned long long* bar_next,
@@ -820,7 +821,8 @@ __global__ void __launch_bounds__(ENG_THREADS, 1)
   // where the others already have.)
   const int gone = S.ctl->status == PRX_ETIMEOUT;
   if (__syncthreads_or(gone)) return;
-  if (blockIdx.x == 0 && threadIdx.x < 2) bar_next[threadIdx.x * 16] = 0ull;
+  if (bar_next && blockIdx.x == 0 && threadIdx.x < 2) bar_next[threadIdx.x * 16] = 0ull;
+  if (nsteps == 0u) nsteps = (uint32_t)min((unsigned long long)ENG_STEPS, S.ctl->steps_left);
   GroupBar gb{bar, &res, gridDim.x, 0u, 0u, 0u, polls};
   eng_run<NL16, CUBIC, F64>(S, blockIdx.x, gb, nsteps, theta, nullptr, smem);
 }

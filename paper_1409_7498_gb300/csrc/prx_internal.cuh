@@ -425,6 +425,10 @@ unsigned device_sms();
 // Polls of a barrier before it gives up (a few seconds): an error status
 // instead of a hang.
 constexpr unsigned ENG_POLLS = 1u << 22;
+// Steps per persistent launch: 3 to 20 ms, after which other streams' work gets
+// its turn on the GPU.  (A launch of a device-driven run costs ~8 us more than
+// one queued by the host.)
+constexpr unsigned ENG_STEPS = 512;
 struct EngPlan {
   const void* kernel = nullptr;
   unsigned blocks = 0;  // 0: the system's runs do not go through a persistent kernel
@@ -434,6 +438,11 @@ struct EngPlan {
 EngPlan engine_plan(const Sys& S, int fp64);
 cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint32_t nsteps, uint32_t theta,
                           unsigned long long* bar, unsigned long long* bar_next);
+// A run of more than one persistent launch is driven by the device (dg.cu):
+// k_eng_arm stores its steps, k_eng_next follows each launch in its graph and
+// launches the graph again until they are done.
+void launch_eng_arm(const Sys& S, cudaStream_t st, unsigned long long steps);
+void launch_eng_next(const Sys& S, cudaStream_t st, unsigned long long* bar);
 // Device-driven runs (dg.cu): k_dg_arm stores the run's step count and the
 // rebuild and reaction device graphs in the control block; k_dg_next, the
 // last kernel of the step's device graph, tail-launches what follows.

@@ -75,9 +75,12 @@ struct prx_system {
   uint32_t dg_steps = 1;  // steps in dg_step
   bool dg_ok = false;
   bool graphs_valid = false;
-  // persistent runs (engine.cu): the barrier words, the plan (once asked
-  // for), the launches so far
+  // persistent runs (engine.cu): the barrier words (two launches' in turn, and
+  // the graph's), the plan (once asked for), the launches so far; the device
+  // graph of one launch, for runs of several (made when first needed)
   unsigned long long* eng_bar = nullptr;
+  cudaGraphExec_t dg_eng = nullptr;
+  bool dg_eng_tried = false;
   EngPlan eng;
   bool eng_planned = false;
   unsigned eng_polls = ENG_POLLS;
@@ -258,7 +261,10 @@ double max_r_react(const prx_system* sys) {
 void destroy_graphs(prx_system* s) {
   // a device-driven run in flight launches these graphs from the device:
   // it must have finished before they go
-  if ((s->dg_step || s->dg_rebuild || s->dg_react) && s->stream) cudaStreamSynchronize(s->stream);
+  if ((s->dg_step || s->dg_rebuild || s->dg_react || s->dg_eng) && s->stream) cudaStreamSynchronize(s->stream);
+  if (s->dg_eng) cudaGraphExecDestroy(s->dg_eng);
+  s->dg_eng = nullptr;
+  s->dg_eng_tried = false;
   if (s->g_step) cudaGraphExecDestroy(s->g_step);
   if (s->g_chunk) cudaGraphExecDestroy(s->g_chunk);
   if (s->g_chunk1) cudaGraphExecDestroy(s->g_chunk1);
@@ -649,13 +655,37 @@ bool engine_fits(prx_system* sys) {
   return sys->eng.blocks > 0;
 }
 
-// nsteps steps in persistent launches of a few hundred steps each (so that
-// other streams' work gets its turn on the GPU in between).
+// nsteps steps in persistent launches of ENG_STEPS steps: one launch, or a graph
+// that launches itself again on the device until they are done (where that
+// cannot be made, the launches one by one).
 int engine_run(prx_system* sys, uint64_t nsteps) {
-  const uint64_t per = std::min<uint64_t>(std::max<uint64_t>(256, (nsteps + 511) / 512), 1u << 16);
   const uint32_t theta = sys->has_rx ? sys->rxd.theta : 0u;
+  if (nsteps > ENG_STEPS && !sys->dg_eng_tried) {
+    unsigned long long* bar = sys->eng_bar + 64;
+    cudaError_t e = capture_device_graph(sys->cap, [&] {
+      launch_engine(sys->S, sys->cap, sys->eng, 0u, theta, bar, nullptr);
+      launch_eng_next(sys->S, sys->cap, bar);
+    }, &sys->dg_eng);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(sys->cap);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      if (sys->dg_eng) cudaGraphExecDestroy(sys->dg_eng);
+      sys->dg_eng = nullptr;
+    }
+    sys->dg_eng_tried = true;
+  }
+  if (nsteps > ENG_STEPS && sys->dg_eng) {
+    launch_eng_arm(sys->S, sys->stream, nsteps);
+    CK(cudaGetLastError());
+    CK(cudaGraphLaunch(sys->dg_eng, sys->stream));
+    if (theta) sys->graph_rx_launches += (sys->host_step + nsteps) / theta - sys->host_step / theta;
+    sys->host_step += nsteps;
+    sys->step_launches += nsteps;
+    sys->other_launches += 1 + (nsteps + ENG_STEPS - 1) / ENG_STEPS;
+    return PRX_OK;
+  }
   while (nsteps) {
-    const uint64_t k = std::min(per, nsteps);
+    const uint64_t k = std::min<uint64_t>(ENG_STEPS, nsteps);
     unsigned long long* bar = sys->eng_bar + 32 * (sys->eng_launches & 1u);
     unsigned long long* next = sys->eng_bar + 32 * ((sys->eng_launches + 1u) & 1u);
     CK(launch_engine(sys->S, sys->stream, sys->eng, (uint32_t)k, theta, bar, next));
@@ -847,7 +877,7 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   A.add(&S.pop, (size_t)POP_REPLICAS * PRX_MAX_TYPES * PRX_MAX_STATES);
   A.add(&S.red, 4 * ((size_t)(n + RX_THREADS - 1) / RX_THREADS + 1));
   A.add(&S.fout, 3 * (size_t)n), A.add(&S.eout, (size_t)n);  // (one after the other: the bond sort's scratch)
-  A.add(&sys->eng_bar, 64), A.add(&sys->hist_dev, 2 * (size_t)kMaxBins + 3), A.add(&sys->obs_dev, 1);
+  A.add(&sys->eng_bar, 96), A.add(&sys->hist_dev, 2 * (size_t)kMaxBins + 3), A.add(&sys->obs_dev, 1);
   if ((rc = A.commit(sys, sys->dev_allocs))) return bail(rc);
   sys->bond_scratch = (size_t)((char*)S.eout - (char*)S.fout) + 8 * (size_t)n;
   if ((rc = setup_grid(sys, grid_rc > rc_w ? grid_rc : rc_w))) return bail(rc);
@@ -982,7 +1012,7 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   if ((rc = up(S.ctl, &c0, sizeof(Ctl)))) return bail(rc);
   sys->host_step = step0;
   if (cudaMemsetAsync(S.hist, 0, sizeof(HistRec) * (S.hist_cap + 2), sys->stream) != cudaSuccess ||
-      cudaMemsetAsync(sys->eng_bar, 0, 8 * 64, sys->stream) != cudaSuccess)
+      cudaMemsetAsync(sys->eng_bar, 0, 8 * 96, sys->stream) != cudaSuccess)
     return bail(fail(sys, PRX_ECUDA, "memset failed"));
 
   if (slot_cells) {
@@ -1475,6 +1505,7 @@ int prx_test_wait_limit(prx_system* sys, uint32_t polls) {
   if (!sys || polls < 1) return PRX_EINVAL;
   sys->eng_polls = polls;
   sys->eng_planned = false;
+  destroy_graphs(sys);
   return PRX_OK;
 }
 
