@@ -3,11 +3,11 @@
 // A run of the one-phase kernels is a chain of launches (step, then the
 // rebuild's seven and the reaction's three when they are due), and for a
 // system of some ten thousand particles that chain costs more than the work:
-// 20 us per step, of which a few are the step itself.  Here a group of
-// resident blocks keeps one system for the whole launch.  Each phase (the
+// 20 us per step, of which a few are the step itself.  Here the blocks of one
+// grid, all resident, keep the system for the whole launch.  Each phase (the
 // step; keys, scan, scatter, permutation and lists of a rebuild; search and
-// selection of a reaction step) is spread over the group's blocks and ends
-// at a barrier of the group, which also carries the "a particle moved more
+// selection of a reaction step) is spread over the grid's blocks and ends
+// at a barrier of the grid, which also carries the "a particle moved more
 // than skin/2" flag, so that a step costs one barrier.
 //
 // The phases do the arithmetic of the one-phase kernels in the same order
@@ -34,7 +34,7 @@ constexpr int ENG_THREADS = 512;
 constexpr unsigned ENG_F64_MAX = 16384;  // particles of a persistent FP64 run
 constexpr int ENG_UNITS = 1024;  // (slot, layer) pairs per tile of the list build
 
-// Barrier of the `nb` blocks of a group.  Two words, used in turn: the low
+// Barrier of the grid's `nb` blocks.  Two words, used in turn: the low
 // half counts arrivals, the high half the blocks that raised the flag.  A
 // block reaches the word's next use only after every block has left the
 // other word's barrier, hence this one, so a count beyond the target cannot
@@ -44,17 +44,16 @@ constexpr int ENG_UNITS = 1024;  // (slot, layer) pairs per tile of the list bui
 // ends with the load that sees the target: 8.95 -> 8.52 us per step (33,096
 // beads), against relaxed polls with a fence after them (a second round trip),
 // whether that fence is __threadfence or fence.acq_rel.
-struct GroupBar {
+struct GridBar {
   unsigned long long* w;
   int* res;  // shared: thread 0's verdict for the block
   uint32_t nb, e, flags0, flags1;
   uint32_t polls;  // of a barrier before it gives up
 
-  // Waits for the whole group; 1 when a thread of any block raised `f`, 0
+  // Waits for the whole grid; 1 when a thread of any block raised `f`, 0
   // when none did, 2 when the wait ran out.
   __device__ __forceinline__ int sync(bool f) {
     const int any = __syncthreads_or(f);
-    if (nb == 1u) return any;
     if (threadIdx.x == 0) {
       unsigned long long* p = w + (e & 1u) * 16u;
       asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(any ? 0x100000001ull : 1ull) : "memory");
@@ -541,7 +540,7 @@ __device__ __forceinline__ void eng_build_tile(const Sys& S, const uint4* P, con
 // the buckets' place.
 template <bool NL16>
 __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA& B, uint4* P, uint32_t b,
-                                                 GroupBar& bar, unsigned char* smem) {
+                                                 GridBar& bar, unsigned char* smem) {
   const uint32_t nb = bar.nb, g = b * ENG_THREADS + threadIdx.x, stride = nb * ENG_THREADS;
   const uint32_t ncell = (uint32_t)S.ncell;
   bool over = false;
@@ -631,7 +630,7 @@ __device__ __forceinline__ int eng_rebuild(const Sys& S, const SoA& A, const SoA
 // Reaction step: each block searches for the eligible A's of its own range
 // of slots (compacted into the same range of tmp), then forms the bonds.
 template <bool NL16>
-__device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4* P, uint32_t b, GroupBar& bar,
+__device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4* P, uint32_t b, GridBar& bar,
                                          unsigned long long step, uint32_t* s_cnt, int32_t* dpop) {
   const RxParams& R = S.R;
   const uint32_t nb = bar.nb;
@@ -703,11 +702,11 @@ __device__ __forceinline__ int eng_react(const Sys& S, const SoA& B, const uint4
   return 0;
 }
 
-// nsteps steps of one system by block b of its group.  until: steps to the
-// next reaction step (0: no scheme), theta apart.
+// nsteps steps of one system by block b of its grid.  theta: steps between
+// reaction steps (0: no scheme).
 template <bool NL16, bool CUBIC, bool F64>
-__device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar, uint32_t nsteps, uint32_t theta,
-                                        uint8_t* rebuilt, unsigned char* smem) {
+__device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GridBar& bar, uint32_t nsteps, uint32_t theta,
+                                        unsigned char* smem) {
   __shared__ uint32_t s_cnt;
   __shared__ int32_t dpop[PRX_MAX_TYPES * PRX_MAX_STATES];
   Ctl* ctl = S.ctl;
@@ -767,7 +766,6 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
       set ^= 1;
       ++rebins;
       if (rv) res_load<NL16>(S, B, Pc, ri, r, smem);
-      if (rebuilt && b == 0u && threadIdx.x == 0) rebuilt[q] = 1u;
     }
     if (reacts) {
       SoA B = set ? S.s1 : S.s0;
@@ -806,7 +804,7 @@ __device__ __forceinline__ void eng_run(const Sys& S, uint32_t b, GroupBar& bar,
   }
 }
 
-// One system, every block of the grid in its group.  bar: this launch's two
+// One system, every block of the grid.  bar: this launch's two
 // words; bar_next: the next launch's, cleared here (launches of a system
 // follow one another on its stream).  nsteps = 0: a launch of a run that the
 // device drives (dg.cu), which has steps_left to go and clears the words itself.
@@ -823,8 +821,8 @@ __global__ void __launch_bounds__(ENG_THREADS, 1)
   if (__syncthreads_or(gone)) return;
   if (bar_next && blockIdx.x == 0 && threadIdx.x < 2) bar_next[threadIdx.x * 16] = 0ull;
   if (nsteps == 0u) nsteps = (uint32_t)min((unsigned long long)ENG_STEPS, S.ctl->steps_left);
-  GroupBar gb{bar, &res, gridDim.x, 0u, 0u, 0u, polls};
-  eng_run<NL16, CUBIC, F64>(S, blockIdx.x, gb, nsteps, theta, nullptr, smem);
+  GridBar gb{bar, &res, gridDim.x, 0u, 0u, 0u, polls};
+  eng_run<NL16, CUBIC, F64>(S, blockIdx.x, gb, nsteps, theta, smem);
 }
 
 // The kernel that runs system S.
