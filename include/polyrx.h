@@ -228,8 +228,12 @@ int prx_set_reactions(prx_system* sys, const prx_reaction_desc* rx, uint32_t n_r
  * reaction step when it is due, and the next steps; where device graphs are not
  * available the library replays host-launched CUDA graphs with a
  * conditional rebuild node after each step instead, with the same kernels
- * and the same result.  PRX_ECUDA while the stream is being captured into a
- * CUDA graph: the run is not queued and the capture goes on. */
+ * and the same result.  A persistent launch has the GPU's SMs to itself: when
+ * several small systems are run at once, each on its own stream, and their
+ * launch chains together would be done sooner, the runs take these (a program
+ * with many small systems is served best by a batch, below).  PRX_ECUDA while
+ * the stream is being captured into a CUDA graph: the run is not queued and
+ * the capture goes on. */
 int prx_run(prx_system* sys, uint64_t nsteps);
 
 /* Waits for queued work; returns the sticky device status. */

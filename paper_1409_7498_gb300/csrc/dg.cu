@@ -50,7 +50,10 @@ __global__ void k_dg_next(Ctl* ctl) {
   if (rebuild) ok = cudaGraphLaunch((cudaGraphExec_t)ctl->dg_rebuild, cudaStreamGraphTailLaunch) == cudaSuccess;
   if (ok && react) ok = cudaGraphLaunch((cudaGraphExec_t)ctl->dg_react, cudaStreamGraphTailLaunch) == cudaSuccess;
   if (ok && left) ok = cudaGraphLaunch(cudaGetCurrentGraphExec(), cudaStreamGraphTailLaunch) == cudaSuccess;
-  if (!ok || !left) ctl->dg_on = 0;
+  if (!ok || !left) {
+    ctl->dg_on = 0;
+    mark_run(ctl);
+  }
   if (!ok) atomicCAS(&ctl->status, 0, PRX_ECUDA);
 }
 
@@ -81,10 +84,12 @@ __global__ void k_eng_next(Ctl* ctl, unsigned long long* bar) {
   bar[0] = bar[16] = 0ull;  // the launch's barrier words
   const unsigned long long rest = status == PRX_ETIMEOUT || left <= ENG_STEPS ? 0ull : left - ENG_STEPS;
   ctl->steps_left = rest;
-  if (rest && cudaGraphLaunch(cudaGetCurrentGraphExec(), cudaStreamGraphTailLaunch) != cudaSuccess) {
+  const bool ok = !rest || cudaGraphLaunch(cudaGetCurrentGraphExec(), cudaStreamGraphTailLaunch) == cudaSuccess;
+  if (!ok) {
     ctl->steps_left = 0ull;
     atomicCAS(&ctl->status, 0, PRX_ECUDA);
   }
+  if (!ok || !rest) mark_run(ctl);
 }
 
 // After a batch step (the last member's epilogue left its decision in

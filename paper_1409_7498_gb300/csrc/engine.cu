@@ -817,12 +817,17 @@ __global__ void __launch_bounds__(ENG_THREADS, 1)
   // a wait of an earlier launch ran out: nothing may build on what it left.
   // (A block that reads the status of this launch's own timeout leaves early
   // where the others already have.)
+  const bool marks = nsteps != 0u && blockIdx.x == 0 && threadIdx.x == 0;
   const int gone = S.ctl->status == PRX_ETIMEOUT;
-  if (__syncthreads_or(gone)) return;
+  if (__syncthreads_or(gone)) {
+    if (marks) mark_run(S.ctl);
+    return;
+  }
   if (bar_next && blockIdx.x == 0 && threadIdx.x < 2) bar_next[threadIdx.x * 16] = 0ull;
   if (nsteps == 0u) nsteps = (uint32_t)min((unsigned long long)ENG_STEPS, S.ctl->steps_left);
   GridBar gb{bar, &res, gridDim.x, 0u, 0u, 0u, polls};
   eng_run<NL16, CUBIC, F64>(S, blockIdx.x, gb, nsteps, theta, smem);
+  if (marks) mark_run(S.ctl);
 }
 
 // The kernel that runs system S.
@@ -891,6 +896,20 @@ static unsigned engine_resident(const void* k, size_t sm) {
 //   20,000 53 -> 58 (by then the FP64 pipe bounds both): up to 16,384.
 // Runs with a force cap (warm-ups) and four-lane runs keep the launch chain,
 // as do boxes with more cells or longer rows than the rebuild holds.
+//
+// And by what else is under way (runtime.cu, runs_persistent): k systems at once,
+// each on its own stream, take the sum of their persistent steps, about 5.8 us
+// plus 0.086 per 1,000 beads each, divided by the grids that fit side by side
+// (FP64: 9.5 plus 1.85 per 1,000), but as chains 17 us plus 0.05 per 1,000 beads
+// of all together (FP64: 28 plus 1.0).  `load` is a system's share of where the
+// two are equal.  us per step of all, persistent / chains:
+//   1,250 beads: k = 3 5.9 / 20, 8 17 / 18, 16 35 / 19
+//   2,048: k = 2 11.7 / 20, 3 17.6 / 17, 4 24 / 17, 8 48 / 18, 16 96 / 19
+//   16,384: k = 2 13.9 / 21, 3 20.6 / 18, 4 28 / 19, 16 113 / 26
+//   33,096: k = 2 16.6 / 23, 3 25.5 / 21, 4 34 / 22, 8 68 / 27, 16 136 / 40
+//   70,000: k = 2 23.8 / 24, 3 36 / 25, 4 48 / 28, 8 96 / 43, 16 192 / 80
+//   FP64: 1,000: k = 2 21.8 / 30, 3 33 / 30, 8 87 / 31; 5,000: k = 2 34 / 35,
+//   3 51 / 40, 8 137 / 61; 10,000: k = 2 59 / 46; 16,000: k = 2 75 / 62, 8 301 / 172
 EngPlan engine_plan(const Sys& S, int fp64) {
   EngPlan p;
   if (!S.n || !S.bucket || S.ncell > (int)ENG_CELLS || !S.eng_ty || S.fcapf > 0.f || S.step_lanes != 1) return p;
@@ -904,6 +923,8 @@ EngPlan engine_plan(const Sys& S, int fp64) {
   // a block per chunk as far as they go (the phases are bound by latency),
   // and one per tile of the list build
   p.blocks = std::min(most, std::max(chunks, (unsigned)(S.eng_tiles_y * S.nc[2])));
+  const double share = 1.0 / (most / p.blocks);  // of the GPU: grids that fit side by side run at once
+  p.load = fp64 ? (9.5 * share + 0.85e-3 * S.n) / 28.0 : (5.8 * share + 3.6e-5 * S.n) / 17.0;
   return p;
 }
 

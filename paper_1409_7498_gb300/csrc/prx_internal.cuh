@@ -99,7 +99,20 @@ struct Ctl {
   int rx_due;                  // a reaction step follows
   unsigned int until_rx;       // steps to the next one
   unsigned long long eng_steps;  // steps that persistent kernels took
+  // marks of finished runs (mark_run): their number, and the pinned host word
+  // that shows it
+  unsigned long long marks;
+  unsigned long long* marks_host;
 };
+
+// A run, or one of its launches, is done: the host learns of it without a call
+// (runtime.cu, runs_persistent).
+__device__ __forceinline__ void mark_run(Ctl* ctl) {
+  const unsigned long long m = ctl->marks + 1ull;
+  unsigned long long* const host = ctl->marks_host;
+  ctl->marks = m;
+  *(volatile unsigned long long*)host = m;
+}
 
 // Observables as they are read back: kinetic energy / 2 and momentum,
 // populations, step, bonds and status.
@@ -434,6 +447,7 @@ struct EngPlan {
   unsigned blocks = 0;  // 0: the system's runs do not go through a persistent kernel
   size_t smem = 0;
   unsigned polls = 0;   // of a barrier before it gives up
+  double load = 0.0;    // share of the runs at once that are still worth it (at most 1)
 };
 EngPlan engine_plan(const Sys& S, int fp64);
 cudaError_t launch_engine(const Sys& S, cudaStream_t st, const EngPlan& p, uint32_t nsteps, uint32_t theta,

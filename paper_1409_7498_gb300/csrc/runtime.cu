@@ -84,6 +84,12 @@ struct prx_system {
   EngPlan eng;
   bool eng_planned = false;
   unsigned eng_polls = ENG_POLLS;
+  // runs in flight (runs_persistent; all but the word under its lock): the
+  // word that shows the marks of finished runs, the marks queued, the system's
+  // own load, and the largest load seen since its latest run was queued
+  unsigned long long* marks_host = nullptr;
+  uint64_t marks = 0;
+  double load = 0.0, crowd = 0.0;
   uint64_t eng_launches = 0;
   size_t bond_scratch = 0;  // bytes of fout and eout together
   // pair histogram: squared bin edges, counts and class sizes; a pinned copy of
@@ -258,13 +264,11 @@ double max_r_react(const prx_system* sys) {
   return r;
 }
 
-void destroy_graphs(prx_system* s) {
+// The graphs of steps, rebuild and reaction.
+void destroy_step_graphs(prx_system* s) {
   // a device-driven run in flight launches these graphs from the device:
   // it must have finished before they go
-  if ((s->dg_step || s->dg_rebuild || s->dg_react || s->dg_eng) && s->stream) cudaStreamSynchronize(s->stream);
-  if (s->dg_eng) cudaGraphExecDestroy(s->dg_eng);
-  s->dg_eng = nullptr;
-  s->dg_eng_tried = false;
+  if ((s->dg_step || s->dg_one || s->dg_rebuild || s->dg_react) && s->stream) cudaStreamSynchronize(s->stream);
   if (s->g_step) cudaGraphExecDestroy(s->g_step);
   if (s->g_chunk) cudaGraphExecDestroy(s->g_chunk);
   if (s->g_chunk1) cudaGraphExecDestroy(s->g_chunk1);
@@ -277,6 +281,14 @@ void destroy_graphs(prx_system* s) {
   s->dg_step = s->dg_rebuild = s->dg_react = s->dg_one = nullptr;
   s->dg_ok = false;
   s->graphs_valid = false;
+}
+
+void destroy_graphs(prx_system* s) {
+  if (s->dg_eng && s->stream) cudaStreamSynchronize(s->stream);  // (as above)
+  if (s->dg_eng) cudaGraphExecDestroy(s->dg_eng);
+  s->dg_eng = nullptr;
+  s->dg_eng_tried = false;
+  destroy_step_graphs(s);
 }
 
 void free_list(std::vector<void*>& l) {
@@ -624,7 +636,7 @@ void build_device_graphs(prx_system* sys, uint64_t nsteps) {
 
 int ensure_graphs(prx_system* sys, uint64_t nsteps) {
   if (sys->graphs_valid) return PRX_OK;
-  destroy_graphs(sys);
+  destroy_step_graphs(sys);
   build_device_graphs(sys, nsteps);
   if (sys->dg_ok) {
     sys->graphs_valid = true;
@@ -655,6 +667,49 @@ bool engine_fits(prx_system* sys) {
   return sys->eng.blocks > 0;
 }
 
+// Systems whose runs fit the persistent kernel and may still be on the GPU.
+struct Flights {
+  std::mutex mu;
+  std::vector<prx_system*> in;
+};
+Flights g_flights;
+
+// Whether a run of a system that fits the persistent kernel takes it.  A
+// persistent launch has its SMs to itself, so that systems run at once, each on
+// its own stream, follow one another, where their launch chains would share the
+// GPU: alone or two at once they are sooner done so, but sixteen of 2,048 beads
+// take 96 us for a step of all, and 19 in chains (engine.cu, engine_plan, has
+// the rule).  The run takes its chain when the loads of the runs
+// in flight and its own exceed 1, or did while its run before was in flight:
+// systems that are advanced together in turn take their chains from the second
+// run on, the first of them too.  The results are the same bits either way.
+bool runs_persistent(prx_system* sys) {
+  std::lock_guard<std::mutex> lk(g_flights.mu);
+  std::vector<prx_system*>& in = g_flights.in;
+  size_t kept = 0;
+  double load = sys->eng.load;
+  for (prx_system* o : in) {
+    if (__atomic_load_n(o->marks_host, __ATOMIC_RELAXED) >= o->marks) continue;
+    in[kept++] = o;
+    if (o != sys) load += o->load;
+  }
+  in.resize(kept);
+  for (prx_system* o : in)
+    if (o != sys) o->crowd = std::max(o->crowd, load);
+  const double before = sys->crowd;
+  sys->crowd = load;
+  return std::max(load, before) <= 1.0;
+}
+
+// A run of the system was queued that leaves a mark.
+void run_queued(prx_system* sys) {
+  std::lock_guard<std::mutex> lk(g_flights.mu);
+  sys->marks++;
+  sys->load = sys->eng.load;
+  std::vector<prx_system*>& in = g_flights.in;
+  if (sys->eng.blocks && std::find(in.begin(), in.end(), sys) == in.end()) in.push_back(sys);
+}
+
 // nsteps steps in persistent launches of ENG_STEPS steps: one launch, or a graph
 // that launches itself again on the device until they are done (where that
 // cannot be made, the launches one by one).
@@ -678,6 +733,7 @@ int engine_run(prx_system* sys, uint64_t nsteps) {
     launch_eng_arm(sys->S, sys->stream, nsteps);
     CK(cudaGetLastError());
     CK(cudaGraphLaunch(sys->dg_eng, sys->stream));
+    run_queued(sys);
     if (theta) sys->graph_rx_launches += (sys->host_step + nsteps) / theta - sys->host_step / theta;
     sys->host_step += nsteps;
     sys->step_launches += nsteps;
@@ -690,6 +746,7 @@ int engine_run(prx_system* sys, uint64_t nsteps) {
     unsigned long long* next = sys->eng_bar + 32 * ((sys->eng_launches + 1u) & 1u);
     CK(launch_engine(sys->S, sys->stream, sys->eng, (uint32_t)k, theta, bar, next));
     sys->eng_launches++;
+    run_queued(sys);
     if (theta) sys->graph_rx_launches += (sys->host_step + k) / theta - sys->host_step / theta;
     sys->host_step += k;
     sys->step_launches += k;
@@ -857,10 +914,12 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   if (cudaMallocHost(&sys->ctl_host, sizeof(Ctl)) != cudaSuccess)
     return bail(fail(sys, PRX_ENOMEM, "pinned control block"));
   const size_t obs_bytes = sizeof(*sys->obs_host) * (PRX_OBS_SLOTS + 1);
-  if (cudaMallocHost(&sys->obs_host, obs_bytes + 8 * (size_t)(kMaxBins + 2)) != cudaSuccess)
+  if (cudaMallocHost(&sys->obs_host, obs_bytes + 8 * (size_t)(kMaxBins + 3)) != cudaSuccess)
     return bail(fail(sys, PRX_ENOMEM, "pinned observables block"));
   static_assert(sizeof(*sys->obs_host) % 8 == 0, "the histogram's counts follow the observables");
   sys->hist_host = (unsigned long long*)((char*)sys->obs_host + obs_bytes);
+  sys->marks_host = sys->hist_host + kMaxBins + 2;
+  *sys->marks_host = 0ull;
   memset(sys->ctl_host, 0, sizeof(Ctl));
 
   DevArena A;
@@ -1009,6 +1068,7 @@ int create_impl(const prx_system_desc* desc, const double* pos, const double* ve
   memset(&c0, 0, sizeof(c0));
   c0.nbonds = n_bonds;
   c0.step = step0;
+  c0.marks_host = sys->marks_host;
   if ((rc = up(S.ctl, &c0, sizeof(Ctl)))) return bail(rc);
   sys->host_step = step0;
   if (cudaMemsetAsync(S.hist, 0, sizeof(HistRec) * (S.hist_cap + 2), sys->stream) != cudaSuccess ||
@@ -1333,6 +1393,11 @@ void prx_destroy(prx_system* sys) {
   if (sys->stream) cudaStreamSynchronize(sys->stream);
   if (sys->slot_batch) free_slot(sys->slot_batch, sys);  // admitted, finished, not yet polled
   if (sys->join_ev) cudaEventDestroy(sys->join_ev);
+  {
+    std::lock_guard<std::mutex> lk(g_flights.mu);
+    std::vector<prx_system*>& in = g_flights.in;
+    in.erase(std::remove(in.begin(), in.end(), sys), in.end());
+  }
   destroy_graphs(sys);
   for (auto& e : sys->prof) {
     cudaEventDestroy(e.a);
@@ -1455,7 +1520,8 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
   }
   int rc;
   if (nsteps && (rc = refuse_capture(sys))) return rc;
-  if (engine_fits(sys)) return engine_run(sys, nsteps);
+  const bool small = engine_fits(sys);
+  if (small && (nsteps == 0 || runs_persistent(sys))) return engine_run(sys, nsteps);
   if ((rc = ensure_graphs(sys, nsteps))) return rc;
   if (sys->dg_ok) {
     // one device-driven chain of nsteps steps (with the rebuilds and the
@@ -1467,6 +1533,7 @@ int prx_run(prx_system* sys, uint64_t nsteps) {
     const cudaError_t launched = cudaGraphLaunch(first, sys->stream);
     if (launched != cudaSuccess) launch_dg_arm(sys->S, sys->stream, 0, 0, 0);  // no run in progress
     CK(launched);
+    run_queued(sys);
     if (sys->has_rx) {
       const uint64_t th = sys->rxd.theta;
       sys->graph_rx_launches += (sys->host_step + nsteps) / th - sys->host_step / th;
