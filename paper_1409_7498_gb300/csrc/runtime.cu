@@ -90,6 +90,8 @@ struct prx_system {
   unsigned long long* marks_host = nullptr;
   uint64_t marks = 0;
   double load = 0.0, crowd = 0.0;
+  bool flying = false;  // in the list of g_flights
+  prx_system* next_flight = nullptr;
   uint64_t eng_launches = 0;
   size_t bond_scratch = 0;  // bytes of fout and eout together
   // pair histogram: squared bin edges, counts and class sizes; a pinned copy of
@@ -668,9 +670,10 @@ bool engine_fits(prx_system* sys) {
 }
 
 // Systems whose runs fit the persistent kernel and may still be on the GPU.
+// (A list through the systems themselves: it never allocates.)
 struct Flights {
   std::mutex mu;
-  std::vector<prx_system*> in;
+  prx_system* first = nullptr;
 };
 Flights g_flights;
 
@@ -685,16 +688,18 @@ Flights g_flights;
 // run on, the first of them too.  The results are the same bits either way.
 bool runs_persistent(prx_system* sys) {
   std::lock_guard<std::mutex> lk(g_flights.mu);
-  std::vector<prx_system*>& in = g_flights.in;
-  size_t kept = 0;
   double load = sys->eng.load;
-  for (prx_system* o : in) {
-    if (__atomic_load_n(o->marks_host, __ATOMIC_RELAXED) >= o->marks) continue;
-    in[kept++] = o;
+  for (prx_system** p = &g_flights.first; *p;) {
+    prx_system* o = *p;
+    if (__atomic_load_n(o->marks_host, __ATOMIC_RELAXED) >= o->marks) {
+      *p = o->next_flight;
+      o->flying = false;
+      continue;
+    }
     if (o != sys) load += o->load;
+    p = &o->next_flight;
   }
-  in.resize(kept);
-  for (prx_system* o : in)
+  for (prx_system* o = g_flights.first; o; o = o->next_flight)
     if (o != sys) o->crowd = std::max(o->crowd, load);
   const double before = sys->crowd;
   sys->crowd = load;
@@ -706,8 +711,10 @@ void run_queued(prx_system* sys) {
   std::lock_guard<std::mutex> lk(g_flights.mu);
   sys->marks++;
   sys->load = sys->eng.load;
-  std::vector<prx_system*>& in = g_flights.in;
-  if (sys->eng.blocks && std::find(in.begin(), in.end(), sys) == in.end()) in.push_back(sys);
+  if (!sys->eng.blocks || sys->flying) return;
+  sys->flying = true;
+  sys->next_flight = g_flights.first;
+  g_flights.first = sys;
 }
 
 // nsteps steps in persistent launches of ENG_STEPS steps: one launch, or a graph
@@ -1395,8 +1402,11 @@ void prx_destroy(prx_system* sys) {
   if (sys->join_ev) cudaEventDestroy(sys->join_ev);
   {
     std::lock_guard<std::mutex> lk(g_flights.mu);
-    std::vector<prx_system*>& in = g_flights.in;
-    in.erase(std::remove(in.begin(), in.end(), sys), in.end());
+    for (prx_system** p = &g_flights.first; sys->flying && *p; p = &(*p)->next_flight)
+      if (*p == sys) {
+        *p = sys->next_flight;
+        break;
+      }
   }
   destroy_graphs(sys);
   for (auto& e : sys->prof) {
