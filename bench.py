@@ -723,7 +723,7 @@ def main():
             ge.history_begin(q % 2)
             if q:
                 ob = ge.history_end((q - 1) % 2)
-            d2h += P.HISTORY_DTYPE.itemsize + 112  # the record and the 112-byte control block
+            d2h += P.HISTORY_DTYPE.itemsize + 184  # the record and the 184-byte control block
         ob = ge.history_end((ke - 1) % 2)
         stt = ge.states()
         bd = ge.bonds()
