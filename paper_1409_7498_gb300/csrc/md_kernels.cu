@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(256) kb_rebin_permute(const Sys* __restrict__ 
 // holds their heads, win the links; slots plus one, 0 the end); a scan of the counts gives the cells' first slots, and a slot's new
 // place is its cell's first slot plus the number of the cell's members with a
 // smaller old slot.  With the plan's work done by the step kernel, four
-// kernels instead of ten: 256 replicas 377 -> 366 us per step.  (A single
+// kernels instead of ten: 256 replicas 377 -> 369 us per step.  (A single
 // system keeps the seven kernels of launch_rebin: at a million beads the
 // permutation by old slot, whose stores are scattered, takes 67 us instead of
 // the 57 of scatter, sort and permutation.)
@@ -849,6 +849,8 @@ __global__ void __launch_bounds__(256) k_build_nlist(Sys S) {
   extern __shared__ __align__(16) unsigned char smem_b[];
   build_nlist_body<NL16>(S, Blk{blockIdx.x, gridDim.x}, smem_b);
 }
+// (Four blocks per SM: 64 registers with 36 bytes of spills, 256 replicas 361.5 us
+// per step; three blocks without spills 366.5.)
 __global__ void __launch_bounds__(256, 4)
     kb_build_nlist(const Sys* __restrict__ T, const BlkMap* __restrict__ M, uint32_t* C, uint32_t* act_n) {
   extern __shared__ __align__(16) unsigned char smem_b[];
