@@ -80,6 +80,20 @@ def test_two_at_once(P):
     close(gs)
 
 
+@pytest.mark.parametrize("n,took", [(2000, 400), (33000, 0)])
+def test_beside_a_large_system(P, n, took):
+    make = step_growth(P, n)
+    ref = alone(make, (400,))
+    with step_growth(P, 300000)() as big, make() as g:
+        big.run(400)
+        g.run(400)
+        assert persistent_steps(P, g) == took
+        got = result(g)
+        for key in ref:
+            assert np.array_equal(got[key], ref[key]), key
+        big.sync()
+
+
 def test_destroyed_while_others_run(P):
     """A system leaves with its run under way: it counts no longer."""
     make = step_growth(P, 2000)
