@@ -105,6 +105,7 @@ struct prx_system {
   cudaStream_t solo_stream = nullptr;  // the system's own stream while in a batch
   prx_batch* slot_batch = nullptr; // batch holding this system's admission slot
   int32_t slot = -1;               // its slot there (admitted until polled)
+  cudaEvent_t cap_ev = nullptr;    // orders the uploads on the capture stream before a run
   cudaEvent_t join_ev = nullptr;   // orders the system's queued work before a batch's
 };
 
@@ -589,6 +590,17 @@ cudaError_t build_dg_step(prx_system* sys, uint32_t steps, cudaGraphExec_t* out)
   }, out);
 }
 
+// What follows on the system's stream waits for the graphs uploaded on its capture
+// stream.  (Not the host: an upload waits for the GPU, which a persistent launch
+// of another system may hold for milliseconds.)
+cudaError_t after_uploads(prx_system* sys) {
+  cudaError_t e = cudaSuccess;
+  if (!sys->cap_ev) e = cudaEventCreateWithFlags(&sys->cap_ev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(sys->cap_ev, sys->cap);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(sys->stream, sys->cap_ev, 0);
+  return e;
+}
+
 // The step graph that suits a run of nsteps steps, made when first needed (the
 // other one where it cannot be made: both run any number of steps).  A run
 // shorter than the longer graph would end in empty step kernels (~2 us each).
@@ -596,8 +608,9 @@ cudaGraphExec_t dg_graph(prx_system* sys, uint64_t nsteps) {
   const bool one = nsteps < sys->dg_steps;
   cudaGraphExec_t& want = one ? sys->dg_one : sys->dg_step;
   if (!want && (build_dg_step(sys, one ? 1 : sys->dg_steps, &want) != cudaSuccess ||
-                cudaStreamSynchronize(sys->cap) != cudaSuccess)) {
+                after_uploads(sys) != cudaSuccess)) {
     cudaGetLastError();
+    cudaStreamSynchronize(sys->cap);
     if (want) cudaGraphExecDestroy(want);
     want = nullptr;
   }
@@ -627,9 +640,10 @@ void build_device_graphs(prx_system* sys, uint64_t nsteps) {
   if (e == cudaSuccess && sys->has_rx)
     e = capture_device_graph(sys->cap, [&] { launch_rx(sys->S, sys->cap, -1, nullptr, nullptr); },
                              &sys->dg_react);
-  sys->dg_ok = e == cudaSuccess && dg_graph(sys, nsteps);  // (waits for the uploads)
+  sys->dg_ok = e == cudaSuccess && dg_graph(sys, nsteps);  // (orders the uploads)
   if (!sys->dg_ok) {
     cudaGetLastError();
+    cudaStreamSynchronize(sys->cap);
     if (sys->dg_rebuild) cudaGraphExecDestroy(sys->dg_rebuild);
     if (sys->dg_react) cudaGraphExecDestroy(sys->dg_react);
     sys->dg_rebuild = sys->dg_react = nullptr;
@@ -733,9 +747,10 @@ int engine_run(prx_system* sys, uint64_t nsteps) {
       launch_engine(sys->S, sys->cap, sys->eng, 0u, theta, bar, nullptr);
       launch_eng_next(sys->S, sys->cap, bar);
     }, &sys->dg_eng);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(sys->cap);
+    if (e == cudaSuccess) e = after_uploads(sys);
     if (e != cudaSuccess) {
       cudaGetLastError();
+      cudaStreamSynchronize(sys->cap);
       if (sys->dg_eng) cudaGraphExecDestroy(sys->dg_eng);
       sys->dg_eng = nullptr;
     }
@@ -1405,6 +1420,7 @@ void prx_destroy(prx_system* sys) {
   if (sys->stream) cudaStreamSynchronize(sys->stream);
   if (sys->slot_batch) free_slot(sys->slot_batch, sys);  // admitted, finished, not yet polled
   if (sys->join_ev) cudaEventDestroy(sys->join_ev);
+  if (sys->cap_ev) cudaEventDestroy(sys->cap_ev);
   {
     std::lock_guard<std::mutex> lk(g_flights.mu);
     for (prx_system** p = &g_flights.first; sys->flying && *p; p = &(*p)->next_flight)

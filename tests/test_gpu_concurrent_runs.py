@@ -4,6 +4,7 @@ share the GPU, and back through the persistent kernel once they run alone.  The
 results are those of each system alone, bit for bit."""
 import ctypes as C
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -92,6 +93,27 @@ def test_beside_a_large_system(P, n, took):
         for key in ref:
             assert np.array_equal(got[key], ref[key]), key
         big.sync()
+
+
+def test_first_chains_return_without_waiting(P):
+    """New systems whose chains are made while a persistent launch has the GPU: a
+    launch of 512 steps takes about 19 ms here, a call that waits for its end up to
+    as long; the limit is a quarter of that.  (The first round loads the kernels.)"""
+    make = step_growth(P, 16000, fp64=True)
+    for _ in range(2):
+        gs = [make() for _ in range(8)]
+        for g in gs:
+            g.sync()
+        calls = []
+        for g in gs:
+            t = time.perf_counter()
+            g.run(2000)
+            calls.append(time.perf_counter() - t)
+        for g in gs:
+            g.sync()
+        assert persistent_steps(P, gs[0]) == 2000 and persistent_steps(P, gs[-1]) == 0
+        close(gs)
+    assert max(calls) < 5e-3, calls
 
 
 def test_destroyed_while_others_run(P):
